@@ -151,7 +151,7 @@ enum {
   TK_BICG = 8
 };
 
-// Spectral kernels (instantiated for float and double) --------------------------------
+// Spectral kernels (FP32: spectral.cuh and the pair files; FP64: spectral_f64.cu) ---------
 // COL_POISSON: divide by the eigenvalues of the 4th-order stencil Laplacian (0 at k = 0);
 // COL_POISSON_LP: the same times the Gaussian exp(-((k1/(M/4))^2 + (k2/(N/4))^2) / 2)
 enum ColMode {
@@ -244,6 +244,21 @@ cudaError_t launch_row_c2r(int mode, const C2<T>* q0, const C2<T>* q1, const C2<
                            double step, double out_scale, int N, int M, const SpecTables& tb,
                            const int* skip, cudaStream_t st, const DevScalars* sc = nullptr,
                            Bat bat = Bat());
+
+// FP64: passes of their own (spectral_f64.cu)
+template <>
+cudaError_t launch_row_r2c<double>(const double*, size_t, const int*, const double*, double2*,
+                                   int, int, const SpecTables&, const int*, cudaStream_t, Bat,
+                                   const DevScalars*);
+template <>
+cudaError_t launch_col<double>(int, const double2*, double2*, double2*, double2*, int, int,
+                               const SpecTables&, const DevScalars*, const int*, cudaStream_t,
+                               Bat);
+template <>
+cudaError_t launch_row_c2r<double>(int, const double2*, const double2*, const double2*,
+                                   const double*, double*, const double*, double*, double,
+                                   double, int, int, const SpecTables&, const int*, cudaStream_t,
+                                   const DevScalars*, Bat);
 
 // register-resident FP32 matvec passes on the transposed half spectrum specT (M/2 x N,
 // entry (k1, k2) at k1 N + k2): mvT_supported(N, M) when N and M/2 are powers of two in
