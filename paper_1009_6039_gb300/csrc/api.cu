@@ -2630,8 +2630,7 @@ extern "C" int ot_ws_trainer_create(ot_ws_trainer** out, int32_t batch,
   if (!tr) return OT_ENOMEM;
   tr->B = batch;
   cudaGetDevice(&tr->device);
-  const long n = ws_param_count(), B = batch, H = OTGB_WS_H;
-  const long S = (B + WS_ROW_CHUNK - 1) / WS_ROW_CHUNK;
+  const long n = ws_param_count();
   bool failed = false;
   auto get = [&](size_t bytes) -> void* {
     void* q = nullptr;
@@ -2647,13 +2646,13 @@ extern "C" int ot_ws_trainer_create(ot_ws_trainer** out, int32_t batch,
   tr->v = (float*)get(n * 4);
   WsTrainBuffers& b = tr->b;
   b.grad = (float*)get(n * 4);
-  b.Xb = (float*)get(B * OTGB_WS_K * 4);
-  b.tb = (float*)get(B * 4);
-  float** planes[] = {&b.Z0, &b.A0, &b.Z1, &b.A1, &b.Z2, &b.A2, &b.dZ1, &b.dZ2};
-  for (float** q : planes) *q = (float*)get(B * H * 4);
-  b.dy = (float*)get(B * 4);
-  b.part = (float*)get(S * H * H * 4);
-  b.loss_part = (double*)get(((B + 7) / 8) * 8);
+  b.sms = 0;
+  cudaDeviceGetAttribute(&b.sms, cudaDevAttrMultiProcessorCount, tr->device);
+  if (b.sms < 1) b.sms = 148;
+  const size_t blocks = ws_train_blocks(batch, b.sms);
+  b.scr = (float*)get(blocks * ws_train_scratch_floats() * 4);
+  b.part = (float*)get(blocks * ws_train_part_floats() * 4);
+  b.loss_part = (double*)get(blocks * 8);
   b.loss = (double*)get(8);
   if (failed) {
     cudaGetLastError();

@@ -416,20 +416,21 @@ cudaError_t launch_convert(const void* in, int in_is_double, void* out, int out_
 // Learned warm start ---------------------------------------------------------------------
 #define OTGB_WS_K 16    // features per grid point
 #define OTGB_WS_H 128   // hidden units per layer (three hidden layers)
-#define WS_ROW_CHUNK 2048  // rows per partial sum of the weight gradients
 constexpr long ws_param_count() {
   return (long)OTGB_WS_H * OTGB_WS_K + OTGB_WS_H +
          2 * ((long)OTGB_WS_H * OTGB_WS_H + OTGB_WS_H) + OTGB_WS_H + 1;
 }
-// buffers of one training step with B rows (FP32 unless noted)
+// buffers of a trainer: SiLU' of two layers and partial gradients per block (at most
+// ws_train_blocks of them), the gradient (ws_param_count()), squared-error sums per block, the
+// mean squared error
 struct WsTrainBuffers {
-  float *Xb, *tb;                  // gathered rows (B x 16) and targets (B)
-  float *Z0, *A0, *Z1, *A1, *Z2, *A2;  // pre-activations / activations (B x H each)
-  float *dy, *dZ1, *dZ2;           // output gradient (B), layer gradients (B x H)
-  float *part;                     // partial sums: ceil(B / WS_ROW_CHUNK) x H x H
-  float *grad;                     // gradient (ws_param_count())
-  double *loss_part, *loss;        // ceil(B / 8) partials, mean squared error
+  float *scr, *part, *grad;
+  double *loss_part, *loss;
+  int sms;
 };
+int ws_train_blocks(int B, int sms);
+size_t ws_train_scratch_floats();  // per block
+size_t ws_train_part_floats();     // per block
 cudaError_t launch_ws_source(const double* f, const double* g, double* src, long P,
                              cudaStream_t st);
 // transport outputs: *dist (device) = mean |grad u|^2 f, div (optional) = u_xx + u_yy;

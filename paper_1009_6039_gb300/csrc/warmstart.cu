@@ -1,5 +1,5 @@
-// Learned warm start: the kernels of the network's input features, of its training (FP32)
-// and of its inference (BF16 on the tcgen05 tensor cores with an FP32 accumulator in TMEM);
+// Learned warm start: the kernels of the network's input features and of its inference
+// (BF16 on the tcgen05 tensor cores with an FP32 accumulator in TMEM); training: ws_train.cu;
 // also the transport outputs of Sec. 5.2, which share the tiled double-float stencils.
 //
 // The paper starts Newton from u0 = 0; the damped iteration only needs an admissible start,
@@ -800,162 +800,6 @@ __global__ void k_ws_pack(const float* __restrict__ params, unsigned char* __res
   st_row8(base, row, k0, v);
 }
 
-// ---------------------------------------------------------------------------------------
-// Training (FP32 on the CUDA cores: a few GFLOP per step, run offline).
-// C[m, n] = sum_k A(m, k) B(k, n) over a 64 x 64 tile per block, 4 x 4 per thread,
-// with A(m, k) = TA ? A[k lda + m] : A[m lda + k] and B(k, n) = TB ? B[n ldb + k] : B[k ldb + n].
-// blockIdx.z selects a slice [z kchunk, (z + 1) kchunk) of k (partial sums to C + z Mr ldc).
-// Epilogues: 0 plain; 1 Z = acc + bias[n], C2 = SiLU(Z); 2 C = acc SiLU'(zp[m, n]).
-// ---------------------------------------------------------------------------------------
-template <bool TA, bool TB, int EPI>
-__global__ void __launch_bounds__(256)
-    k_gemm(int Mr, int Nc, int Kd, const float* __restrict__ A, int lda,
-           const float* __restrict__ B, int ldb, float* __restrict__ C, int ldc,
-           const float* __restrict__ bias, float* __restrict__ C2, const float* __restrict__ zp,
-           int kchunk) {
-  __shared__ float As[16][64 + 4], Bs[16][64 + 4];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  const int kbeg = blockIdx.z * kchunk, kend = min(Kd, kbeg + kchunk);
-  float acc[4][4] = {};
-  for (int k0 = kbeg; k0 < kend; k0 += 16) {
-    for (int q = threadIdx.x; q < 16 * 64; q += 256) {
-      const int kk = TA ? q / 64 : q % 16, mm = TA ? q % 64 : q / 16;
-      const int m = m0 + mm, k = k0 + kk;
-      As[kk][mm] = (m < Mr && k < kend) ? (TA ? A[(long)k * lda + m] : A[(long)m * lda + k]) : 0.f;
-      const int kb = TB ? q % 16 : q / 64, nn = TB ? q / 16 : q % 64;
-      const int n = n0 + nn, k2 = k0 + kb;
-      Bs[kb][nn] = (n < Nc && k2 < kend) ? (TB ? B[(long)n * ldb + k2] : B[(long)k2 * ldb + n]) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        a[q] = As[kk][ty * 4 + q];
-        b[q] = Bs[kk][tx * 4 + q];
-      }
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(a[p], b[q], acc[p][q]);
-    }
-    __syncthreads();
-  }
-  float* Cz = C + (long)blockIdx.z * Mr * ldc;
-#pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    const int m = m0 + ty * 4 + p;
-    if (m >= Mr) continue;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int n = n0 + tx * 4 + q;
-      if (n >= Nc) continue;
-      const long o = (long)m * ldc + n;
-      float v = acc[p][q];
-      if (EPI == 1) {
-        v += bias[n];
-        Cz[o] = v;
-        C2[o] = v / (1.0f + expf(-v));
-      } else if (EPI == 2) {
-        const float z = zp[o], s = 1.0f / (1.0f + expf(-z));
-        Cz[o] = v * s * (1.0f + z * (1.0f - s));
-      } else {
-        Cz[o] = v;
-      }
-    }
-  }
-}
-
-// sum of S partial planes of n values each (fixed order) into out
-__global__ void k_sum_partials(const float* __restrict__ part, int S, long n,
-                               float* __restrict__ out) {
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n;
-       q += (long)gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int z = 0; z < S; ++z) s += part[(long)z * n + q];
-    out[q] = s;
-  }
-}
-
-// column sums of a (rows x cols) matrix over row chunks of `chunk` rows: part[z, col]
-__global__ void k_colsum(const float* __restrict__ A, int rows, int cols, int chunk,
-                         float* __restrict__ part) {
-  const int col = blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= cols) return;
-  const int r0 = blockIdx.y * chunk, r1 = min(rows, r0 + chunk);
-  float s = 0.f;
-  for (int rr = r0; rr < r1; ++rr) s += A[(long)rr * cols + col];
-  part[(long)blockIdx.y * cols + col] = s;
-}
-
-__global__ void k_gather_rows(const float* __restrict__ X, const float* __restrict__ t,
-                              const long long* __restrict__ idx, int B, float* __restrict__ Xb,
-                              float* __restrict__ tb) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= B * 4) return;
-  const int b = q >> 2, part = q & 3;
-  const long long r = idx[b];
-  reinterpret_cast<float4*>(Xb)[(long)b * 4 + part] =
-      reinterpret_cast<const float4*>(X)[r * 4 + part];
-  if (part == 0) tb[b] = t[r];
-}
-
-// output layer: y = A2 w3 + b3, e = y - t, dy = 2 e / B, dZ2 = dy w3 SiLU'(Z2); loss partials
-__global__ void k_ws_out(const float* __restrict__ A2, const float* __restrict__ Z2,
-                         const float* __restrict__ params, const float* __restrict__ tb, int B,
-                         float* __restrict__ dy, float* __restrict__ dZ2,
-                         double* __restrict__ loss_part) {
-  const int b = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const float* w3 = params + H * K + 3 * H + 2 * H * H;
-  const float b3 = params[H * K + 4 * H + 2 * H * H];
-  double e2 = 0.0;
-  if (b < B) {
-    float s = 0.f;
-    for (int j = lane; j < H; j += 32) s = fmaf(A2[(long)b * H + j], w3[j], s);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const float e = s + b3 - tb[b];
-    const float d = 2.0f * e / (float)B;
-    if (lane == 0) dy[b] = d;
-    for (int j = lane; j < H; j += 32) {
-      const float z = Z2[(long)b * H + j], sg = 1.0f / (1.0f + expf(-z));
-      dZ2[(long)b * H + j] = d * w3[j] * sg * (1.0f + z * (1.0f - sg));
-    }
-    e2 = (double)e * (double)e;
-  }
-  __shared__ double red[8];
-  if (lane == 0) red[threadIdx.x >> 5] = e2;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < 8; ++w) s += red[w];
-    loss_part[blockIdx.x] = s;
-  }
-}
-
-__global__ void k_sum_f64(const double* __restrict__ part, int n, double scale,
-                          double* __restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s = 0.0;
-  for (int q = 0; q < n; ++q) s += part[q];
-  *out = s * scale;
-}
-
-__global__ void k_adam(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ g, long n, float lr, float b1, float b2,
-                       float c1, float c2, float eps) {
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < n;
-       q += (long)gridDim.x * blockDim.x) {
-    const float gq = g[q];
-    const float mq = b1 * m[q] + (1.0f - b1) * gq;
-    const float vq = b2 * v[q] + (1.0f - b2) * gq * gq;
-    m[q] = mq;
-    v[q] = vq;
-    p[q] -= lr * (mq / c1) / (sqrtf(vq / c2) + eps);
-  }
-}
-
 inline dim3 grid2(int N, int M) { return dim3((M + 127) / 128, N); }
 inline int nblk(long P, int t = 256) {
   long b = (P + t - 1) / t;
@@ -1140,62 +984,6 @@ cudaError_t launch_ws_mlp(const unsigned char* wpack, const float* params, const
   const long grid = ctas < (long)sms ? ctas : (long)sms;
   k_ws_mlp_tc<<<(unsigned)grid, 128 * WS_CH, SM_TOTAL, st>>>(wpack, params, X, rows, out, err,
                                                             stall);
-  return cudaGetLastError();
-}
-
-// one training step's kernels (gradient only; the trainer adds Adam)
-cudaError_t launch_ws_grad(const float* params, const float* X, const float* t,
-                           const long long* idx, int B, WsTrainBuffers& tb, cudaStream_t st) {
-  const long HH = (long)H * H;
-  const long oW0 = 0, ob0 = H * K, oW1 = ob0 + H, ob1 = oW1 + HH, oW2 = ob1 + H, ob2 = oW2 + HH,
-             ow3 = ob2 + H, ob3 = ow3 + H;
-  k_gather_rows<<<(B * 4 + 255) / 256, 256, 0, st>>>(X, t, idx, B, tb.Xb, tb.tb);
-  const dim3 gf(H / 64, (B + 63) / 64, 1);
-  // forward
-  k_gemm<false, true, 1><<<gf, 256, 0, st>>>(B, H, K, tb.Xb, K, params + oW0, K, tb.Z0, H,
-                                             params + ob0, tb.A0, nullptr, K);
-  k_gemm<false, true, 1><<<gf, 256, 0, st>>>(B, H, H, tb.A0, H, params + oW1, H, tb.Z1, H,
-                                             params + ob1, tb.A1, nullptr, H);
-  k_gemm<false, true, 1><<<gf, 256, 0, st>>>(B, H, H, tb.A1, H, params + oW2, H, tb.Z2, H,
-                                             params + ob2, tb.A2, nullptr, H);
-  const int nout = (B + 7) / 8;
-  k_ws_out<<<nout, 256, 0, st>>>(tb.A2, tb.Z2, params, tb.tb, B, tb.dy, tb.dZ2, tb.loss_part);
-  k_sum_f64<<<1, 32, 0, st>>>(tb.loss_part, nout, 1.0 / (double)B, tb.loss);
-  // backward: weight gradients over row chunks, data gradients through the layers
-  const int chunk = WS_ROW_CHUNK, S = (B + chunk - 1) / chunk;
-  float* g = tb.grad;
-  auto wgrad = [&](const float* dZ, const float* Ain, int kin, long ow, long ob) {
-    const dim3 gw((kin + 63) / 64, H / 64, S);
-    k_gemm<true, false, 0><<<gw, 256, 0, st>>>(H, kin, B, dZ, H, Ain, kin, tb.part, kin,
-                                               nullptr, nullptr, nullptr, chunk);
-    k_sum_partials<<<nblk((long)H * kin), 256, 0, st>>>(tb.part, S, (long)H * kin, g + ow);
-    k_colsum<<<dim3((H + 127) / 128, S), 128, 0, st>>>(dZ, B, H, chunk, tb.part);
-    k_sum_partials<<<1, 128, 0, st>>>(tb.part, S, H, g + ob);
-  };
-  // w3, b3: column sums of A2 dy and of dy
-  {
-    const dim3 gw(1, H / 64, S);
-    k_gemm<true, false, 0><<<gw, 256, 0, st>>>(H, 1, B, tb.A2, H, tb.dy, 1, tb.part, 1, nullptr,
-                                               nullptr, nullptr, chunk);
-    k_sum_partials<<<1, 128, 0, st>>>(tb.part, S, H, g + ow3);
-    k_colsum<<<dim3(1, S), 128, 0, st>>>(tb.dy, B, 1, chunk, tb.part);
-    k_sum_partials<<<1, 32, 0, st>>>(tb.part, S, 1, g + ob3);
-  }
-  wgrad(tb.dZ2, tb.A1, H, oW2, ob2);
-  k_gemm<false, false, 2><<<gf, 256, 0, st>>>(B, H, H, tb.dZ2, H, params + oW2, H, tb.dZ1, H,
-                                              nullptr, nullptr, tb.Z1, H);
-  wgrad(tb.dZ1, tb.A0, H, oW1, ob1);
-  k_gemm<false, false, 2><<<gf, 256, 0, st>>>(B, H, H, tb.dZ1, H, params + oW1, H, tb.dZ2, H,
-                                              nullptr, nullptr, tb.Z0, H);
-  wgrad(tb.dZ2, tb.Xb, K, oW0, ob0);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_ws_adam(float* p, float* m, float* v, const float* g, long n, float lr,
-                           int t, cudaStream_t st) {
-  const double b1 = 0.9, b2 = 0.999;
-  const float c1 = (float)(1.0 - pow(b1, t)), c2 = (float)(1.0 - pow(b2, t));
-  k_adam<<<nblk(n), 256, 0, st>>>(p, m, v, g, n, lr, (float)b1, (float)b2, c1, c2, 1e-8f);
   return cudaGetLastError();
 }
 
