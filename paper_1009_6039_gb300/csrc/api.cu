@@ -135,12 +135,13 @@ template <typename T> static const SpecTables& tables(ot_plan* p);
 template <> const SpecTables& tables<double>(ot_plan* p) { return p->tb64; }
 template <> const SpecTables& tables<float>(ot_plan* p) { return p->tb32; }
 
-// residual + coefficients of the iterate: FP64 kernel, or the double-float kernel in mixed
-// mode (which reads the split copies of the plan's f and c)
+// residual + coefficients of the iterate: FP64 kernel (coefficients to coef64 when given, else
+// to the plan's planes), or the double-float kernel in mixed mode (which reads the split copies
+// of the plan's f and c)
 template <typename T>
 static cudaError_t residual_launch(ot_plan* p, const double* f, const double* c,
                                    const double* ua, double* Fraw, const double* ub = nullptr,
-                                   int sel = 0) {
+                                   int sel = 0, double* coef64 = nullptr) {
   const size_t P = (size_t)p->N * p->M;
   Interp ip;
   if (p->interp) {
@@ -154,8 +155,8 @@ static cudaError_t residual_launch(ot_plan* p, const double* f, const double* c,
     return launch_residual_dd(p->fdd, p->cdd, ua, p->N, p->M, Fraw, (float*)p->coef,
                               p->partials, p->sc, p->stream, ub, sel, p->op_simple, btc(p),
                               ip);
-  return launch_residual<double>(f, c, ua, p->N, p->M, Fraw, (double*)p->coef, p->partials,
-                                 p->sc, p->stream, ub, sel, nullptr, p->op_simple, ip);
+  return launch_residual(f, c, ua, p->N, p->M, Fraw, coef64 ? coef64 : (double*)p->coef,
+                         p->partials, p->sc, p->stream, ub, sel, p->op_simple, ip);
 }
 
 static bool reorth_on(const ot_plan* p) { return p->reorth == 1; }
@@ -2347,12 +2348,14 @@ static int eval_residual_impl(ot_plan* p, const double* f, const double* c, cons
   if (p->interp)  // c holds g: its grid gradient for the interpolated grad g
     LAUNCH(p, OT_PROF_OTHER, -1, 1,
            launch_grad4(c, N, M, p->gxy, p->gxy + P, p->gxy32, p->gxy32 + P, p->stream));
+  // FP64: the coefficients straight into the caller's planes, unless these overlap an input
+  auto apart = [&](const double* x) { return !x || x + P <= coef || coef + 5 * P <= x; };
+  const bool direct = sizeof(T) == 8 && coef && apart(f) && apart(c) && apart(u);
   LAUNCH(p, OT_PROF_RESIDUAL, -1, 1,
-         residual_launch<T>(p, f, c, u, p->Fraw, nullptr, 0));
+         residual_launch<T>(p, f, c, u, p->Fraw, nullptr, 0, direct ? coef : nullptr));
   LAUNCH(p, OT_PROF_OTHER, -1, 1,
-         launch_residual_l2(p->Fraw, N, M, p->partials, p->sc, p->stream));
-  if (F) LAUNCH(p, OT_PROF_OTHER, -1, 1, launch_shifted_residual(p->Fraw, F, N, M, p->sc, p->stream));
-  if (coef)
+         launch_residual_l2(p->Fraw, N, M, p->partials, p->sc, p->stream, Bat(), F));
+  if (coef && !direct)
     LAUNCH(p, OT_PROF_OTHER, -1, 1,
            launch_convert<T>(p->coef, sizeof(T) == 8, coef, 1, 5 * P, p->stream));
   RET(read_scalars(p));

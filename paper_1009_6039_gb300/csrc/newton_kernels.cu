@@ -484,18 +484,6 @@ __device__ __forceinline__ int wrap_near(int a, int L) {  // a in [-L, 2L)
   return a < 0 ? a + L : (a >= L ? a - L : a);
 }
 
-struct ResidConsts {
-  double Mh, Nh, Mh2, Nh2;  // M/12, N/12, M^2/12, N^2/12
-  double MNh;               // M N / 144
-  double w3M, w3N;          // 1/(3M), 1/(3N): Simpson weights (2 or 4) x these
-  int nob;                  // 1: the simplified operator (b = 0, Sec. 3.3 remark)
-  // interpolation of g (Sec. 4 intro; Sec. 5.2, 5.3): 0 cubic B-spline of the coefficients c;
-  // 1 bilinear, 2 nearest node of the grid values (then c = g) and of the grid gradient gx, gy
-  int interp;
-  const double* gx;
-  const double* gy;
-};
-
 template <typename G>
 __device__ __forceinline__ void bspline_w(G t, G w[4], G dw[4]) {
   const G s = (G)1 - t;
@@ -509,225 +497,6 @@ __device__ __forceinline__ void bspline_w(G t, G w[4], G dw[4]) {
   dw[1] = (G)0.5 * ((G)3 * t2 - (G)4 * t);
   dw[2] = (G)0.5 * ((G)-3 * t2 + (G)2 * t + (G)1);
   dw[3] = (G)0.5 * t2;
-}
-
-// value weights only; w[2] from the partition of unity sum w = 1
-__device__ __forceinline__ void bspline_v(double t, double w[4]) {
-  const double s = 1.0 - t;
-  const double t2 = t * t, t3 = t2 * t;
-  const double sixth = 1.0 / 6.0;
-  w[0] = s * s * s * sixth;
-  w[1] = fma(0.5, t3, (2.0 / 3.0) - t2);
-  w[3] = t3 * sixth;
-  w[2] = 1.0 - w[0] - w[1] - w[3];
-}
-
-template <typename T>
-__global__ void __launch_bounds__(RTX * RTY / RPT)
-    k_residual(const double* __restrict__ f, const double* __restrict__ c,
-               const float* __restrict__ c32, const double* __restrict__ ua,
-               const double* __restrict__ ub, int sel, int N, int M, ResidConsts K,
-               double* __restrict__ Fraw, T* __restrict__ coef, double* partials,
-               DevScalars* sc) {
-  __shared__ double tile[RTY + 4][RTX + 4];
-  __shared__ double dyt[RTY][RTX + 4];  // unscaled y-difference of u (halo 2 in x)
-  const double* __restrict__ u = (ub && ((sc->upar ^ sel) & 1)) ? ub : ua;
-  const int bx = blockIdx.x * RTX, by = blockIdx.y * RTY;
-  const int tid = threadIdx.x;
-  for (int idx = tid; idx < (RTY + 4) * (RTX + 4); idx += blockDim.x) {
-    const int r = idx / (RTX + 4), cc = idx - r * (RTX + 4);
-    int gi = by + r - 2, gj = bx + cc - 2;
-    while (gi < 0) gi += N;
-    while (gi >= N) gi -= N;
-    while (gj < 0) gj += M;
-    while (gj >= M) gj -= M;
-    tile[r][cc] = u[(size_t)gi * M + gj];
-  }
-  __syncthreads();
-  for (int idx = tid; idx < RTY * (RTX + 4); idx += blockDim.x) {
-    const int r = idx / (RTX + 4), cc = idx - r * (RTX + 4);
-    dyt[r][cc] = -tile[r + 4][cc] + 8.0 * tile[r + 3][cc] - 8.0 * tile[r + 1][cc] + tile[r][cc];
-  }
-  __syncthreads();
-  // FP64 partials: sum fn, max Fraw, min Fraw, min det, non-finite count; Simpson sums of
-  // the coefficients (Jacobian only) in the coefficient precision T
-  double v64[5] = {0.0, -INFINITY, INFINITY, INFINITY, 0.0};
-  const int kind64[5] = {0, 1, 2, 2, 0};
-  T simp[5] = {(T)0, (T)0, (T)0, (T)0, (T)0};
-  const int tx = tid % RTX, ty0 = tid / RTX;
-  const int j = bx + tx;
-  const size_t P = (size_t)N * M;
-  const T wx = (T)(((j & 1) ? 4.0 : 2.0) * K.w3M);
-#pragma unroll 1
-  for (int rr = 0; rr < RPT; ++rr) {
-    const int ty = ty0 + rr * (RTY / RPT);
-    const int i = by + ty;
-    if (i >= N || j >= M) continue;
-    const int r = ty + 2, q = tx + 2;
-    const double ux =
-        (-tile[r][q + 2] + 8.0 * tile[r][q + 1] - 8.0 * tile[r][q - 1] + tile[r][q - 2]) * K.Mh;
-    const double uy = dyt[ty][q] * K.Nh;
-    const double uxx = (-tile[r][q + 2] + 16.0 * tile[r][q + 1] - 30.0 * tile[r][q] +
-                        16.0 * tile[r][q - 1] - tile[r][q - 2]) * K.Mh2;
-    const double uyy = (-tile[r + 2][q] + 16.0 * tile[r + 1][q] - 30.0 * tile[r][q] +
-                        16.0 * tile[r - 1][q] - tile[r - 2][q]) * K.Nh2;
-    const double uxy = (-dyt[ty][q + 2] + 8.0 * dyt[ty][q + 1] - 8.0 * dyt[ty][q - 1] +
-                        dyt[ty][q - 2]) * K.MNh;
-    // g at the displaced point x + grad u, in grid units, periodic cubic B-spline
-    const double gxp = (double)j + (double)M * ux, gyp = (double)i + (double)N * uy;
-    const double fj = floor(gxp), fi = floor(gyp);
-    const double tx_ = gxp - fj, ty_ = gyp - fi;
-    const int j0 = wrapi((int)fj, M), i0 = wrapi((int)fi, N);
-    int jj[4], ii[4];
-    jj[0] = j0 == 0 ? M - 1 : j0 - 1;
-    jj[1] = j0;
-    jj[2] = wrap_near(j0 + 1, M);
-    jj[3] = wrap_near(j0 + 2, M);
-    ii[0] = i0 == 0 ? N - 1 : i0 - 1;
-    ii[1] = i0;
-    ii[2] = wrap_near(i0 + 1, N);
-    ii[3] = wrap_near(i0 + 2, N);
-    double G = 0.0;
-    T Gx, Gy;
-    if (K.interp == 2) {  // nearest node (round half up)
-      const size_t q = (size_t)wrapi((int)floor(gyp + 0.5), N) * M + wrapi((int)floor(gxp + 0.5), M);
-      G = __ldg(c + q);
-      Gx = (T)__ldg(K.gx + q);
-      Gy = (T)__ldg(K.gy + q);
-    } else if (K.interp == 1) {  // bilinear on the cell (i0, j0) .. (i0 + 1, j0 + 1)
-      const double w[4] = {(1.0 - tx_) * (1.0 - ty_), tx_ * (1.0 - ty_), (1.0 - tx_) * ty_,
-                           tx_ * ty_};
-      const size_t q[4] = {(size_t)ii[1] * M + jj[1], (size_t)ii[1] * M + jj[2],
-                           (size_t)ii[2] * M + jj[1], (size_t)ii[2] * M + jj[2]};
-      double a = 0.0, b = 0.0;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        G += w[k] * __ldg(c + q[k]);
-        a += w[k] * __ldg(K.gx + q[k]);
-        b += w[k] * __ldg(K.gy + q[k]);
-      }
-      Gx = (T)a;
-      Gy = (T)b;
-    } else if (sizeof(T) == 8) {
-      double wxv[4], dwx[4], wyv[4], dwy[4];
-      bspline_w<double>(tx_, wxv, dwx);
-      bspline_w<double>(ty_, wyv, dwy);
-      double gx = 0.0, gy = 0.0;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const double* crow = c + (size_t)ii[b] * M;
-        double sv = 0.0, sd = 0.0;
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          const double cv = __ldg(crow + jj[a]);
-          sv += cv * wxv[a];
-          sd += cv * dwx[a];
-        }
-        G += sv * wyv[b];
-        gx += sd * wyv[b];
-        gy += sv * dwy[b];
-      }
-      Gx = (T)(gx * (double)M);
-      Gy = (T)(gy * (double)N);
-    } else {
-      // value in FP64 (it enters the residual); gradient (Jacobian only) in FP32 from the
-      // FP32 copy of the coefficients
-      double wxv[4], wyv[4];
-      bspline_v(tx_, wxv);
-      bspline_v(ty_, wyv);
-      float wxf[4], dwx[4], wyf[4], dwy[4];
-      bspline_w<float>((float)tx_, wxf, dwx);
-      bspline_w<float>((float)ty_, wyf, dwy);
-      float gx = 0.f, gy = 0.f;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const double* crow = c + (size_t)ii[b] * M;
-        const float* crow32 = c32 + (size_t)ii[b] * M;
-        double sv = 0.0;
-        float svf = 0.f, sdf = 0.f;
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          sv += __ldg(crow + jj[a]) * wxv[a];
-          const float cf = __ldg(crow32 + jj[a]);
-          svf += cf * wxf[a];
-          sdf += cf * dwx[a];
-        }
-        G += sv * wyv[b];
-        gx += sdf * wyf[b];
-        gy += svf * dwy[b];
-      }
-      Gx = (T)(gx * (float)M);
-      Gy = (T)(gy * (float)N);
-    }
-    const double det = (1.0 + uxx) * (1.0 + uyy) - uxy * uxy;
-    const double fn = G * det;
-    const size_t p = (size_t)i * M + j;
-    const double fr = f[p] - fn;
-    Fraw[p] = fr;
-    // coefficients of the linearisation (Jacobian only): precision T
-    const T Gt = (T)G, dett = (T)det;
-    const T a11 = Gt * ((T)1 + (T)uyy), a12 = -Gt * (T)uxy, a22 = Gt * ((T)1 + (T)uxx);
-    const T b1 = K.nob ? (T)0 : dett * Gx, b2 = K.nob ? (T)0 : dett * Gy;
-    coef[p] = a11;
-    coef[P + p] = a12;
-    coef[2 * P + p] = a22;
-    coef[3 * P + p] = b1;
-    coef[4 * P + p] = b2;
-    const T w = (T)((i & 1) ? 4.0 : 2.0) * (T)K.w3N * wx;
-    simp[0] += w * a11;
-    simp[1] += w * a12;
-    simp[2] += w * a22;
-    simp[3] += w * b1;
-    simp[4] += w * b2;
-    if (isfinite(fn)) {
-      v64[0] += fn;
-      v64[1] = fmax(v64[1], fr);
-      v64[2] = fmin(v64[2], fr);
-    } else {
-      v64[4] += 1.0;
-    }
-    v64[3] = fmin(v64[3], det);
-  }
-  double v[10];
-  const int kind[10] = {0, 0, 0, 0, 0, 0, 1, 2, 2, 0};
-  block_reduce<5>(v64, kind64);
-  if (sizeof(T) == 8) {
-    double sd[5];
-    const int k5[5] = {0, 0, 0, 0, 0};
-#pragma unroll
-    for (int a = 0; a < 5; ++a) sd[a] = (double)simp[a];
-    block_reduce<5>(sd, k5);
-#pragma unroll
-    for (int a = 0; a < 5; ++a) v[1 + a] = sd[a];
-  } else {
-    float sf[5];
-#pragma unroll
-    for (int a = 0; a < 5; ++a) sf[a] = (float)simp[a];
-    block_sum_f<5>(sf);
-#pragma unroll
-    for (int a = 0; a < 5; ++a) v[1 + a] = (double)sf[a];
-  }
-  v[0] = v64[0];
-  v[6] = v64[1];
-  v[7] = v64[2];
-  v[8] = v64[3];
-  v[9] = v64[4];
-  if (!publish_partials<10>(v, partials, &sc->ticket[TK_RESID])) return;
-  const unsigned int nb = gridDim.x * gridDim.y;
-  reduce_partials<10>(v, kind, partials, nb);
-  if (threadIdx.x == 0) {
-    const double Pd = (double)N * (double)M;
-    const double mean_fn = v[0] / Pd;
-    const double shift = mean_fn - 1.0;
-    sc->mean_fn = mean_fn;
-    sc->shift = shift;
-    sc->res_inf = fmax(fabs(v[6] + shift), fabs(v[7] + shift));
-    for (int a = 0; a < 5; ++a) sc->abar[a] = v[1 + a];
-    sc->min_det = v[8];
-    sc->k1_nonfinite = (int)v[9];
-    sc->admissible = (v[9] == 0.0 && isfinite(sc->res_inf) && v[8] > 0.0) ? 1 : 0;
-    sc->ticket[TK_RESID] = 0;
-  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1078,91 +847,6 @@ cudaError_t launch_residual_dd(const float2* fdd, const float2* cdd, const doubl
   if (ip.mode && !(ip.gx32 && ip.gy32)) return cudaErrorInvalidValue;
   k_residual_dd<<<bgrid(grid, bat), RTX * RTY / RPT, 0, st>>>(fdd, cdd, ua, ub, sel, N, M, K,
                                                                 Fraw, coef, partials, sc, bat);
-  return cudaGetLastError();
-}
-
-int residual_partial_blocks(int N, int M) {
-  return ((M + RTX - 1) / RTX) * ((N + RTY - 1) / RTY);
-}
-
-template <typename T>
-cudaError_t launch_residual(const double* f, const double* c, const double* ua, int N, int M,
-                            double* Fraw, T* coef, double* partials, DevScalars* sc,
-                            cudaStream_t st, const double* ub, int sel, const float* c32,
-                            int simplified, Interp ip) {
-  dim3 grid((M + RTX - 1) / RTX, (N + RTY - 1) / RTY);
-  ResidConsts K;
-  K.Mh = (double)M / 12.0;
-  K.Nh = (double)N / 12.0;
-  K.Mh2 = (double)M * (double)M / 12.0;
-  K.Nh2 = (double)N * (double)N / 12.0;
-  K.MNh = K.Mh * K.Nh;
-  K.w3M = 1.0 / (3.0 * (double)M);
-  K.w3N = 1.0 / (3.0 * (double)N);
-  K.nob = simplified ? 1 : 0;
-  K.interp = ip.mode;
-  K.gx = ip.gx;
-  K.gy = ip.gy;
-  if (ip.mode && !(ip.gx && ip.gy)) return cudaErrorInvalidValue;
-  if (sizeof(T) == 4 && !c32) return cudaErrorInvalidValue;
-  k_residual<T><<<grid, RTX * RTY / RPT, 0, st>>>(f, c, c32, ua, ub, sel, N, M, K, Fraw, coef,
-                                                  partials, sc);
-  return cudaGetLastError();
-}
-
-// sum of (Fraw + shift)^2 -> res_l2sum
-__global__ void k_residual_l2(const double* __restrict__ Fraw, long P, double* partials,
-                              DevScalars* sc, Bat bat) {
-  Fraw = badv(Fraw, bat);
-  partials = badv(partials, bat);
-  sc = badv(sc, bat);
-  if (bskip(sc, bat)) return;
-  const double s = sc->shift;
-  double v[1] = {0.0};
-  const int kind[1] = {0};
-  for (long p = blockIdx.x * (long)blockDim.x + threadIdx.x; p < P;
-       p += (long)gridDim.x * blockDim.x) {
-    const double r = Fraw[p] + s;
-    v[0] += r * r;
-  }
-  block_reduce<1>(v, kind);
-  if (!publish_partials<1>(v, partials, &sc->ticket[TK_NORM])) return;
-  reduce_partials<1>(v, kind, partials, gridDim.x);
-  if (threadIdx.x == 0) {
-    sc->res_l2sum = v[0];
-    sc->ticket[TK_NORM] = 0;
-  }
-}
-
-cudaError_t launch_residual_l2(const double* Fraw, int N, int M, double* partials,
-                               DevScalars* sc, cudaStream_t st, Bat bat) {
-  k_residual_l2<<<bgrid(dim3(reduce_blocks()), bat), 256, 0, st>>>(Fraw, (long)N * M, partials,
-                                                                   sc, bat);
-  return cudaGetLastError();
-}
-
-__global__ void k_shifted(const double* __restrict__ Fraw, double* __restrict__ F, long P,
-                          const DevScalars* __restrict__ sc) {
-  const double s = sc->shift;
-  for (long p = blockIdx.x * (long)blockDim.x + threadIdx.x; p < P;
-       p += (long)gridDim.x * blockDim.x)
-    F[p] = Fraw[p] + s;
-}
-
-// in-place form (F += shift): one pointer, so no aliasing of restrict-qualified arguments
-__global__ void k_shift_inplace(double* F, long P, const DevScalars* __restrict__ sc) {
-  const double s = sc->shift;
-  for (long p = blockIdx.x * (long)blockDim.x + threadIdx.x; p < P;
-       p += (long)gridDim.x * blockDim.x)
-    F[p] += s;
-}
-
-cudaError_t launch_shifted_residual(const double* Fraw, double* F, int N, int M,
-                                    const DevScalars* sc, cudaStream_t st) {
-  if (Fraw == F)
-    k_shift_inplace<<<reduce_blocks(), 256, 0, st>>>(F, (long)N * M, sc);
-  else
-    k_shifted<<<reduce_blocks(), 256, 0, st>>>(Fraw, F, (long)N * M, sc);
   return cudaGetLastError();
 }
 
@@ -2007,10 +1691,6 @@ cudaError_t launch_convert(const void* in, int in_d, void* out, int out_d, long 
 }
 
 #define OTGB_INST_NEWTON(T)                                                                   \
-  template cudaError_t launch_residual<T>(const double*, const double*, const double*, int,   \
-                                          int, double*, T*, double*, DevScalars*,             \
-                                          cudaStream_t, const double*, int, const float*, int,  \
-                                          Interp);                                            \
   template cudaError_t launch_gmres_init<T>(const double*, const T*, T*, long, int, double*,  \
                                             DevScalars*, int, cudaStream_t, T*, Bat);         \
   template cudaError_t launch_gmres_dots<T>(const T*, const T*, long, double*, DevScalars*,   \

@@ -16,8 +16,9 @@
 namespace {
 
 // Largest grid served: N, M <= 2048.  The residual kernel uses one block per 32 x 32 tile,
-// i.e. at most 64 * 64 = 4096 blocks with 10 partials each; the l2 reduction uses 2 blocks
-// per SM with 1 partial each (far fewer).
+// i.e. at most 64 * 64 = 4096 blocks with 10 partials each, and lower tiles only where that
+// makes fewer than 4 * 608 blocks; the l2 reduction uses at most 2 blocks per SM with 1 partial
+// each (far fewer).
 constexpr int kMaxSide = 2048;
 constexpr size_t kMaxResidualBlocks = (kMaxSide / 32) * (kMaxSide / 32);
 constexpr size_t kHeaderBytes = (sizeof(otgb::DevScalars) + 255) / 256 * 256;
@@ -77,10 +78,8 @@ extern "C" int ot_eval_residual_noalloc(int32_t N, int32_t M, const double* f, c
   // the array keeps the previous call's contents: the reduction tickets must start at zero
   if (cudaMemsetAsync(sc, 0, sizeof(DevScalars), st) != cudaSuccess) return OT_ECUDA;
   // F receives f - f_n first, then the mass translation shift in place
-  if (launch_residual<double>(f, c, u, N, M, F, coef, partials, sc, st) != cudaSuccess)
-    return OT_ECUDA;
-  if (launch_residual_l2(F, N, M, partials, sc, st) != cudaSuccess) return OT_ECUDA;
-  if (launch_shifted_residual(F, F, N, M, sc, st) != cudaSuccess) return OT_ECUDA;
+  if (launch_residual(f, c, u, N, M, F, coef, partials, sc, st) != cudaSuccess) return OT_ECUDA;
+  if (launch_residual_l2(F, N, M, partials, sc, st, Bat(), F) != cudaSuccess) return OT_ECUDA;
   DevScalars h;
   if (cudaMemcpyAsync(&h, sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, st) != cudaSuccess)
     return OT_ECUDA;

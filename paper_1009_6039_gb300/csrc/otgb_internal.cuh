@@ -320,14 +320,12 @@ struct Interp {
 cudaError_t launch_grad4(const double* g, int N, int M, double* gx, double* gy, float* gx32,
                          float* gy32, cudaStream_t st);
 // u = ub ? (upar ^ sel ? ub : ua) : ua   (sel 0: current iterate, 1: candidate);
-// simplified: b = 0 in the coefficients (the operator without the grad g term)
-// c32 (optional, FP32 copy of c): used for the gradient of the interpolant in FP32 mode
-template <typename T>
+// simplified: b = 0 in the coefficients (the operator without the grad g term).  FP64
+// (residual_f64.cu); partials: 10 doubles per block, residual_partial_blocks(N, M) blocks
 cudaError_t launch_residual(const double* f, const double* c, const double* ua, int N, int M,
-                            double* Fraw, T* coef, double* partials, DevScalars* sc,
+                            double* Fraw, double* coef, double* partials, DevScalars* sc,
                             cudaStream_t st, const double* ub = nullptr, int sel = 0,
-                            const float* c32 = nullptr, int simplified = 0,
-                            Interp ip = Interp());
+                            int simplified = 0, Interp ip = Interp());
 // mixed mode: the residual in double-float arithmetic from (hi, lo) float pairs of f and c
 cudaError_t launch_residual_dd(const float2* fdd, const float2* cdd, const double* ua, int N,
                                int M, double* Fraw, float* coef, double* partials,
@@ -337,10 +335,10 @@ cudaError_t launch_residual_dd(const float2* fdd, const float2* cdd, const doubl
 // out[k] = (hi, lo) float pair of in[k]
 cudaError_t launch_split_dd(const double* in, float2* out, long n, cudaStream_t st,
                             Bat bat = Bat());
+// res_l2sum = sum of (Fraw + shift)^2; F (optional, may be Fraw) = Fraw + shift
 cudaError_t launch_residual_l2(const double* Fraw, int N, int M, double* partials,
-                               DevScalars* sc, cudaStream_t st, Bat bat = Bat());
-cudaError_t launch_shifted_residual(const double* Fraw, double* F, int N, int M,
-                                    const DevScalars* sc, cudaStream_t st);
+                               DevScalars* sc, cudaStream_t st, Bat bat = Bat(),
+                               double* F = nullptr);
 cudaError_t launch_subtract_mean(double* u, int N, int M, double* partials, DevScalars* sc,
                                  double* mean_out, cudaStream_t st);
 // out = u[upar] - mean(u[upar])
