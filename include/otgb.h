@@ -157,7 +157,7 @@ extern "C" {
                                    conditional WHILE node, a step per iteration (0 <= s <= 16,
                                    default 7; a plan set captures every step plainly).  Same
                                    arithmetic for every s */
-#define OT_OPT_KRYLOV_BLOCKS 29 /* blocks of 256 threads per SM for the GMRES vector kernels
+#define OT_OPT_KRYLOV_BLOCKS 29 /* most blocks of 256 threads per SM for the GMRES vector kernels
                                    (multi-dot, update, init, combine), 1..8 (default 2); the
                                    block partial sums change with it, so results differ in
                                    the last bits between settings (each is deterministic) */

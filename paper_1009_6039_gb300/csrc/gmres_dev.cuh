@@ -8,10 +8,10 @@
 
 namespace otgb {
 
-// Finish the FP32 multi-dot of step j = J - 1 from the dots kernel's per-block sums (nb
-// blocks, J + 1 values each: V_i.w for i < J, then w.w): every sum is taken by one warp in a
-// fixed order (lane-strided, then a shuffle tree), so that every block of the calling grid
-// obtains the same values.  h_i = scale_i V_i.w, and ||w - sum h_i v_i||^2 = w.w - sum h_i^2
+// Finish the multi-dot of step j = J - 1 from the dots kernel's per-block sums (nb blocks, J + 1
+// values each: V_i.w for i < J, then w.w; FP32: block by block, FP64: value by value): every sum
+// is taken by one warp in a fixed order (lane-strided, then a shuffle tree), so that every block
+// of the calling grid obtains the same values.  h_i = scale_i V_i.w, and ||w - sum h_i v_i||^2 = w.w - sum h_i^2
 // (Pythagoras, v_i orthonormal): below 1e-6 w.w the step is weak and the cycle ends (the
 // restart's explicit residual decides).  The FP64 scalars are formed by thread 0 alone (FP64
 // runs at a small fraction of the FP32 rate on this GPU, and every thread of a large grid
@@ -19,20 +19,21 @@ namespace otgb {
 // Out, in every thread: the update's coefficients h_i scale_i (the basis is stored unscaled)
 // and 1 / hn (0 when weak); in thread 0 only: h, hn = ||w - sum h_i v_i|| and weak.  All
 // threads of the block call it (two barriers).
-template <int J>
-__device__ __forceinline__ void finish_multidot_f32(const double* partials, int nb,
-                                                    const DevScalars* sc, double (&hv)[J],
-                                                    double& hn, double& inv_hn, bool& weak,
-                                                    float (&coefs)[J]) {
-  // (the sums in FP32, as the block sums themselves)
-  __shared__ float sv[OTGB_MAXM + 1];
-  __shared__ float scoef[OTGB_MAXM];
+template <typename T, int J>
+__device__ __forceinline__ void finish_multidot(const double* partials, int nb,
+                                                const DevScalars* sc, double (&hv)[J],
+                                                double& hn, double& inv_hn, bool& weak,
+                                                T (&coefs)[J]) {
+  // (the sums in the vectors' precision, as the block sums themselves)
+  __shared__ T sv[OTGB_MAXM + 1];
+  __shared__ T scoef[OTGB_MAXM];
   __shared__ double sinv;
-  const float* pf = reinterpret_cast<const float*>(partials);
+  const T* pf = reinterpret_cast<const T*>(partials);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int a = wid; a <= J; a += nw) {
-    float x = 0.f;
-    for (int b = lane; b < nb; b += 32) x += pf[(size_t)b * (J + 1) + a];
+    T x = (T)0;
+    for (int b = lane; b < nb; b += 32)
+      x += pf[sizeof(T) == 4 ? (size_t)b * (J + 1) + a : (size_t)a * nb + b];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     if (lane == 0) sv[a] = x;
@@ -50,7 +51,7 @@ __device__ __forceinline__ void finish_multidot_f32(const double* partials, int 
     inv_hn = weak ? 0.0 : rsqrt(hn2);
     hn = hn2 * inv_hn;
 #pragma unroll
-    for (int i = 0; i < J; ++i) scoef[i] = (float)(hv[i] * sc->scale[i]);
+    for (int i = 0; i < J; ++i) scoef[i] = (T)(hv[i] * sc->scale[i]);
     sinv = inv_hn;
   }
   __syncthreads();
@@ -65,10 +66,10 @@ __device__ __forceinline__ void finish_multidot_f32(const double* partials, int 
 // count, and (in a graph) the conditional handle of the next step.  Every scalar it needs is
 // loaded first, as independent loads, so that the one thread that runs it waits for one
 // memory round trip instead of one per dependent access.
-// FAST (the FP32 step): the rotation from one reciprocal square root, c = a / r = a rsqrt(r^2)
+// FAST (single problems): the rotation from one reciprocal square root, c = a / r = a rsqrt(r^2)
 // and s = b rsqrt(r^2), and the basis scale 1 / hn passed in (rsqrt of the Pythagorean
 // square), in place of a square root and divisions, whose FP64 forms are slow on this GPU
-// (the close is one thread on the step's critical path); the FP64 step keeps them.
+// (the close is one thread on the step's critical path); a plan set's classes keep them.
 template <int J, bool FAST = false>
 __device__ void arnoldi_close_j(DevScalars* sc, const double (&h)[J], double hn, bool weak,
                                 double inv_hn = 0.0) {
@@ -116,7 +117,7 @@ __device__ void arnoldi_close_j(DevScalars* sc, const double (&h)[J], double hn,
   sc->gv[j] = c * gvj;
   sc->iters = iters + 1;
   sc->jend = j + 1;
-  if (!FAST) sc->relres = fabs(g1) / bnorm;  // informational (the FP32 step skips it)
+  if (!FAST) sc->relres = fabs(g1) / bnorm;  // informational (the fast close skips it)
   int done = 0;
   if (weak) {
     done = 1;

@@ -1059,7 +1059,7 @@ __device__ __forceinline__ void dots_j(const T* __restrict__ V, const T* __restr
   double v[J + 1];
   if constexpr (sizeof(T) == 4) {
     if (split && pass == 0 && !sc->reorth) {
-      // single-reduction step in FP32 (split): the block's sums go to its partials and the
+      // single-reduction step (split): the block's sums go to its partials and the
       // update kernel finishes the step (every block of it sums the partials in the same
       // order; its block 0 closes the step) -- no last-block pass and no serial close here
       block_sum_f<J + 1>(acc);
@@ -1075,6 +1075,14 @@ __device__ __forceinline__ void dots_j(const T* __restrict__ V, const T* __restr
 #pragma unroll
     for (int i = 0; i <= J; ++i) v[i] = (double)acc[i];
   } else {
+    if (split && pass == 0 && !sc->reorth) {
+      // the same split in FP64, the sums value by value
+      double s;
+      if (block_fold<J + 1>(acc, s))
+        partials[(size_t)(threadIdx.x >> 3) * gridDim.x + blockIdx.x] = s;
+      if (blockIdx.x == 0 && threadIdx.x == 0) sc->jd = J - 1;
+      return;
+    }
     int kind[J + 1];
 #pragma unroll
     for (int i = 0; i <= J; ++i) {
@@ -1151,11 +1159,8 @@ __device__ __forceinline__ void update_j(T* __restrict__ V, const T* __restrict_
   T coefs[J];
   double hv[J], hn = 0.0, inv_hn = 0.0;
   bool weak = false;
-  if (sizeof(T) == 4 && mode == 3 && split) {
-    float cf[J];
-    finish_multidot_f32<J>(partials, gridDim.x, sc, hv, hn, inv_hn, weak, cf);
-#pragma unroll
-    for (int i = 0; i < J; ++i) coefs[i] = (T)cf[i];
+  if (mode == 3 && split) {
+    finish_multidot<T, J>(partials, gridDim.x, sc, hv, hn, inv_hn, weak, coefs);
   } else {
 #pragma unroll
     for (int i = 0; i < J; ++i)
@@ -1166,9 +1171,9 @@ __device__ __forceinline__ void update_j(T* __restrict__ V, const T* __restrict_
   const T* src = (mode == 2) ? Vn : w;
   T acc = (T)0;
   constexpr int W = Vec16<T>::W;
-  // FP32 mode 3: block 0 closes the step (one thread's serial FP64 work and round trips)
+  // split mode 3: block 0 closes the step (one thread's serial FP64 work and round trips)
   // while the other blocks form v_(j+1); otherwise every block takes part
-  const bool closer = sizeof(T) == 4 && mode == 3 && split && gridDim.x > 1;
+  const bool closer = mode == 3 && split && gridDim.x > 1;
   if (closer && blockIdx.x == 0) {
     if (threadIdx.x == 0) {
 #pragma unroll
@@ -1202,10 +1207,9 @@ __device__ __forceinline__ void update_j(T* __restrict__ V, const T* __restrict_
     acc += x * x;
   }
   // mode 1: first of two passes, the norm follows the second; mode 3: the step was closed
-  // by block 0 above (FP32) or by the multi-dot (FP64)
+  // by block 0 above (single problems) or by the multi-dot (a plan set's classes)
   if (mode == 1 || mode == 3) {
-    if (sizeof(T) == 4 && mode == 3 && split && !closer && blockIdx.x == 0 &&
-        threadIdx.x == 0) {
+    if (mode == 3 && split && !closer && blockIdx.x == 0 && threadIdx.x == 0) {
 #pragma unroll
       for (int i = 0; i < J; ++i) sc->hcol[i] = hv[i];
       arnoldi_close_j<J, true>(sc, hv, hn, weak, inv_hn);
@@ -1237,10 +1241,10 @@ __global__ void k_gmres_update(T* __restrict__ V, const T* __restrict__ w, long 
   partials = badv(partials, bat);
   sc = badv(sc, bat);
   if (bskip(sc, bat) || sc->cycle_done) return;
-  // mode 3 follows the multi-dot of step jd (FP32, single problem: the update closes the
-  // step itself and advances sc->j, so it reads the step from jd; FP64 and plan-set classes:
-  // the multi-dot closed it and advanced sc->j)
-  const bool split = sizeof(T) == 4 && !bat.on;
+  // mode 3 follows the multi-dot of step jd (single problem: the update closes the step
+  // itself and advances sc->j, so it reads the step from jd; plan-set classes: the multi-dot
+  // closed it and advanced sc->j)
+  const bool split = !bat.on;
   switch (mode == 3 ? (split ? sc->jd : sc->j - 1) : sc->j) {
 #define OTGB_UPD_CASE(k) \
   case k:                \

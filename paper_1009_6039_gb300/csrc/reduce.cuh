@@ -53,6 +53,40 @@ __device__ void block_reduce(double (&v)[NV], const int (&kind)[NV]) {
   __syncthreads();
 }
 
+// Sums of NV <= 16 values per thread over a block of 256: the lanes of a warp exchange halves of
+// the values, so that a warp takes NP + 4 - log2(NP) FP64 additions (NP: NV rounded up to a power
+// of two) where a shuffle tree per value takes 5 NV; FP64 starts one warp instruction per 16
+// clocks and SM here.  Thread 8 a (a < NV) receives sum a; true in those threads.
+template <int NV>
+__device__ bool block_fold(const double (&v)[NV], double& sum) {
+  constexpr int NP = NV > 8 ? 16 : (NV > 4 ? 8 : (NV > 2 ? 4 : NV));
+  __shared__ double red[8][NP];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  double x[NP];
+#pragma unroll
+  for (int a = 0; a < NP; ++a) x[a] = a < NV ? v[a] : 0.0;
+  int o = 16;
+#pragma unroll
+  for (int h = NP / 2; h > 0; h /= 2, o /= 2) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int a = 0; a < h; ++a)
+      x[a] = (up ? x[a + h] : x[a]) + __shfl_xor_sync(0xffffffffu, up ? x[a] : x[a + h], o);
+  }
+#pragma unroll
+  for (; o > 0; o /= 2) x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+  if (lane % (32 / NP) == 0) red[wid][lane / (32 / NP)] = x[0];
+  __syncthreads();
+  const int a = threadIdx.x >> 3;
+  if (wid * 4 >= NV) return false;  // (whole warps)
+  double s = a < NV ? red[threadIdx.x & 7][a] : 0.0;
+  s += __shfl_xor_sync(0xffffffffu, s, 4);
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  sum = s;
+  return (threadIdx.x & 7) == 0 && a < NV;
+}
+
 // Write the block's partials, take a ticket; returns true in the (whole) last block,
 // after which `partials` of all blocks are visible.
 template <int NV>

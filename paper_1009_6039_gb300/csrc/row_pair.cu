@@ -124,7 +124,7 @@ __device__ __forceinline__ void update_r2c_pair_j(float* __restrict__ V,
   double hv[J], hn = 0.0, inv_hn = 0.0;
   bool weak = false;
   float coefs[J];
-  finish_multidot_f32<J>(partials, nb, sc, hv, hn, inv_hn, weak, coefs);
+  finish_multidot<float, J>(partials, nb, sc, hv, hn, inv_hn, weak, coefs);
   if (blockIdx.x == 0) {
     if (threadIdx.x == 0) {
 #pragma unroll
