@@ -128,6 +128,12 @@ static Bat btc(const ot_plan* p) {
   b.n = p->batch;
   b.slab = p->slab;
   b.mask = b.on ? p->cur_mask : MASK_ALL;
+  // The Arnoldi step's close in the update while the class has at most 2048 update blocks (each
+  // finishes the multi-dot's sums, with FP64 scalars by one thread, which for hundreds of pairs
+  // costs more than the close in the multi-dot's last block).  Multi-dot + update at step 4, us,
+  // close in the multi-dot / in the update: 5 pairs of 128^2 7.7 + 3.8 / 3.6 + 4.7, 5 of 512^2
+  // 14.0 + 9.1 / 8.5 + 10.4, 16 of 512^2 (2048 blocks) 41.4 + 35.7 / 32.8 + 37.8.
+  b.split = b.on && (long)p->kblocks * p->batch <= 2048;
   return b;
 }
 
@@ -1969,6 +1975,10 @@ static int run_autotune(ot_plan* p) {
     if (cls == 1) tb.col_q = bestq;
     tsum += tbest;
   }
+  // row lengths with a factor 3: the only row pass whose transform the Arnoldi update can run
+  // is the pair form (row pass + update at 192^2 and 384^2: 7.3 + 4.3 us with the generic row
+  // pass, 6.9 and 6.5 us fused)
+  if ((M / 2) % 3 == 0 && update_pair_supported(N, M)) tb.var_r2c = VAR_PAIR;
   // the register-resident passes on the transposed spectrum replace all three at once:
   // kept when their summed time is below the per-pass choice's (two rounds, faster kept)
   if (tb.t2rA) {

@@ -66,13 +66,13 @@ __device__ __forceinline__ void finish_multidot(const double* partials, int nb,
 // count, and (in a graph) the conditional handle of the next step.  Every scalar it needs is
 // loaded first, as independent loads, so that the one thread that runs it waits for one
 // memory round trip instead of one per dependent access.
-// FAST (single problems): the rotation from one reciprocal square root, c = a / r = a rsqrt(r^2)
-// and s = b rsqrt(r^2), and the basis scale 1 / hn passed in (rsqrt of the Pythagorean
-// square), in place of a square root and divisions, whose FP64 forms are slow on this GPU
-// (the close is one thread on the step's critical path); a plan set's classes keep them.
-template <int J, bool FAST = false>
+// The rotation comes from one reciprocal square root, c = a / r = a rsqrt(r^2) and s = b
+// rsqrt(r^2), and the basis scale 1 / hn is passed in (rsqrt of the Pythagorean square), in place
+// of a square root and divisions, whose FP64 forms are slow on this GPU (the close is one thread
+// on the step's critical path).
+template <int J>
 __device__ void arnoldi_close_j(DevScalars* sc, const double (&h)[J], double hn, bool weak,
-                                double inv_hn = 0.0) {
+                                double inv_hn) {
   constexpr int j = J - 1;
   double cs[J], sn[J];
 #pragma unroll
@@ -94,18 +94,9 @@ __device__ void arnoldi_close_j(DevScalars* sc, const double (&h)[J], double hn,
     col[i + 1] = -sn[i] * t0 + cs[i] * t1;
   }
   const double a = col[j], b = col[j + 1];
-  double r, c, sj;
-  if (FAST) {
-    const double r2 = a * a + b * b;
-    const double y = r2 > 0.0 ? rsqrt(r2) : 0.0;
-    r = r2 * y;
-    c = (r2 > 0.0) ? a * y : 1.0;
-    sj = (r2 > 0.0) ? b * y : 0.0;
-  } else {
-    r = sqrt(a * a + b * b);
-    c = (r == 0.0) ? 1.0 : a / r;
-    sj = (r == 0.0) ? 0.0 : b / r;
-  }
+  const double r2 = a * a + b * b;
+  const double y = r2 > 0.0 ? rsqrt(r2) : 0.0;
+  const double r = r2 * y, c = (r2 > 0.0) ? a * y : 1.0, sj = (r2 > 0.0) ? b * y : 0.0;
   col[j] = r;
   col[j + 1] = 0.0;
 #pragma unroll
@@ -117,7 +108,6 @@ __device__ void arnoldi_close_j(DevScalars* sc, const double (&h)[J], double hn,
   sc->gv[j] = c * gvj;
   sc->iters = iters + 1;
   sc->jend = j + 1;
-  if (!FAST) sc->relres = fabs(g1) / bnorm;  // informational (the fast close skips it)
   int done = 0;
   if (weak) {
     done = 1;
@@ -125,7 +115,7 @@ __device__ void arnoldi_close_j(DevScalars* sc, const double (&h)[J], double hn,
     sc->converged = 1;
     done = 1;
   } else {
-    sc->scale[j + 1] = FAST ? inv_hn : 1.0 / hn;
+    sc->scale[j + 1] = inv_hn;
     if (j + 1 == m) done = 1;
   }
   if (done) sc->cycle_done = 1;

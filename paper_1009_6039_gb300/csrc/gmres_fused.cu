@@ -31,7 +31,7 @@ __device__ __forceinline__ void update_r2c_j(float* __restrict__ V, const float*
     if (threadIdx.x == 0) {
 #pragma unroll
       for (int i = 0; i < J; ++i) sc->hcol[i] = hv[i];
-      arnoldi_close_j<J, true>(sc, hv, hn, weak, inv_hn);
+      arnoldi_close_j<J>(sc, hv, hn, weak, inv_hn);
     }
     return;
   }
@@ -110,7 +110,7 @@ static int update_r2c_rows(int N, int M, int E) {
 }
 
 bool update_r2c_fits(int N, int M, int var_r2c) {
-  if (var_r2c == VAR_PAIR && comb_pair_supported(N, M)) return true;
+  if (var_r2c == VAR_PAIR && update_pair_supported(N, M)) return true;
   const int E = update_r2c_E(M, var_r2c);
   return E != 0 && update_r2c_rows(N, M, E) > 0;
 }
@@ -134,7 +134,7 @@ cudaError_t launch_gmres_update_r2c(float* V, const float* w, long P, const doub
                                     int nb, DevScalars* sc, float2* spec, int N, int M,
                                     const SpecTables& tb, cudaStream_t st) {
   // the row pair pass's fused form (the same transform and split as that pass)
-  if (tb.var_r2c == VAR_PAIR && comb_pair_supported(N, M))
+  if (tb.var_r2c == VAR_PAIR && update_pair_supported(N, M))
     return launch_gmres_update_r2c_pair(V, w, P, partials, nb, sc, spec, N, M, tb, st);
   switch (update_r2c_E(M, tb.var_r2c)) {
     case 4: return update_r2c_launch<4>(V, w, P, partials, nb, sc, spec, N, M, tb, st);

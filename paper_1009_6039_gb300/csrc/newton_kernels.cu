@@ -1112,7 +1112,8 @@ __device__ __forceinline__ void dots_j(const T* __restrict__ V, const T* __restr
       }
       const double ww = v[J], hn2 = ww - hs;
       const bool weak = !(hn2 > 1e-6 * ww);
-      arnoldi_close_j<J>(sc, h, weak ? 0.0 : sqrt(hn2), weak);
+      const double inv_hn = weak ? 0.0 : rsqrt(hn2);
+      arnoldi_close_j<J>(sc, h, hn2 * inv_hn, weak, inv_hn);
     } else if (pass == 0) {
 #pragma unroll
       for (int i = 0; i < J; ++i) sc->H[i * m + j] = sc->scale[i] * v[i];
@@ -1136,9 +1137,9 @@ __global__ void k_gmres_dots(const T* __restrict__ V, const T* __restrict__ w, l
   sc = badv(sc, bat);
   if (bskip(sc, bat) || sc->cycle_done) return;
   if (pass) w = V + (size_t)(sc->j + 1) * P;
-  // the split step (close in the update) serves single problems; a plan set's classes keep
-  // the close in the multi-dot's last block (measured faster for their small per-pair grids)
-  const bool split = !bat.on;
+  // the split step (close in the update) serves single problems and small classes of a plan
+  // set; large classes close in the multi-dot's last block
+  const bool split = !bat.on || bat.split;
   switch (sc->j) {
 #define OTGB_DOTS_CASE(k) \
   case k:                 \
@@ -1178,7 +1179,7 @@ __device__ __forceinline__ void update_j(T* __restrict__ V, const T* __restrict_
     if (threadIdx.x == 0) {
 #pragma unroll
       for (int i = 0; i < J; ++i) sc->hcol[i] = hv[i];
-      arnoldi_close_j<J, true>(sc, hv, hn, weak, inv_hn);
+      arnoldi_close_j<J>(sc, hv, hn, weak, inv_hn);
     }
     return;
   }
@@ -1212,7 +1213,7 @@ __device__ __forceinline__ void update_j(T* __restrict__ V, const T* __restrict_
     if (mode == 3 && split && !closer && blockIdx.x == 0 && threadIdx.x == 0) {
 #pragma unroll
       for (int i = 0; i < J; ++i) sc->hcol[i] = hv[i];
-      arnoldi_close_j<J, true>(sc, hv, hn, weak, inv_hn);
+      arnoldi_close_j<J>(sc, hv, hn, weak, inv_hn);
     }
     return;
   }
@@ -1241,10 +1242,10 @@ __global__ void k_gmres_update(T* __restrict__ V, const T* __restrict__ w, long 
   partials = badv(partials, bat);
   sc = badv(sc, bat);
   if (bskip(sc, bat) || sc->cycle_done) return;
-  // mode 3 follows the multi-dot of step jd (single problem: the update closes the step
-  // itself and advances sc->j, so it reads the step from jd; plan-set classes: the multi-dot
-  // closed it and advanced sc->j)
-  const bool split = !bat.on;
+  // mode 3 follows the multi-dot of step jd (split: the update closes the step itself and
+  // advances sc->j, so it reads the step from jd; else the multi-dot closed it and advanced
+  // sc->j)
+  const bool split = !bat.on || bat.split;
   switch (mode == 3 ? (split ? sc->jd : sc->j - 1) : sc->j) {
 #define OTGB_UPD_CASE(k) \
   case k:                \

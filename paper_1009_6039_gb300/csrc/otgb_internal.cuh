@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "dd.cuh"
 
 #define OTGB_MAXM 16  // largest GMRES restart length + 1 held on the device
@@ -106,12 +108,15 @@ struct Bat {
   int n = 1;
   size_t slab = 0;
   int mask = MASK_ALL;
+  int split = 0;  // Arnoldi step: the close in the update (as a single problem's), see btc()
 };
 template <typename T>
 __device__ __forceinline__ T* badv(T* p, const Bat& b) {
-  return (p && b.on)
-             ? reinterpret_cast<T*>(reinterpret_cast<uintptr_t>(p) + (size_t)blockIdx.z * b.slab)
-             : p;
+  // (pointer arithmetic, not a cast through an integer: the result stays based on the kernel's
+  // __restrict__ parameter)
+  using B = typename std::conditional<std::is_const<T>::value, const char, char>::type;
+  const size_t off = b.on ? (size_t)blockIdx.z * b.slab : 0;
+  return p ? reinterpret_cast<T*>(reinterpret_cast<B*>(p) + off) : p;
 }
 // the pair of this block does not take part in the launch (sc: this pair's scalars)
 __device__ __forceinline__ bool bskip(const DevScalars* sc, const Bat& b) {
@@ -199,33 +204,39 @@ struct SpecTables {
 };
 enum { VAR_DEFAULT = -1, VAR_GENERIC = 0, VAR_PAR = 1, VAR_WARP = 2, VAR_E4 = 3, VAR_PAIR = 4 };
 
-// the FP32 row combine pass on row pairs (M / 2 a power of two in 256..1024, N even)
+// Pair passes (two rows or columns side by side, packed FP32; pair.cuh): rows of M / 2 in 64, 96,
+// .. 1024 and N even, columns of N in 96, 128, .. 2048 and M a multiple of 4 (powers of two and
+// three times them).  A batched launch (bat) needs the pairs' scalars.
+// the FP32 row combine pass
 bool comb_pair_supported(int N, int M);
 cudaError_t launch_comb_pair(const float2* q0, const float2* q1, const float2* q2,
                              const float* coef, float* out, int N, int M, const SpecTables& tb,
-                             const int* skip, cudaStream_t st);
-// the FP32 row real-to-complex pass on row pairs, and the Arnoldi update fused with it
-// (the sizes of the combine pair pass)
+                             const int* skip, cudaStream_t st, const DevScalars* msc = nullptr,
+                             Bat bat = Bat());
+// the FP32 row real-to-complex pass, and the Arnoldi update fused with it (M / 2 >= 96)
 cudaError_t launch_row_r2c_pair(const float* x, size_t xs, const int* jptr, const double* scale,
                                 float2* spec, int N, int M, const SpecTables& tb,
-                                const int* skip, cudaStream_t st);
+                                const int* skip, cudaStream_t st,
+                                const DevScalars* msc = nullptr, Bat bat = Bat());
+bool update_pair_supported(int N, int M);
 cudaError_t launch_gmres_update_r2c_pair(float* V, const float* w, long P,
                                          const double* partials, int nb, DevScalars* sc,
                                          float2* spec, int N, int M, const SpecTables& tb,
                                          cudaStream_t st);
-// theta's double-float column pass (modes COL_LBARINV, COL_POISSON, COL_POISSON_LP) on
-// column pairs and its row pass + update on row pairs (the sizes of the FP32 pair passes)
+// theta's double-float column pass (modes COL_LBARINV, COL_POISSON, COL_POISSON_LP) and its row
+// pass + update
 cudaError_t launch_col_lbarinv_pair(const float2* spec, ddc* out, int N, int M,
                                     const SpecTables& tb32, const SpecTables& tbdd,
-                                    const DevScalars* sc, cudaStream_t st, int mode);
+                                    const DevScalars* sc, cudaStream_t st, int mode,
+                                    Bat bat = Bat());
 cudaError_t launch_row_update_pair(const ddc* q, const double* u_in, double* u_out,
                                    double step, int N, int M, const SpecTables& tbdd,
-                                   const DevScalars* sc, cudaStream_t st);
-// the FP32 column matvec pass on column pairs (power-of-two N in 256..2048, M % 4 == 0)
+                                   const DevScalars* sc, cudaStream_t st, Bat bat = Bat());
+// the FP32 column matvec pass
 bool col_pair_supported(int N, int M);
 cudaError_t launch_col_pair(const float2* spec, float2* o0, float2* o1, float2* o2, int N,
                             int M, const SpecTables& tb, const DevScalars* sc, const int* skip,
-                            cudaStream_t st);
+                            cudaStream_t st, Bat bat = Bat());
 
 bool fft_length_supported(int L);
 

@@ -33,7 +33,7 @@ __device__ __forceinline__ void r2c_pair_transform_split(PC* P0, PC* P1, float2*
                                                          float2* outb, int t,
                                                          const ulonglong2* __restrict__ tw4,
                                                          const float2* __restrict__ twM) {
-  constexpr int TPT = L / 4;
+  constexpr int TPT = pthreads<L>();
   {
     PC* const a[1] = {P0};
     PC* const b[1] = {P1};
@@ -79,13 +79,19 @@ constexpr size_t row_pair_smem() {
 
 // rows of x = xbase + (*jptr) x_stride (jptr NULL: xbase), times scale[*jptr] (NULL: 1)
 template <int L>
-__global__ void __launch_bounds__(L / 4)
+__global__ void __launch_bounds__(pthreads<L>())
     k_row_r2c_pair(const float* __restrict__ xbase, size_t x_stride, const int* __restrict__ jptr,
                    const double* __restrict__ scale, float2* __restrict__ spec,
                    const float2* __restrict__ twL, const float2* __restrict__ twM,
-                   const int* __restrict__ skip) {
-  if (skip && *skip) return;
-  constexpr int TPT = L / 4, M = 2 * L;
+                   const int* __restrict__ skip, const DevScalars* __restrict__ msc, Bat bat) {
+  xbase = badv(xbase, bat);
+  jptr = badv(jptr, bat);
+  scale = badv(scale, bat);
+  spec = badv(spec, bat);
+  skip = badv(skip, bat);
+  msc = badv(msc, bat);
+  if ((skip && *skip) || (bat.on && bskip(msc, bat))) return;
+  constexpr int TPT = pthreads<L>(), E = pelems<L>(), M = 2 * L;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ulonglong2* tw4 = reinterpret_cast<ulonglong2*>(smem_raw);
   PC* P0 = reinterpret_cast<PC*>(tw4 + L);
@@ -99,7 +105,7 @@ __global__ void __launch_bounds__(L / 4)
   const float2* xa = reinterpret_cast<const float2*>(x + (size_t)r0 * M);
   const float2* xb = xa + L;
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int n = t + e * TPT;
     const float2 za = xa[n], zb = xb[n];
     PC v;
@@ -120,7 +126,7 @@ __device__ __forceinline__ void update_r2c_pair_j(float* __restrict__ V,
                                                   const float2* __restrict__ twL,
                                                   const float2* __restrict__ twM) {
   constexpr int j = J - 1;
-  constexpr int TPT = L / 4, M = 2 * L;
+  constexpr int TPT = pthreads<L>(), E = pelems<L>(), M = 2 * L;
   double hv[J], hn = 0.0, inv_hn = 0.0;
   bool weak = false;
   float coefs[J];
@@ -129,7 +135,7 @@ __device__ __forceinline__ void update_r2c_pair_j(float* __restrict__ V,
     if (threadIdx.x == 0) {
 #pragma unroll
       for (int i = 0; i < J; ++i) sc->hcol[i] = hv[i];
-      arnoldi_close_j<J, true>(sc, hv, hn, weak, inv_hn);
+      arnoldi_close_j<J>(sc, hv, hn, weak, inv_hn);
     }
     return;
   }
@@ -143,7 +149,7 @@ __device__ __forceinline__ void update_r2c_pair_j(float* __restrict__ V,
   const bool next = J < sc->m;    // a next product (block-uniform)
   if (next) load_tw4<L>(tw4, twL, t, TPT);
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int n = t + e * TPT;
     float2 xr[2];
 #pragma unroll
@@ -173,7 +179,7 @@ __device__ __forceinline__ void update_r2c_pair_j(float* __restrict__ V,
 }
 
 template <int L>
-__global__ void __launch_bounds__(L / 4)
+__global__ void __launch_bounds__(pthreads<L>())
     k_gmres_update_r2c_pair(float* __restrict__ V, const float* __restrict__ w, long P,
                             const double* partials, int nb, DevScalars* sc,
                             float2* __restrict__ spec, const float2* __restrict__ twL,
@@ -194,12 +200,12 @@ __global__ void __launch_bounds__(L / 4)
 template <int L>
 cudaError_t row_r2c_pair_L(const float* x, size_t xs, const int* jptr, const double* scale,
                            float2* spec, int N, const SpecTables& tb, const int* skip,
-                           cudaStream_t st) {
+                           cudaStream_t st, const DevScalars* msc, Bat bat) {
   const size_t sm = row_pair_smem<L>();
-  cudaError_t e = prepare_launch(k_row_r2c_pair<L>, L / 4, sm);
+  cudaError_t e = prepare_launch(k_row_r2c_pair<L>, pthreads<L>(), sm);
   if (e != cudaSuccess) return e;
-  k_row_r2c_pair<L><<<N / 2, L / 4, sm, st>>>(x, xs, jptr, scale, spec, (const float2*)tb.twL,
-                                              (const float2*)tb.twM, skip);
+  k_row_r2c_pair<L><<<bgrid(dim3(N / 2), bat), pthreads<L>(), sm, st>>>(
+      x, xs, jptr, scale, spec, (const float2*)tb.twL, (const float2*)tb.twM, skip, msc, bat);
   return cudaGetLastError();
 }
 
@@ -207,25 +213,30 @@ template <int L>
 cudaError_t update_r2c_pair_L(float* V, const float* w, long P, const double* partials, int nb,
                               DevScalars* sc, float2* spec, int N, const SpecTables& tb,
                               cudaStream_t st) {
-  const size_t sm = row_pair_smem<L>();
-  cudaError_t e = prepare_launch(k_gmres_update_r2c_pair<L>, L / 4, sm);
-  if (e != cudaSuccess) return e;
-  k_gmres_update_r2c_pair<L><<<1 + N / 2, L / 4, sm, st>>>(
-      V, w, P, partials, nb, sc, spec, (const float2*)tb.twL, (const float2*)tb.twM);
-  return cudaGetLastError();
+  if constexpr (pthreads<L>() < 32) {  // the multi-dot's finish takes whole warps
+    return cudaErrorInvalidValue;
+  } else {
+    const size_t sm = row_pair_smem<L>();
+    cudaError_t e = prepare_launch(k_gmres_update_r2c_pair<L>, pthreads<L>(), sm);
+    if (e != cudaSuccess) return e;
+    k_gmres_update_r2c_pair<L><<<1 + N / 2, pthreads<L>(), sm, st>>>(
+        V, w, P, partials, nb, sc, spec, (const float2*)tb.twL, (const float2*)tb.twM);
+    return cudaGetLastError();
+  }
 }
 
 }  // namespace
 
+bool update_pair_supported(int N, int M) { return comb_pair_supported(N, M) && M / 2 >= 96; }
+
 cudaError_t launch_row_r2c_pair(const float* x, size_t xs, const int* jptr, const double* scale,
                                 float2* spec, int N, int M, const SpecTables& tb,
-                                const int* skip, cudaStream_t st) {
-  if (!comb_pair_supported(N, M)) return cudaErrorInvalidValue;
-  switch (M / 2) {
-    case 256: return row_r2c_pair_L<256>(x, xs, jptr, scale, spec, N, tb, skip, st);
-    case 512: return row_r2c_pair_L<512>(x, xs, jptr, scale, spec, N, tb, skip, st);
-    case 1024: return row_r2c_pair_L<1024>(x, xs, jptr, scale, spec, N, tb, skip, st);
-  }
+                                const int* skip, cudaStream_t st, const DevScalars* msc,
+                                Bat bat) {
+  if (!comb_pair_supported(N, M) || (bat.on && !msc)) return cudaErrorInvalidValue;
+#define OTGB_CALL(n) row_r2c_pair_L<n>(x, xs, jptr, scale, spec, N, tb, skip, st, msc, bat)
+  OTGB_ROW_LENGTHS(M / 2, OTGB_CALL)
+#undef OTGB_CALL
   return cudaErrorInvalidValue;
 }
 
@@ -233,12 +244,10 @@ cudaError_t launch_gmres_update_r2c_pair(float* V, const float* w, long P,
                                          const double* partials, int nb, DevScalars* sc,
                                          float2* spec, int N, int M, const SpecTables& tb,
                                          cudaStream_t st) {
-  if (!comb_pair_supported(N, M)) return cudaErrorInvalidValue;
-  switch (M / 2) {
-    case 256: return update_r2c_pair_L<256>(V, w, P, partials, nb, sc, spec, N, tb, st);
-    case 512: return update_r2c_pair_L<512>(V, w, P, partials, nb, sc, spec, N, tb, st);
-    case 1024: return update_r2c_pair_L<1024>(V, w, P, partials, nb, sc, spec, N, tb, st);
-  }
+  if (!update_pair_supported(N, M)) return cudaErrorInvalidValue;
+#define OTGB_CALL(n) update_r2c_pair_L<n>(V, w, P, partials, nb, sc, spec, N, tb, st)
+  OTGB_ROW_LENGTHS(M / 2, OTGB_CALL)
+#undef OTGB_CALL
   return cudaErrorInvalidValue;
 }
 

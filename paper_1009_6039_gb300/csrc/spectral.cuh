@@ -1900,13 +1900,19 @@ template <typename T>
 cudaError_t launch_row_r2c(const T* x, size_t xs, const int* jptr, const double* scale,
                            C2<T>* spec, int N, int M, const SpecTables& tb, const int* skip,
                            cudaStream_t st, Bat bat, const DevScalars* msc) {
-  if (bat.on) {  // batched: the generic kernels
+  if (bat.on) {  // batched: the pair pass, else the generic kernels
+    if constexpr (sizeof(T) == 4) {
+      if (msc && comb_pair_supported(N, M))
+        return launch_row_r2c_pair(reinterpret_cast<const float*>(x), xs, jptr, scale,
+                                   reinterpret_cast<float2*>(spec), N, M, tb, skip, st, msc, bat);
+    }
     if (fft_E(M / 2) == 12)
       return row_r2c_E<T, 12>(x, xs, jptr, scale, spec, N, M, tb, skip, st, bat, msc);
     return row_r2c_E<T, 8>(x, xs, jptr, scale, spec, N, M, tb, skip, st, bat, msc);
   }
   if constexpr (sizeof(T) == 4) {
-    if (tb.var_r2c == VAR_PAIR && !msc && comb_pair_supported(N, M))
+    // (where the fused update has the pair form too: the two agree bit for bit)
+    if (tb.var_r2c == VAR_PAIR && !msc && update_pair_supported(N, M))
       return launch_row_r2c_pair(reinterpret_cast<const float*>(x), xs, jptr, scale,
                                  reinterpret_cast<float2*>(spec), N, M, tb, skip, st);
   }
@@ -1981,8 +1987,14 @@ template <typename T>
 cudaError_t launch_col(int mode, const C2<T>* spec, C2<T>* o0, C2<T>* o1, C2<T>* o2, int N,
                        int M, const SpecTables& tb, const DevScalars* sc, const int* skip,
                        cudaStream_t st, Bat bat) {
-  if (bat.on) {  // batched: the generic kernels (the matvec mode only)
+  if (bat.on) {  // batched (the matvec mode only): the pair pass, else the generic kernels
     if (mode != COL_MATVEC) return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 4) {
+      if (sc && col_pair_supported(N, M))
+        return launch_col_pair(reinterpret_cast<const float2*>(spec),
+                               reinterpret_cast<float2*>(o0), reinterpret_cast<float2*>(o1),
+                               reinterpret_cast<float2*>(o2), N, M, tb, sc, skip, st, bat);
+    }
     if (fft_E(N) == 12)
       return col_E<T, 12, COL_MATVEC>(spec, o0, o1, o2, N, M, tb, sc, skip, st, bat);
     return col_E<T, 8, COL_MATVEC>(spec, o0, o1, o2, N, M, tb, sc, skip, st, bat);
@@ -2064,8 +2076,15 @@ cudaError_t launch_row_c2r(int mode, const C2<T>* q0, const C2<T>* q1, const C2<
                            const T* coef, T* out, const double* u_in, double* u_out,
                            double step, double os, int N, int M, const SpecTables& tb,
                            const int* skip, cudaStream_t st, const DevScalars* sc, Bat bat) {
-  if (bat.on) {  // batched: the generic kernels (the combine mode only)
+  if (bat.on) {  // batched (the combine mode only): the pair pass, else the generic kernels
     if (mode != ROWINV_COMBINE) return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 4) {
+      if (sc && comb_pair_supported(N, M))
+        return launch_comb_pair(
+            reinterpret_cast<const float2*>(q0), reinterpret_cast<const float2*>(q1),
+            reinterpret_cast<const float2*>(q2), reinterpret_cast<const float*>(coef),
+            reinterpret_cast<float*>(out), N, M, tb, skip, st, sc, bat);
+    }
     if (fft_E(M / 2) == 12)
       return row_c2r_E<T, 12, ROWINV_COMBINE>(q0, q1, q2, coef, out, u_in, u_out, step, os, N,
                                               M, tb, skip, st, sc, bat);

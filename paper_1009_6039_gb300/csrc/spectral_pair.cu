@@ -15,6 +15,8 @@
 // stage).  Shared memory is addressed through an XOR swizzle of the 16-byte element index,
 // i ^ ((i >> 2) & 7), under which every stage's reads and writes of a quarter warp fall in
 // distinct bank groups.  The symbol multiplies are the scalar operations of k_col.
+// (In place on three buffers -- 64 N instead of 112 N bytes, two barriers a stage -- measured the
+// same within 3 % for plan sets' classes and single grids of 512^2 to 2048^2.)
 #include "pair.cuh"
 
 namespace otgb {
@@ -23,14 +25,20 @@ namespace {
 using namespace pair;
 
 template <int N>
-__global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
+__global__ void __launch_bounds__(pthreads<N>(), N <= 1024 ? 2 : 1)
     k_col_pair(const float2* __restrict__ spec, float2* __restrict__ out0,
                float2* __restrict__ out1, float2* __restrict__ out2, int M, float inv,
                const float2* __restrict__ twN, const DevScalars* __restrict__ sc,
                const int* __restrict__ skip, const float2* __restrict__ symx,
-               const float2* __restrict__ symy) {
-  if (skip && *skip) return;
-  constexpr int TPT = N / 4;
+               const float2* __restrict__ symy, Bat bat) {
+  spec = badv(spec, bat);
+  out0 = badv(out0, bat);
+  out1 = badv(out1, bat);
+  out2 = badv(out2, bat);
+  sc = badv(sc, bat);
+  skip = badv(skip, bat);
+  if ((skip && *skip) || (bat.on && bskip(sc, bat))) return;
+  constexpr int TPT = pthreads<N>(), E = pelems<N>();
   constexpr bool ODD = pstage_count<N>() % 2 == 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ulonglong2* tw4 = reinterpret_cast<ulonglong2*>(smem_raw);
@@ -42,13 +50,13 @@ __global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
 
   // the column pair: one 16-byte load per row, issued before the twiddle table is built so
   // that both sets of loads are in flight together, then regrouped into (re, im) pairs
-  float4 xs[4];
+  float4 xs[E];
 #pragma unroll
-  for (int e = 0; e < 4; ++e)
+  for (int e = 0; e < E; ++e)
     xs[e] = *reinterpret_cast<const float4*>(spec + (size_t)(t + e * TPT) * Lc + c0);
   load_tw4<N>(tw4, twN, t, TPT);
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     PC v;
     v.re = pk(xs[e].x, xs[e].z);
     v.im = pk(xs[e].y, xs[e].w);
@@ -73,7 +81,7 @@ __global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
   for (int q = 0; q < 5; ++q) ab[q] = sc ? (float)sc->abar[q] : 0.f;
   const float2 sxa = symx[c0], sxb = symx[c0 + 1];
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int k = t + e * TPT;
     const PC z = F[swz(k)];
     float2 za, zb;
@@ -122,7 +130,7 @@ __global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
 #pragma unroll
   for (int o = 0; o < 3; ++o) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
+    for (int e = 0; e < E; ++e) {
       const int n = t + e * TPT;
       const PC v = res[o][swz(n)];
       float4 x;
@@ -143,14 +151,21 @@ __global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
 // the N / 2 blocks of a 1024 x 1024 grid run in one wave.
 // ---------------------------------------------------------------------------------------
 template <int L>
-__global__ void __launch_bounds__(L / 4, L <= 512 ? 4 : 2)
+__global__ void __launch_bounds__(pthreads<L>(), L <= 512 ? 4 : 2)
     k_comb_pair(const float2* __restrict__ q0, const float2* __restrict__ q1,
                 const float2* __restrict__ q2, const float* __restrict__ coef,
                 float* __restrict__ out, int N, const float2* __restrict__ twL,
                 const float2* __restrict__ twM, const int* __restrict__ skip,
-                const float2* __restrict__ symx) {
-  if (skip && *skip) return;
-  constexpr int TPT = L / 4;
+                const float2* __restrict__ symx, const DevScalars* __restrict__ msc, Bat bat) {
+  q0 = badv(q0, bat);
+  q1 = badv(q1, bat);
+  q2 = badv(q2, bat);
+  coef = badv(coef, bat);
+  out = badv(out, bat);
+  skip = badv(skip, bat);
+  msc = badv(msc, bat);
+  if ((skip && *skip) || (bat.on && bskip(msc, bat))) return;
+  constexpr int TPT = pthreads<L>(), E = pelems<L>();
   constexpr int M = 2 * L;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ulonglong2* tw4 = reinterpret_cast<ulonglong2*>(smem_raw);
@@ -163,9 +178,9 @@ __global__ void __launch_bounds__(L / 4, L <= 512 ? 4 : 2)
   // which Q0 carries premultiplied); the rows' loads are issued before the twiddle table is
   // built, so that both sets of loads are in flight together
   const size_t oa = (size_t)r0 * L, ob = oa + L;
-  float2 ld[4][6];
+  float2 ld[E][6];
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int k = t + e * TPT;
     ld[e][0] = q0[oa + k];
     ld[e][1] = q0[ob + k];
@@ -176,7 +191,7 @@ __global__ void __launch_bounds__(L / 4, L <= 512 ? 4 : 2)
   }
   load_tw4<L>(tw4, twL, t, TPT);
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int k = t + e * TPT;
     const float2 a0 = ld[e][0], b0 = ld[e][1];
     const float2 a1 = ld[e][2], b1 = ld[e][3];
@@ -232,20 +247,20 @@ __global__ void __launch_bounds__(L / 4, L <= 512 ? 4 : 2)
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
         const PC xk = B[q][dk], xm = B[q][dm];
-        PC E, D;
-        E.re = add2(xk.re, xm.re);
-        E.im = sub2(xk.im, xm.im);
+        PC S, D;
+        S.re = add2(xk.re, xm.re);
+        S.im = sub2(xk.im, xm.im);
         D.re = sub2(xk.re, xm.re);
         D.im = add2(xk.im, xm.im);
         const PC O = cmulp<+1>(D, wx, wy, nwy);
         PC zk;
-        zk.re = sub2(E.re, O.im);
-        zk.im = add2(E.im, O.re);
+        zk.re = sub2(S.re, O.im);
+        zk.im = add2(S.im, O.re);
         B[q][dk] = zk;
         if (2 * k != L) {
           PC zm;
-          zm.re = add2(E.re, O.im);
-          zm.im = sub2(O.re, E.im);
+          zm.re = add2(S.re, O.im);
+          zm.im = sub2(O.re, S.im);
           B[q][dm] = zm;
         }
       }
@@ -266,7 +281,7 @@ __global__ void __launch_bounds__(L / 4, L <= 512 ? 4 : 2)
   float2* ov = reinterpret_cast<float2*>(out);
   const u64 two = pk(2.f, 2.f);
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int n = t + e * TPT;
     const int d = swz(n);
     const size_t ia = ra / 2 + n, ib = rb / 2 + n;
@@ -295,26 +310,26 @@ __global__ void __launch_bounds__(L / 4, L <= 512 ? 4 : 2)
 template <int L>
 cudaError_t comb_pair_L(const float2* q0, const float2* q1, const float2* q2, const float* coef,
                         float* out, int N, const SpecTables& tb, const int* skip,
-                        cudaStream_t st) {
+                        cudaStream_t st, const DevScalars* msc, Bat bat) {
   const size_t sm = (size_t)L * sizeof(ulonglong2) + 5 * (size_t)L * sizeof(PC);
-  cudaError_t e = prepare_launch(k_comb_pair<L>, L / 4, sm);
+  cudaError_t e = prepare_launch(k_comb_pair<L>, pthreads<L>(), sm);
   if (e != cudaSuccess) return e;
-  k_comb_pair<L><<<N / 2, L / 4, sm, st>>>(q0, q1, q2, coef, out, N, (const float2*)tb.twL,
-                                           (const float2*)tb.twM, skip,
-                                           (const float2*)tb.symx);
+  k_comb_pair<L><<<bgrid(dim3(N / 2), bat), pthreads<L>(), sm, st>>>(
+      q0, q1, q2, coef, out, N, (const float2*)tb.twL, (const float2*)tb.twM, skip,
+      (const float2*)tb.symx, msc, bat);
   return cudaGetLastError();
 }
 
 template <int N>
 cudaError_t col_pair_N(const float2* spec, float2* o0, float2* o1, float2* o2, int M,
                        const SpecTables& tb, const DevScalars* sc, const int* skip,
-                       cudaStream_t st) {
+                       cudaStream_t st, Bat bat) {
   const size_t sm = (size_t)N * sizeof(ulonglong2) + 6 * (size_t)N * sizeof(PC);
-  cudaError_t e = prepare_launch(k_col_pair<N>, N / 4, sm);
+  cudaError_t e = prepare_launch(k_col_pair<N>, pthreads<N>(), sm);
   if (e != cudaSuccess) return e;
-  k_col_pair<N><<<M / 4, N / 4, sm, st>>>(
+  k_col_pair<N><<<bgrid(dim3(M / 4), bat), pthreads<N>(), sm, st>>>(
       spec, o0, o1, o2, M, (float)(1.0 / ((double)N * (double)M)), (const float2*)tb.twN, sc,
-      skip, (const float2*)tb.symx, (const float2*)tb.symy);
+      skip, (const float2*)tb.symx, (const float2*)tb.symy, bat);
   return cudaGetLastError();
 }
 
@@ -322,38 +337,31 @@ cudaError_t col_pair_N(const float2* spec, float2* o0, float2* o1, float2* o2, i
 
 bool comb_pair_supported(int N, int M) {
   const int L = M / 2;
-  return (L == 256 || L == 512 || L == 1024) && M == 2 * L && N >= 2 && N % 2 == 0;
+  return row_pair_length(L) && M == 2 * L && N >= 2 && N % 2 == 0;
 }
 
 cudaError_t launch_comb_pair(const float2* q0, const float2* q1, const float2* q2,
                              const float* coef, float* out, int N, int M, const SpecTables& tb,
-                             const int* skip, cudaStream_t st) {
-  if (!comb_pair_supported(N, M)) return cudaErrorInvalidValue;
-  switch (M / 2) {
-    case 256: return comb_pair_L<256>(q0, q1, q2, coef, out, N, tb, skip, st);
-    case 512: return comb_pair_L<512>(q0, q1, q2, coef, out, N, tb, skip, st);
-    case 1024: return comb_pair_L<1024>(q0, q1, q2, coef, out, N, tb, skip, st);
-  }
+                             const int* skip, cudaStream_t st, const DevScalars* msc, Bat bat) {
+  if (!comb_pair_supported(N, M) || (bat.on && !msc)) return cudaErrorInvalidValue;
+#define OTGB_CALL(n) comb_pair_L<n>(q0, q1, q2, coef, out, N, tb, skip, st, msc, bat)
+  OTGB_ROW_LENGTHS(M / 2, OTGB_CALL)
+#undef OTGB_CALL
   return cudaErrorInvalidValue;
 }
 
-bool col_pair_supported(int N, int M) {
-  return (N == 256 || N == 512 || N == 1024 || N == 2048) && M >= 4 && M % 4 == 0;
-}
+bool col_pair_supported(int N, int M) { return col_pair_length(N) && M >= 4 && M % 4 == 0; }
 
 cudaError_t launch_col_pair(const float2* spec, float2* o0, float2* o1, float2* o2, int N,
                             int M, const SpecTables& tb, const DevScalars* sc, const int* skip,
-                            cudaStream_t st) {
-  if (!col_pair_supported(N, M)) return cudaErrorInvalidValue;
+                            cudaStream_t st, Bat bat) {
+  if (!col_pair_supported(N, M) || (bat.on && !sc)) return cudaErrorInvalidValue;
   // 16-byte loads and stores of a column pair need 16-byte aligned planes
-  if (((uintptr_t)spec | (uintptr_t)o0 | (uintptr_t)o1 | (uintptr_t)o2) & 15)
+  if (((uintptr_t)spec | (uintptr_t)o0 | (uintptr_t)o1 | (uintptr_t)o2 | bat.slab) & 15)
     return cudaErrorMisalignedAddress;
-  switch (N) {
-    case 256: return col_pair_N<256>(spec, o0, o1, o2, M, tb, sc, skip, st);
-    case 512: return col_pair_N<512>(spec, o0, o1, o2, M, tb, sc, skip, st);
-    case 1024: return col_pair_N<1024>(spec, o0, o1, o2, M, tb, sc, skip, st);
-    case 2048: return col_pair_N<2048>(spec, o0, o1, o2, M, tb, sc, skip, st);
-  }
+#define OTGB_CALL(n) col_pair_N<n>(spec, o0, o1, o2, M, tb, sc, skip, st, bat)
+  OTGB_COL_LENGTHS(N, OTGB_CALL)
+#undef OTGB_CALL
   return cudaErrorInvalidValue;
 }
 

@@ -48,6 +48,20 @@ template <int SIGN> struct BflyDC<2, SIGN> {
     v[1] = dc_sub(a, b);
   }
 };
+template <int SIGN> struct BflyDC<3, SIGN> {  // the scalar butterfly's operations
+  __device__ __forceinline__ static void run(DC* v) {
+    const DC a = v[0], s = dc_add(v[1], v[2]), d = dc_sub(v[1], v[2]);
+    const D2 half{pk(0.5f, 0.5f), 0ull};
+    const dd c = dd(OTGB_SQRT3_HALF);
+    const D2 cc{pk(c.hi, c.hi), pk(c.lo, c.lo)};
+    const DC t{d2_sub(a.re, d2_mul(half, s.re)), d2_sub(a.im, d2_mul(half, s.im))};
+    const DC e = dc_mul_si<SIGN>(d);
+    const DC u{d2_mul(e.re, cc), d2_mul(e.im, cc)};
+    v[0] = dc_add(a, s);
+    v[1] = dc_add(t, u);
+    v[2] = dc_sub(t, u);
+  }
+};
 template <int SIGN> struct BflyDC<4, SIGN> {
   __device__ __forceinline__ static void run(DC* v) {
     const DC t0 = dc_add(v[0], v[2]), t1 = dc_sub(v[0], v[2]);
@@ -83,12 +97,12 @@ __device__ __forceinline__ void dc_to(DC v, ddc& a, ddc& b) {
   upk(v.im.l, a.y.lo, b.y.lo);
 }
 
-// the stage twiddles of the 4-element double-float transforms of length L, broadcast to both
+// the stage twiddles of the double-float transforms of length L, broadcast to both
 // lanes: high words (x, y) in th, low words in tl
 template <int L>
 __device__ __forceinline__ void load_twdd(ulonglong2* th, ulonglong2* tl,
                                           const ddc* __restrict__ twb, int t, int nthreads) {
-  const ddc* __restrict__ st = twb + (size_t)stage_table_slot<4>() * L;
+  const ddc* __restrict__ st = pstage_table<L>(twb);
   for (int i = t; i < L; i += nthreads) {
     const ddc w = st[i];
     th[i] = make_ulonglong2(pk(w.x.hi, w.x.hi), pk(w.y.hi, w.y.hi));
@@ -96,42 +110,47 @@ __device__ __forceinline__ void load_twdd(ulonglong2* th, ulonglong2* tl,
   }
 }
 
-// one double-float stage of radix R (span Ns), 4 elements per thread, in -> out (in place:
-// the stores wait for every thread's loads)
+// one double-float stage of radix R (span Ns), in -> out (in place: the stores wait for every
+// thread's loads); the threads as in pstage
 template <int R, int SIGN, int L, int Ns, bool INPLACE>
 __device__ __forceinline__ void dstage(DBuf in, DBuf out, int t,
                                        const ulonglong2* __restrict__ th,
                                        const ulonglong2* __restrict__ tl) {
-  constexpr int E = 4, TPT = L / E, LR = L / R;
-  constexpr int a = Ns == 1 ? 0 : __builtin_ctz(Ns);
-  DC v[E];
+  constexpr int NB = R == 3 ? 1 : 4 / R;
+  constexpr int T = R == 3 ? L / 3 : L / 4, LR = L / R;
+  const bool active = L % 3 != 0 || R == 3 || t < T;
+  DC v[NB * R];
+  if (active) {
 #pragma unroll
-  for (int b = 0; b < E / R; ++b) {
-    const int j = t + b * TPT;
+    for (int b = 0; b < NB; ++b) {
+      const int j = t + b * T;
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[b * R + r] = dld(in, swz(j + r * LR));
+      for (int r = 0; r < R; ++r) v[b * R + r] = dld(in, swz(j + r * LR));
+    }
   }
   if (INPLACE) __syncthreads();
+  if (active) {
 #pragma unroll
-  for (int b = 0; b < E / R; ++b) {
-    const int j = t + b * TPT;
-    const int qd = j >> a;
-    const int k = j & (Ns - 1);
-    if (Ns > 1) {
+    for (int b = 0; b < NB; ++b) {
+      const int j = t + b * T;
+      const int qd = (int)((unsigned)j / (unsigned)Ns);
+      const int k = j - qd * Ns;
+      if (Ns > 1) {
 #pragma unroll
-      for (int r = 1; r < R; ++r) {
-        const int ti = (Ns - 1) + (r - 1) * Ns + k;
-        const ulonglong2 wh = th[ti], wl = tl[ti];
-        const D2 wx{wh.x, wl.x};
-        D2 wy{wh.y, wl.y};
-        if (SIGN > 0) wy = d2_neg(wy);
-        v[b * R + r] = dc_mul(v[b * R + r], wx, wy);
+        for (int r = 1; r < R; ++r) {
+          const int ti = (Ns - 1) + (r - 1) * Ns + k;
+          const ulonglong2 wh = th[ti], wl = tl[ti];
+          const D2 wx{wh.x, wl.x};
+          D2 wy{wh.y, wl.y};
+          if (SIGN > 0) wy = d2_neg(wy);
+          v[b * R + r] = dc_mul(v[b * R + r], wx, wy);
+        }
       }
-    }
-    BflyDC<R, SIGN>::run(&v[b * R]);
-    const int d = qd * (Ns * R) + k;
+      BflyDC<R, SIGN>::run(&v[b * R]);
+      const int d = qd * (Ns * R) + k;
 #pragma unroll
-    for (int r = 0; r < R; ++r) dst(out, swz(d + r * Ns), v[b * R + r]);
+      for (int r = 0; r < R; ++r) dst(out, swz(d + r * Ns), v[b * R + r]);
+    }
   }
   __syncthreads();
 }
@@ -142,7 +161,7 @@ template <int SIGN, int L, int Ns, int REM, bool INPLACE, bool FROM_A>
 __device__ __forceinline__ void dfft(DBuf a, DBuf b, int t, const ulonglong2* __restrict__ th,
                                      const ulonglong2* __restrict__ tl) {
   if constexpr (REM > 1) {
-    constexpr int R = REM % 4 == 0 ? 4 : 2;
+    constexpr int R = pradix<REM>();
     if constexpr (INPLACE)
       dstage<R, SIGN, L, Ns, true>(a, a, t, th, tl);
     else if constexpr (FROM_A)
@@ -153,28 +172,28 @@ __device__ __forceinline__ void dfft(DBuf a, DBuf b, int t, const ulonglong2* __
   }
 }
 
-template <int REM>
-__host__ __device__ constexpr int dstage_count() {
-  if constexpr (REM > 1)
-    return 1 + dstage_count<REM / (REM % 4 == 0 ? 4 : 2)>();
-  else
-    return 0;
+__device__ __forceinline__ float lowpass_of(int mode, int k1, int k2, int M, int N) {
+  return mode == COL_POISSON_LP ? lowpass_f<COL_POISSON_LP>(k1, k2, M, N) : 1.f;
 }
 
-// theta's column pass (MODE COL_LBARINV: S = rho-bar(abar_n) sigma-hat / (N M)) or the
-// Poisson solves' (COL_POISSON, COL_POISSON_LP: division by the 4th-order FD Laplacian's
+// theta's column pass (mode COL_LBARINV: S = rho-bar(abar_n) sigma-hat / (N M)) or, POISSON, the
+// Poisson solves' (modes COL_POISSON, COL_POISSON_LP: division by the 4th-order FD Laplacian's
 // eigenvalues, zero mode -> 0, _LP with the Gaussian low-pass) on column pairs: the FP32
 // forward column transform, the scalar symbol step of k_col_lbarinv_dd per column, the
 // double-float inverse column transform (out of place), ddc output
-template <int N, int MODE>
-__global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
-    k_col_lbarinv_pair(const float2* __restrict__ spec, ddc* __restrict__ out, int M,
+template <int N, bool POISSON>
+__global__ void __launch_bounds__(pthreads<N>(), N <= 1024 ? 2 : 1)
+    k_col_lbarinv_pair(const float2* __restrict__ spec, ddc* __restrict__ out, int M, int mode,
                        float inv, const float2* __restrict__ twN32,
                        const float2* __restrict__ twM32, const ddc* __restrict__ twNdd,
                        const DevScalars* __restrict__ sc, const float2* __restrict__ symx,
-                       const float2* __restrict__ symy) {
-  constexpr int TPT = N / 4;
-  constexpr bool FODD = dstage_count<N>() % 2 == 1;
+                       const float2* __restrict__ symy, Bat bat) {
+  spec = badv(spec, bat);
+  out = badv(out, bat);
+  sc = badv(sc, bat);
+  if (bat.on && bskip(sc, bat)) return;
+  constexpr int TPT = pthreads<N>(), E = pelems<N>();
+  constexpr bool FODD = pstage_count<N>() % 2 == 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ulonglong2* tw4 = reinterpret_cast<ulonglong2*>(smem_raw);
   ulonglong2* th = tw4 + N;
@@ -188,14 +207,14 @@ __global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
   const int c0 = 2 * blockIdx.x;
   const int t = threadIdx.x;
   // the column pair's loads first, so that they are in flight with the twiddle tables' loads
-  float4 xs[4];
+  float4 xs[E];
 #pragma unroll
-  for (int e = 0; e < 4; ++e)
+  for (int e = 0; e < E; ++e)
     xs[e] = *reinterpret_cast<const float4*>(spec + (size_t)(t + e * TPT) * Lc + c0);
   load_tw4<N>(tw4, twN32, t, TPT);
   load_twdd<N>(th, tl, twNdd, t, TPT);
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     PC v;
     v.re = pk(xs[e].x, xs[e].z);
     v.im = pk(xs[e].y, xs[e].w);
@@ -211,9 +230,9 @@ __global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
 
   float ab[5];
 #pragma unroll
-  for (int q = 0; q < 5; ++q) ab[q] = MODE == COL_LBARINV ? (float)sc->abar_n[q] : 0.f;
+  for (int q = 0; q < 5; ++q) ab[q] = !POISSON ? (float)sc->abar_n[q] : 0.f;
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int k = t + e * TPT;
     const PC z2 = F[swz(k)];
     float2 zc[2];
@@ -232,7 +251,7 @@ __global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
         upk(p2.im, pz.y, pother.y);
         float2 Av = mk2<float>(0.5f * (z.x + pz.x), 0.5f * (z.y - pz.y));
         float2 Bv = mk2<float>(0.5f * (z.y + pz.y), -0.5f * (z.x - pz.x));
-        if (MODE == COL_LBARINV) {
+        if (!POISSON) {
           Av = cmul<float>(rho_bar<float>(ab, symx[0], symy[k]), Av);
           Bv = cmul<float>(rho_bar<float>(ab, symx[M / 2], symy[k]), Bv);
         } else {
@@ -240,19 +259,19 @@ __global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
           const int k2 = sfreq(k, N, &nyq2);
           const float ly = fd_lap_w(twN32[k], N);
           const float lxn = -16.f / 3.f * (float)M * (float)M;  // k1 = M/2 (cos t = -1)
-          Av = cscale<float>(Av, inv_or_zero<float>(ly) * lowpass_f<MODE>(0, k2, M, N));
+          Av = cscale<float>(Av, inv_or_zero<float>(ly) * lowpass_of(mode, 0, k2, M, N));
           Bv = cscale<float>(Bv,
-                             inv_or_zero<float>(lxn + ly) * lowpass_f<MODE>(M / 2, k2, M, N));
+                             inv_or_zero<float>(lxn + ly) * lowpass_of(mode, M / 2, k2, M, N));
         }
         r = mk2<float>(Av.x - Bv.y, Av.y + Bv.x);
-      } else if (MODE == COL_LBARINV) {
+      } else if (!POISSON) {
         r = cmul<float>(rho_bar<float>(ab, symx[col], symy[k]), z);
       } else {
         bool nyq2;
         const int k2 = sfreq(k, N, &nyq2);
         r = cscale<float>(z, inv_or_zero<float>(fd_lap_w(twM32[col], M) +
                                                 fd_lap_w(twN32[k], N)) *
-                                 lowpass_f<MODE>(col, k2, M, N));
+                                 lowpass_of(mode, col, k2, M, N));
       }
       s[h] = mk2<float>(r.x * inv, r.y * inv);
     }
@@ -266,7 +285,7 @@ __global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
   dfft<+1, N, 1, N, false, true>(B, A, t, th, tl);
   const DBuf res = FODD ? A : B;
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int n = t + e * TPT;
     ddc a, b;
     dc_to(dld(res, swz(n)), a, b);
@@ -280,11 +299,16 @@ __global__ void __launch_bounds__(N / 4, N <= 1024 ? 2 : 1)
 // in FP64 (u_in == nullptr: u_out = step theta; with sc the step and the current / candidate
 // buffers come from the device scalars, as in k_row_c2r_update_dd); in-place stages
 template <int L>
-__global__ void __launch_bounds__(L / 4, L <= 512 ? 4 : 2)
+__global__ void __launch_bounds__(pthreads<L>(), L <= 512 ? 4 : 2)
     k_row_update_pair(const ddc* __restrict__ q, const double* __restrict__ u_in,
                       double* __restrict__ u_out, double step, int N,
                       const ddc* __restrict__ twL, const ddc* __restrict__ twM,
-                      const DevScalars* __restrict__ sc) {
+                      const DevScalars* __restrict__ sc, Bat bat) {
+  q = badv(q, bat);
+  u_in = badv(u_in, bat);
+  u_out = badv(u_out, bat);
+  sc = badv(sc, bat);
+  if (bat.on && bskip(sc, bat)) return;
   if (sc) {
     step = sc->step_s;
     if (sc->upar & 1) {
@@ -293,7 +317,7 @@ __global__ void __launch_bounds__(L / 4, L <= 512 ? 4 : 2)
       u_out = tmp;
     }
   }
-  constexpr int TPT = L / 4;
+  constexpr int TPT = pthreads<L>(), E = pelems<L>();
   constexpr int M = 2 * L;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ulonglong2* th = reinterpret_cast<ulonglong2*>(smem_raw);
@@ -304,15 +328,15 @@ __global__ void __launch_bounds__(L / 4, L <= 512 ? 4 : 2)
   // the rows' loads first, so that they are in flight with the twiddle table's loads
   const ddc* qa = q + (size_t)r0 * L;
   const ddc* qb = qa + L;
-  ddc ra[4], rb[4];
+  ddc ra[E], rb[E];
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     ra[e] = qa[t + e * TPT];
     rb[e] = qb[t + e * TPT];
   }
   load_twdd<L>(th, tl, twL, t, TPT);
 #pragma unroll
-  for (int e = 0; e < 4; ++e) dst(A, swz(t + e * TPT), dc_from(ra[e], rb[e]));
+  for (int e = 0; e < E; ++e) dst(A, swz(t + e * TPT), dc_from(ra[e], rb[e]));
   __syncthreads();
   // complex-to-real pre-processing (as c2r_preprocess on dd): each pair (k, L - k) by one
   // thread
@@ -342,7 +366,7 @@ __global__ void __launch_bounds__(L / 4, L <= 512 ? 4 : 2)
   double2* uoa = reinterpret_cast<double2*>(u_out + (size_t)r0 * M);
   double2* uob = uoa + L;
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int n = t + e * TPT;
     ddc za, zb;
     dc_to(dld(A, swz(n)), za, zb);
@@ -357,41 +381,38 @@ __global__ void __launch_bounds__(L / 4, L <= 512 ? 4 : 2)
   }
 }
 
-template <int N, int MODE>
-cudaError_t col_lbarinv_pair_N(const float2* spec, ddc* out, int M, const SpecTables& tb32,
-                               const SpecTables& tbdd, const DevScalars* sc, cudaStream_t st) {
+template <int N, bool POISSON>
+cudaError_t col_lbarinv_pair_launch(const float2* spec, ddc* out, int M, const SpecTables& tb32,
+                               const SpecTables& tbdd, const DevScalars* sc, cudaStream_t st,
+                               int mode, Bat bat) {
   const size_t sm = 7 * (size_t)N * sizeof(ulonglong2);
-  cudaError_t e = prepare_launch(k_col_lbarinv_pair<N, MODE>, N / 4, sm);
+  cudaError_t e = prepare_launch(k_col_lbarinv_pair<N, POISSON>, pthreads<N>(), sm);
   if (e != cudaSuccess) return e;
-  k_col_lbarinv_pair<N, MODE><<<M / 4, N / 4, sm, st>>>(
-      spec, out, M, (float)(1.0 / ((double)N * (double)M)), (const float2*)tb32.twN,
+  k_col_lbarinv_pair<N, POISSON><<<bgrid(dim3(M / 4), bat), pthreads<N>(), sm, st>>>(
+      spec, out, M, mode, (float)(1.0 / ((double)N * (double)M)), (const float2*)tb32.twN,
       (const float2*)tb32.twM, (const ddc*)tbdd.twN, sc, (const float2*)tb32.symx,
-      (const float2*)tb32.symy);
+      (const float2*)tb32.symy, bat);
   return cudaGetLastError();
 }
 
-template <int MODE>
-cudaError_t col_lbarinv_pair_mode(const float2* spec, ddc* out, int N, int M,
-                                  const SpecTables& tb32, const SpecTables& tbdd,
-                                  const DevScalars* sc, cudaStream_t st) {
-  switch (N) {
-    case 256: return col_lbarinv_pair_N<256, MODE>(spec, out, M, tb32, tbdd, sc, st);
-    case 512: return col_lbarinv_pair_N<512, MODE>(spec, out, M, tb32, tbdd, sc, st);
-    case 1024: return col_lbarinv_pair_N<1024, MODE>(spec, out, M, tb32, tbdd, sc, st);
-    case 2048: return col_lbarinv_pair_N<2048, MODE>(spec, out, M, tb32, tbdd, sc, st);
-  }
-  return cudaErrorInvalidValue;
+template <int N>
+cudaError_t col_lbarinv_pair_N(const float2* spec, ddc* out, int M, const SpecTables& tb32,
+                               const SpecTables& tbdd, const DevScalars* sc, cudaStream_t st,
+                               int mode, Bat bat) {
+  if (mode == COL_LBARINV)
+    return col_lbarinv_pair_launch<N, false>(spec, out, M, tb32, tbdd, sc, st, mode, bat);
+  return col_lbarinv_pair_launch<N, true>(spec, out, M, tb32, tbdd, sc, st, mode, bat);
 }
 
 template <int L>
 cudaError_t row_update_pair_L(const ddc* q, const double* u_in, double* u_out, double step,
                               int N, const SpecTables& tbdd, const DevScalars* sc,
-                              cudaStream_t st) {
+                              cudaStream_t st, Bat bat) {
   const size_t sm = 4 * (size_t)L * sizeof(ulonglong2);
-  cudaError_t e = prepare_launch(k_row_update_pair<L>, L / 4, sm);
+  cudaError_t e = prepare_launch(k_row_update_pair<L>, pthreads<L>(), sm);
   if (e != cudaSuccess) return e;
-  k_row_update_pair<L><<<N / 2, L / 4, sm, st>>>(q, u_in, u_out, step, N, (const ddc*)tbdd.twL,
-                                                 (const ddc*)tbdd.twM, sc);
+  k_row_update_pair<L><<<bgrid(dim3(N / 2), bat), pthreads<L>(), sm, st>>>(
+      q, u_in, u_out, step, N, (const ddc*)tbdd.twL, (const ddc*)tbdd.twM, sc, bat);
   return cudaGetLastError();
 }
 
@@ -399,30 +420,25 @@ cudaError_t row_update_pair_L(const ddc* q, const double* u_in, double* u_out, d
 
 cudaError_t launch_col_lbarinv_pair(const float2* spec, ddc* out, int N, int M,
                                     const SpecTables& tb32, const SpecTables& tbdd,
-                                    const DevScalars* sc, cudaStream_t st, int mode) {
+                                    const DevScalars* sc, cudaStream_t st, int mode, Bat bat) {
   if (!col_pair_supported(N, M)) return cudaErrorInvalidValue;
-  if ((uintptr_t)spec & 15) return cudaErrorMisalignedAddress;
-  switch (mode) {
-    case COL_LBARINV:
-      if (!sc) return cudaErrorInvalidValue;
-      return col_lbarinv_pair_mode<COL_LBARINV>(spec, out, N, M, tb32, tbdd, sc, st);
-    case COL_POISSON:
-      return col_lbarinv_pair_mode<COL_POISSON>(spec, out, N, M, tb32, tbdd, sc, st);
-    case COL_POISSON_LP:
-      return col_lbarinv_pair_mode<COL_POISSON_LP>(spec, out, N, M, tb32, tbdd, sc, st);
-  }
+  if (mode != COL_LBARINV && mode != COL_POISSON && mode != COL_POISSON_LP)
+    return cudaErrorInvalidValue;
+  if ((mode == COL_LBARINV || bat.on) && !sc) return cudaErrorInvalidValue;
+  if (((uintptr_t)spec | bat.slab) & 15) return cudaErrorMisalignedAddress;
+#define OTGB_CALL(n) col_lbarinv_pair_N<n>(spec, out, M, tb32, tbdd, sc, st, mode, bat)
+  OTGB_COL_LENGTHS(N, OTGB_CALL)
+#undef OTGB_CALL
   return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_row_update_pair(const ddc* q, const double* u_in, double* u_out,
                                    double step, int N, int M, const SpecTables& tbdd,
-                                   const DevScalars* sc, cudaStream_t st) {
-  if (!comb_pair_supported(N, M)) return cudaErrorInvalidValue;
-  switch (M / 2) {
-    case 256: return row_update_pair_L<256>(q, u_in, u_out, step, N, tbdd, sc, st);
-    case 512: return row_update_pair_L<512>(q, u_in, u_out, step, N, tbdd, sc, st);
-    case 1024: return row_update_pair_L<1024>(q, u_in, u_out, step, N, tbdd, sc, st);
-  }
+                                   const DevScalars* sc, cudaStream_t st, Bat bat) {
+  if (!comb_pair_supported(N, M) || (bat.on && !sc)) return cudaErrorInvalidValue;
+#define OTGB_CALL(n) row_update_pair_L<n>(q, u_in, u_out, step, N, tbdd, sc, st, bat)
+  OTGB_ROW_LENGTHS(M / 2, OTGB_CALL)
+#undef OTGB_CALL
   return cudaErrorInvalidValue;
 }
 
