@@ -15,9 +15,7 @@
 
 namespace otgb {
 
-#define RTX 32  // residual tile width (x / columns)
-#define RTY 32  // residual tile height (y / rows); 8 warps, 4 rows per thread
-#define RPT 4   // rows per thread
+#define RTX 32  // residual tile width (x / columns); 8 warps
 
 // Block sum of NV floats (result valid in thread 0).
 template <int NV>
@@ -161,18 +159,36 @@ __global__ void k_input_stats(const double* __restrict__ f, const double* __rest
   partials = badv(partials, bat);
   sc = badv(sc, bat);
   if (bskip(sc, bat)) return;
+  // per thread: the sums in FP64, minima and counts on the integer pipe (FP64 starts two
+  // instructions per clock and SM on this GPU); four loads of each plane in flight
   double v[6] = {0.0, 0.0, INFINITY, INFINITY, 0.0, 0.0};
   const int kind[6] = {0, 0, 2, 2, 0, 0};
-  for (long p = blockIdx.x * (long)blockDim.x + threadIdx.x; p < P;
-       p += (long)gridDim.x * blockDim.x) {
-    double a = f[p], b = g[p];
-    v[0] += a;
-    v[1] += b;
-    v[2] = fmin(v[2], a);
-    v[3] = fmin(v[3], b);
-    v[4] += isfinite(a) ? 0.0 : 1.0;
-    v[5] += isfinite(b) ? 0.0 : 1.0;
+  long long kf = ordered_key(INFINITY), kg = kf;
+  int bf = 0, bg = 0;
+  const long nth = (long)gridDim.x * blockDim.x;
+  for (long p = blockIdx.x * (long)blockDim.x + threadIdx.x; p < P; p += 4 * nth) {
+    double a[4], b[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const bool in = p + k * nth < P;
+      a[k] = in ? f[p + k * nth] : 0.0;
+      b[k] = in ? g[p + k * nth] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (p + k * nth >= P) break;
+      v[0] += a[k];
+      v[1] += b[k];
+      bf += !finite_key(a[k]);
+      bg += !finite_key(b[k]);
+      if (!nan_key(a[k])) kf = min(kf, ordered_key(a[k]));
+      if (!nan_key(b[k])) kg = min(kg, ordered_key(b[k]));
+    }
   }
+  v[2] = key_value(kf);
+  v[3] = key_value(kg);
+  v[4] = (double)bf;
+  v[5] = (double)bg;
   // per-thread FP64, then the block and grid reductions in double-float (FP32 pipes)
   dd r[6];
 #pragma unroll
@@ -223,215 +239,6 @@ static int reduce_blocks() {
     nb = (sms > 0 ? sms : 148) * 2;
   }
   return nb;
-}
-
-// ---------------------------------------------------------------------------------------
-// Cubic B-spline prefilter (Sec. 4, interpolation of g: the coefficients c, with
-// (c[k-1] + 4 c[k] + c[k+1]) / 6 = g[k] along each axis, periodic) as recursive filters.
-// The periodic inverse of the stencil (1, 4, 1) / 6 is 6 h * with h[k] = z z^|k| / (z^2 - 1),
-// z = sqrt(3) - 2 the root of z^2 + 4 z + 1 inside the unit circle (its DTFT is
-// 1 / (4 + 2 cos t)), and sum_k z^|k| s[i - k] = cp[i] + ca[i] - s[i] with the first-order
-// recursions cp[i] = s[i] + z cp[i - 1] (causal) and ca[i] = s[i] + z ca[i + 1]
-// (anticausal).  A thread runs both over a chunk of PRE_CH points of one line, starting each
-// from PRE_K periodic terms beyond the chunk (|z|^PRE_K < 1e-22, below FP64 round-off): the
-// circular deconvolution to FP64 round-off with a few multiply-adds per point, where the
-// spectral form takes three FP64 transform passes.  (256 threads = 32 lines x 8 chunks of
-// PRE_CH = 32 points per tile of 256 points.)
-// ---------------------------------------------------------------------------------------
-constexpr int PRE_K = 40, PRE_CH = 32;
-
-// One axis, tiled: a block stages 32 lines x (256 points + PRE_K on each side, periodic) in
-// shared memory with coalesced loads (all of them in flight at once: the recursions
-// themselves are short serial chains, so the loads' latency is what a direct version waits
-// on), runs the two recursions per thread over a chunk of PRE_CH points of one line, and
-// writes the tile back coalesced.  XPASS: lines are rows (points along x), else columns.
-// dd_out (optional) also receives the result split as (hi, lo) floats.
-constexpr int PT_LN = 32, PT_TP = 256, PT_SW = PT_LN + 1;
-constexpr size_t PT_SMEM = (size_t)(PT_TP + 2 * PRE_K) * PT_SW * sizeof(double);
-
-template <bool XPASS>
-__global__ void __launch_bounds__(256)
-    k_prefilter_tile(const double* __restrict__ s, double* __restrict__ out,
-                     float2* __restrict__ dd_out, int N, int M, double z, double A, Bat bat) {
-  extern __shared__ __align__(16) double smp[];  // [k][line], k = point - p0 + PRE_K
-  s = badv(s, bat);
-  out = badv(out, bat);
-  dd_out = badv(dd_out, bat);
-  const int tid = threadIdx.x;
-  const int L = XPASS ? M : N, nlines = XPASS ? N : M;
-  const long ls = XPASS ? M : 1, ps = XPASS ? 1 : M;
-  const int line0 = blockIdx.x * PT_LN, p0 = blockIdx.y * PT_TP;
-  const int tpl = min(PT_TP, L - p0), nk = tpl + 2 * PRE_K;
-  // stage (lines fastest for columns, points fastest for rows: both coalesced)
-  for (int e = tid; e < nk * PT_LN; e += blockDim.x) {
-    const int k = XPASS ? e % nk : e / PT_LN, ln = XPASS ? e / nk : e % PT_LN;
-    const int line = line0 + ln;
-    const int pt = ((p0 - PRE_K + k) % L + L) % L;
-    smp[k * PT_SW + ln] = line < nlines ? s[line * ls + pt * ps] : 0.0;
-  }
-  __syncthreads();
-  const int ln = tid % PT_LN, c0 = (tid / PT_LN) * PRE_CH, n = min(PRE_CH, tpl - c0);
-  double v[PRE_CH];
-  if (n > 0) {
-    double cp = 0.0, ca = 0.0;
-    for (int k = c0; k < c0 + PRE_K; ++k) cp = fma(z, cp, smp[k * PT_SW + ln]);
-    for (int k = c0 + n + 2 * PRE_K - 1; k >= c0 + n + PRE_K; --k)
-      ca = fma(z, ca, smp[k * PT_SW + ln]);
-#pragma unroll
-    for (int i = 0; i < PRE_CH; ++i)
-      if (i < n) {
-        cp = fma(z, cp, smp[(c0 + PRE_K + i) * PT_SW + ln]);
-        v[i] = cp;
-      }
-#pragma unroll
-    for (int i = PRE_CH - 1; i >= 0; --i)
-      if (i < n) {
-        const double xi = smp[(c0 + PRE_K + i) * PT_SW + ln];
-        ca = fma(z, ca, xi);
-        v[i] = A * (v[i] + ca - xi);
-      }
-  }
-  __syncthreads();  // every chunk has read its neighbours' points
-  if (n > 0) {
-#pragma unroll
-    for (int i = 0; i < PRE_CH; ++i)
-      if (i < n) smp[(c0 + PRE_K + i) * PT_SW + ln] = v[i];
-  }
-  __syncthreads();
-  for (int e = tid; e < tpl * PT_LN; e += blockDim.x) {
-    const int k = XPASS ? e % tpl : e / PT_LN, l2 = XPASS ? e / tpl : e % PT_LN;
-    const int line = line0 + l2;
-    if (line >= nlines) continue;
-    const double r = smp[(k + PRE_K) * PT_SW + l2];
-    const long o = line * ls + (long)(p0 + k) * ps;
-    out[o] = r;
-    if (dd_out) {
-      const float hi = __double2float_rn(r);
-      dd_out[o] = make_float2(hi, __double2float_rn(r - (double)hi));
-    }
-  }
-}
-
-// The same two passes in double-float arithmetic for the mixed mode (FP64 runs at a small
-// fraction of the FP32 rate on this GPU, and the FP64 recursions had become the largest of a
-// solve's one-off kernels): the columns' pass reads g in FP64 and leaves the dd result in
-// `mid`, the rows' pass reads that and writes c as dd (hi, lo) and as its FP64 sum.  The
-// recursions, the chunking and the warm-up length are those of the FP64 kernel; each step
-// z cp + s is a dd product and sum (relative error ~2^-47 per step, damped by |z| = 0.27).
-template <bool XPASS>
-__global__ void __launch_bounds__(256)
-    k_prefilter_tile_dd(const double* __restrict__ s64, const float2* __restrict__ sdd,
-                        float2* __restrict__ out_dd, double* __restrict__ out64, int N, int M,
-                        double z, double A, Bat bat) {
-  extern __shared__ __align__(16) float2 smq[];  // [k][line] as (hi, lo)
-  s64 = badv(s64, bat);
-  sdd = badv(sdd, bat);
-  out_dd = badv(out_dd, bat);
-  out64 = badv(out64, bat);
-  const int tid = threadIdx.x;
-  const int L = XPASS ? M : N, nlines = XPASS ? N : M;
-  const long ls = XPASS ? M : 1, ps = XPASS ? 1 : M;
-  const int line0 = blockIdx.x * PT_LN, p0 = blockIdx.y * PT_TP;
-  const int tpl = min(PT_TP, L - p0), nk = tpl + 2 * PRE_K;
-  for (int e = tid; e < nk * PT_LN; e += blockDim.x) {
-    const int k = XPASS ? e % nk : e / PT_LN, ln = XPASS ? e / nk : e % PT_LN;
-    const int line = line0 + ln;
-    const int pt = ((p0 - PRE_K + k) % L + L) % L;
-    float2 x = make_float2(0.f, 0.f);
-    if (line < nlines) {
-      const long o = line * ls + pt * ps;
-      if (s64) {
-        const dd d = dd_from_double(s64[o]);
-        x = make_float2(d.hi, d.lo);
-      } else {
-        x = sdd[o];
-      }
-    }
-    smq[k * PT_SW + ln] = x;
-  }
-  __syncthreads();
-  const dd zd = dd(z), Ad = dd(A);
-  const int ln = tid % PT_LN, c0 = (tid / PT_LN) * PRE_CH, n = min(PRE_CH, tpl - c0);
-  dd v[PRE_CH];
-  auto at = [&](int k) {
-    const float2 q = smq[k * PT_SW + ln];
-    return dd{q.x, q.y};
-  };
-  if (n > 0) {
-    dd cp{0.f, 0.f}, ca{0.f, 0.f};
-    for (int k = c0; k < c0 + PRE_K; ++k) cp = dd_add(dd_mul(zd, cp), at(k));
-    for (int k = c0 + n + 2 * PRE_K - 1; k >= c0 + n + PRE_K; --k)
-      ca = dd_add(dd_mul(zd, ca), at(k));
-#pragma unroll
-    for (int i = 0; i < PRE_CH; ++i)
-      if (i < n) {
-        cp = dd_add(dd_mul(zd, cp), at(c0 + PRE_K + i));
-        v[i] = cp;
-      }
-#pragma unroll
-    for (int i = PRE_CH - 1; i >= 0; --i)
-      if (i < n) {
-        const dd xi = at(c0 + PRE_K + i);
-        ca = dd_add(dd_mul(zd, ca), xi);
-        v[i] = dd_mul(Ad, dd_sub(dd_add(v[i], ca), xi));
-      }
-  }
-  __syncthreads();  // every chunk has read its neighbours' points
-  if (n > 0) {
-#pragma unroll
-    for (int i = 0; i < PRE_CH; ++i)
-      if (i < n) smq[(c0 + PRE_K + i) * PT_SW + ln] = make_float2(v[i].hi, v[i].lo);
-  }
-  __syncthreads();
-  for (int e = tid; e < tpl * PT_LN; e += blockDim.x) {
-    const int k = XPASS ? e % tpl : e / PT_LN, l2 = XPASS ? e / tpl : e % PT_LN;
-    const int line = line0 + l2;
-    if (line >= nlines) continue;
-    const float2 r = smq[(k + PRE_K) * PT_SW + l2];
-    const long o = line * ls + (long)(p0 + k) * ps;
-    out_dd[o] = r;
-    if (out64) out64[o] = (double)r.x + (double)r.y;
-  }
-}
-
-cudaError_t launch_prefilter(const double* g, double* scratch, double* c, float2* cdd, int N,
-                             int M, cudaStream_t st, Bat bat) {
-  static bool attr_set[64] = {false};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (!attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(k_prefilter_tile<false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, PT_SMEM);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_prefilter_tile<true>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, PT_SMEM);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_prefilter_tile_dd<false>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, PT_SMEM);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_prefilter_tile_dd<true>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, PT_SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set[dev] = true;
-  }
-  const double z = sqrt(3.0) - 2.0;
-  const double A = 6.0 * z / (z * z - 1.0);
-  // columns (along y), then rows (along x)
-  const dim3 gy((M + PT_LN - 1) / PT_LN, (N + PT_TP - 1) / PT_TP);
-  const dim3 gx((N + PT_LN - 1) / PT_LN, (M + PT_TP - 1) / PT_TP);
-  if (cdd) {  // mixed mode: double-float passes (the scratch plane holds the dd middle)
-    float2* mid = reinterpret_cast<float2*>(scratch);
-    k_prefilter_tile_dd<false><<<bgrid(gy, bat), 256, PT_SMEM, st>>>(g, nullptr, mid, nullptr,
-                                                                      N, M, z, A, bat);
-    k_prefilter_tile_dd<true><<<bgrid(gx, bat), 256, PT_SMEM, st>>>(nullptr, mid, cdd, c, N, M,
-                                                                     z, A, bat);
-    return cudaGetLastError();
-  }
-  k_prefilter_tile<false><<<bgrid(gy, bat), 256, PT_SMEM, st>>>(g, scratch, nullptr, N, M, z, A,
-                                                                 bat);
-  k_prefilter_tile<true><<<bgrid(gx, bat), 256, PT_SMEM, st>>>(scratch, c, cdd, N, M, z, A, bat);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_input_stats(const double* f, const double* g, int N, int M,
@@ -575,11 +382,14 @@ __device__ __forceinline__ int dd_floor(dd p, dd* t) {
   return (int)fl;
 }
 
-__global__ void __launch_bounds__(RTX * RTY / RPT, 3)
+// A block covers 32 columns x 8 RPT rows, RPT rows per thread.
+template <int RPT>
+__global__ void __launch_bounds__(8 * RTX, 3)
     k_residual_dd(const float2* __restrict__ fdd, const float2* __restrict__ cdd,
                   const double* __restrict__ ua, const double* __restrict__ ub, int sel, int N,
                   int M, ResidConstsDD K, double* __restrict__ Fraw, float* __restrict__ coef,
                   double* partials, DevScalars* sc, Bat bat) {
+  constexpr int RTY = 8 * RPT;
   __shared__ dd tile[RTY + 4][RTX + 4];
   __shared__ dd dyt[RTY][RTX + 4];  // unscaled y-difference of u (halo 2 in x)
   fdd = badv(fdd, bat);
@@ -622,7 +432,7 @@ __global__ void __launch_bounds__(RTX * RTY / RPT, 3)
   const float wx = ((j & 1) ? 4.0f : 2.0f) * K.w3M;
 #pragma unroll 1
   for (int rr = 0; rr < RPT; ++rr) {
-    const int ty = ty0 + rr * (RTY / RPT);
+    const int ty = ty0 + rr * 8;
     const int i = by + ty;
     if (i >= N || j >= M) continue;
     const int r = ty + 2, q = tx + 2;
@@ -828,7 +638,6 @@ cudaError_t launch_residual_dd(const float2* fdd, const float2* cdd, const doubl
                                int M, double* Fraw, float* coef, double* partials,
                                DevScalars* sc, cudaStream_t st, const double* ub, int sel,
                                int simplified, Bat bat, Interp ip) {
-  dim3 grid((M + RTX - 1) / RTX, (N + RTY - 1) / RTY);
   ResidConstsDD K;
   K.Mh = host_dd((double)M / 12.0);
   K.Nh = host_dd((double)N / 12.0);
@@ -845,8 +654,17 @@ cudaError_t launch_residual_dd(const float2* fdd, const float2* cdd, const doubl
   K.gx = ip.gx32;
   K.gy = ip.gy32;
   if (ip.mode && !(ip.gx32 && ip.gy32)) return cudaErrorInvalidValue;
-  k_residual_dd<<<bgrid(grid, bat), RTX * RTY / RPT, 0, st>>>(fdd, cdd, ua, ub, sel, N, M, K,
-                                                                Fraw, coef, partials, sc, bat);
+  // 32-row tiles (four points per thread), 8-row tiles on the smallest grids: a thread's four
+  // points follow each other, 20 us however few the blocks.  32-row / 8-row tiles, us: 20.5 / 12.1
+  // at 16 tiles (128^2), 21.3 / 15.9 at 64 (256^2), 20.9 / 17.0 at 80 (five of 128^2), but
+  // 22.3 / 24.9 at 144 (384^2) and 29.2 / 36.6 at 256 (512^2), where the block sums weigh more.
+  const int mx = (M + RTX - 1) / RTX;
+  if ((long)mx * ((N + 31) / 32) * (bat.on ? bat.n : 1) > 96)
+    k_residual_dd<4><<<bgrid(dim3(mx, (N + 31) / 32), bat), 8 * RTX, 0, st>>>(
+        fdd, cdd, ua, ub, sel, N, M, K, Fraw, coef, partials, sc, bat);
+  else
+    k_residual_dd<1><<<bgrid(dim3(mx, (N + 7) / 8), bat), 8 * RTX, 0, st>>>(
+        fdd, cdd, ua, ub, sel, N, M, K, Fraw, coef, partials, sc, bat);
   return cudaGetLastError();
 }
 

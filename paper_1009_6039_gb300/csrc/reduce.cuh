@@ -9,6 +9,24 @@
 
 namespace otgb {
 
+// doubles as integers of the same order (not for NaN), and tests on the bits: comparisons on the
+// integer pipe
+__device__ __forceinline__ long long ordered_bits(long long b) {
+  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ long long ordered_key(double x) {
+  return ordered_bits(__double_as_longlong(x));
+}
+__device__ __forceinline__ double key_value(long long k) {
+  return __longlong_as_double(ordered_bits(k));
+}
+__device__ __forceinline__ bool finite_key(double x) {
+  return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
+}
+__device__ __forceinline__ bool nan_key(double x) {
+  return (__double_as_longlong(x) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
+}
+
 // ---------------------------------------------------------------------------------------
 // block reductions
 // ---------------------------------------------------------------------------------------

@@ -44,20 +44,6 @@ __device__ __forceinline__ int wrap_any(int a, int L) {
   return r < 0 ? r + L : r;
 }
 
-// doubles as integers of the same order (not for NaN); its own inverse
-__device__ __forceinline__ long long ordered(long long b) {
-  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
-}
-__device__ __forceinline__ long long key(double x) { return ordered(__double_as_longlong(x)); }
-__device__ __forceinline__ double unkey(long long k) { return __longlong_as_double(ordered(k)); }
-__device__ __forceinline__ bool finite_bits(double x) {
-  return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
-}
-__device__ __forceinline__ bool nan_bits(double x) {
-  const long long b = __double_as_longlong(x) & 0x7fffffffffffffffLL;
-  return b > 0x7ff0000000000000LL;
-}
-
 // floor of x and the fraction t = x - floor(x) in [0, 1] (for any x: the index is wrapped later)
 __device__ __forceinline__ int floor_frac(double x, double* t) {
   const double m = x + 6755399441055744.0;  // 1.5 x 2^52: the nearest integer in the low bits
@@ -171,8 +157,8 @@ __global__ void __launch_bounds__(TWX * (TH < 8 ? TH : 8), TH == 32 ? 3 : 4)
   Red red;
 #pragma unroll
   for (int a = 0; a < 6; ++a) red.s[a] = 0.0;
-  red.kmax = key(-INFINITY);
-  red.kmin = red.kdet = key(INFINITY);
+  red.kmax = ordered_key(-INFINITY);
+  red.kmin = red.kdet = ordered_key(INFINITY);
   red.bad = 0;
   const int tx = tid & 31, ty0 = tid >> 5;
   const int j = bx + tx;
@@ -274,14 +260,14 @@ __global__ void __launch_bounds__(TWX * (TH < 8 ? TH : 8), TH == 32 ? 3 : 4)
     red.s[3] += a22;
     red.s[4] += b1;
     red.s[5] += b2;
-    if (finite_bits(fn)) {
+    if (finite_key(fn)) {
       red.s[0] += fn;
-      red.kmax = max(red.kmax, key(fr));
-      red.kmin = min(red.kmin, key(fr));
+      red.kmax = max(red.kmax, ordered_key(fr));
+      red.kmin = min(red.kmin, ordered_key(fr));
     } else {
       red.bad += 1;
     }
-    if (!nan_bits(det)) red.kdet = min(red.kdet, key(det));
+    if (!nan_key(det)) red.kdet = min(red.kdet, ordered_key(det));
   }
   // composite Simpson: weights 2 / 4 by the parity of i and j, both fixed per thread
   const double w = (((by + ty0) & 1) ? 4.0 : 2.0) * ((j & 1) ? 4.0 : 2.0) * K.w3;
@@ -310,8 +296,8 @@ __global__ void __launch_bounds__(TWX * (TH < 8 ? TH : 8), TH == 32 ? 3 : 4)
   __threadfence();
 #pragma unroll
   for (int a = 0; a < 6; ++a) red.s[a] = 0.0;
-  red.kmax = key(-INFINITY);
-  red.kmin = red.kdet = key(INFINITY);
+  red.kmax = ordered_key(-INFINITY);
+  red.kmin = red.kdet = ordered_key(INFINITY);
   red.bad = 0;
   for (unsigned int b = tid; b < nb; b += NT) {
     const double* q = partials + (size_t)b * 10;
@@ -329,10 +315,10 @@ __global__ void __launch_bounds__(TWX * (TH < 8 ? TH : 8), TH == 32 ? 3 : 4)
   for (int a = 0; a < 6; ++a) tot[a] = __shfl_sync(0xffffffffu, red.s[0], a);
   if (tid == 0) {
     const double mean_fn = tot[0] / ((double)N * (double)M);
-    const double shift = mean_fn - 1.0, dmin = unkey(red.kdet);
+    const double shift = mean_fn - 1.0, dmin = key_value(red.kdet);
     sc->mean_fn = mean_fn;
     sc->shift = shift;
-    sc->res_inf = fmax(fabs(unkey(red.kmax) + shift), fabs(unkey(red.kmin) + shift));
+    sc->res_inf = fmax(fabs(key_value(red.kmax) + shift), fabs(key_value(red.kmin) + shift));
     for (int a = 0; a < 5; ++a) sc->abar[a] = tot[1 + a];
     sc->min_det = dmin;
     sc->k1_nonfinite = red.bad;
