@@ -23,12 +23,43 @@ struct dd {
 
 __device__ __forceinline__ dd dd_make(float hi, float lo) { return dd(hi, lo); }
 
-// split an FP64 value: hi = nearest float, lo = nearest float to the (exact) remainder
-__device__ __forceinline__ dd dd_from_double(double a) {
+// Conversions to and from FP64 on the integer pipe: the cvt instructions run at the FP64 rate (a
+// warp instruction per 16 clocks and SM on GB300), four of them per split and three per sum, which
+// had become a third to a half of the time of the passes that read or write FP64 planes.
+//
+// The split with cvt instructions (hi rounds ties to even), also for a kernel that has no registers
+// left for the integer form: the residual kernel would spill 108 bytes at its 80 registers and take
+// 79 instead of 75 us at 1024x1024.
+__device__ __forceinline__ dd dd_from_double_cvt(double a) {
   const float h = __double2float_rn(a);
   return dd{h, __double2float_rn(a - (double)h)};
 }
-__device__ __forceinline__ double dd_to_double(dd a) { return (double)a.hi + (double)a.lo; }
+// split an FP64 value: hi = nearest float (ties away from zero), lo = nearest float to the (exact)
+// remainder
+__device__ __forceinline__ dd dd_from_double(double a) {
+  const unsigned int h = __double2hiint(a), l = __double2loint(a);
+  const unsigned int e = (h >> 20) & 0x7ff;
+  if (e - 949u <= 200u) {  // 2^-74 <= |a| < 2^127: hi and the scale of lo are normal floats
+    const unsigned int sign = h & 0x80000000u;
+    const int up = (l >> 28) & 1, rem = (int)(l & 0x1fffffffu) - (up << 29);
+    // exponent and the top 23 mantissa bits, rebiased by 896
+    const unsigned int f = __funnelshift_l(l, h, 3) - 0xC0000000u + up;
+    const float scale = __uint_as_float(((e - 948u) << 23) | sign);  // 2^(e - 1023 - 52)
+    return dd{__uint_as_float((f & 0x7fffffffu) | sign), __fmul_rn((float)rem, scale)};
+  }
+  return dd_from_double_cvt(a);
+}
+// the double of a float
+__device__ __forceinline__ double float_to_double(float x) {
+  const unsigned int b = __float_as_uint(x);
+  if (((b >> 23) & 0xff) - 1u < 254u)
+    return __hiloint2double((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u), b << 29);
+  if ((b << 1) == 0) return __hiloint2double(b, 0);
+  return (double)x;  // denormal, infinite, NaN
+}
+__device__ __forceinline__ double dd_to_double(dd a) {
+  return float_to_double(a.hi) + float_to_double(a.lo);
+}
 
 // s + e = a + b exactly (Knuth)
 __device__ __forceinline__ dd two_sum(float a, float b) {

@@ -111,11 +111,6 @@ __device__ void block_reduce_dd(dd (&v)[NV], const int (&kind)[NV]) {
   }
   __syncthreads();
 }
-// a double as (hi, lo) floats; infinities keep lo = 0
-__device__ __forceinline__ dd dd_of_double(double a) {
-  const float h = __double2float_rn(a);
-  return dd{h, isfinite(h) ? __double2float_rn(a - (double)h) : 0.0f};
-}
 // grid-wide: per-block (hi, lo) partials, the last block to take a ticket combines them in
 // block order; true in that block, totals in thread 0 (2-D grids allowed)
 template <int NV>
@@ -152,6 +147,42 @@ __device__ bool grid_reduce_dd(dd (&v)[NV], const int (&kind)[NV], double* parti
 // Input translation (Eq. translation applied to both densities, as for the images of
 // Sec. 5.2): d <- d - mean(d) + 1; rejects non-finite input or a non-positive result.
 // ---------------------------------------------------------------------------------------
+// block sums of v, minima of kf and kg (ordered_key) and counts bf, bg, in thread 0 of 256
+__device__ __forceinline__ void input_reduce(double (&v)[2], long long& kf, long long& kg, int& bf,
+                                             int& bg) {
+  __shared__ double ss[2];
+  __shared__ long long sk[8][2];
+  __shared__ int sb[8][2];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    kf = min(kf, __shfl_xor_sync(0xffffffffu, kf, o));
+    kg = min(kg, __shfl_xor_sync(0xffffffffu, kg, o));
+  }
+  bf = __reduce_add_sync(0xffffffffu, bf);
+  bg = __reduce_add_sync(0xffffffffu, bg);
+  if (lane == 0) {
+    sk[wid][0] = kf;
+    sk[wid][1] = kg;
+    sb[wid][0] = bf;
+    sb[wid][1] = bg;
+  }
+  double s;
+  if (block_fold<2>(v, s)) ss[threadIdx.x >> 3] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    v[0] = ss[0];
+    v[1] = ss[1];
+    for (int w = 1; w < 8; ++w) {
+      kf = min(kf, sk[w][0]);
+      kg = min(kg, sk[w][1]);
+      bf += sb[w][0];
+      bg += sb[w][1];
+    }
+  }
+  __syncthreads();
+}
+
 __global__ void k_input_stats(const double* __restrict__ f, const double* __restrict__ g,
                               long P, double* partials, DevScalars* sc, Bat bat) {
   f = badv(f, bat);
@@ -161,8 +192,7 @@ __global__ void k_input_stats(const double* __restrict__ f, const double* __rest
   if (bskip(sc, bat)) return;
   // per thread: the sums in FP64, minima and counts on the integer pipe (FP64 starts two
   // instructions per clock and SM on this GPU); four loads of each plane in flight
-  double v[6] = {0.0, 0.0, INFINITY, INFINITY, 0.0, 0.0};
-  const int kind[6] = {0, 0, 2, 2, 0, 0};
+  double v[2] = {0.0, 0.0};
   long long kf = ordered_key(INFINITY), kg = kf;
   int bf = 0, bg = 0;
   const long nth = (long)gridDim.x * blockDim.x;
@@ -185,29 +215,48 @@ __global__ void k_input_stats(const double* __restrict__ f, const double* __rest
       if (!nan_key(b[k])) kg = min(kg, ordered_key(b[k]));
     }
   }
-  v[2] = key_value(kf);
-  v[3] = key_value(kg);
-  v[4] = (double)bf;
-  v[5] = (double)bg;
-  // per-thread FP64, then the block and grid reductions in double-float (FP32 pipes)
-  dd r[6];
-#pragma unroll
-  for (int a = 0; a < 6; ++a) r[a] = dd_of_double(v[a]);
-  if (!grid_reduce_dd<6>(r, kind, partials, &sc->ticket[TK_INPUT])) return;
+  input_reduce(v, kf, kg, bf, bg);
+  __shared__ bool last;
   if (threadIdx.x == 0) {
-#pragma unroll
-    for (int a = 0; a < 6; ++a) v[a] = (double)r[a].hi + (double)r[a].lo;
+    double* q = partials + (size_t)blockIdx.x * 6;
+    q[0] = v[0];
+    q[1] = v[1];
+    q[2] = __longlong_as_double(kf);
+    q[3] = __longlong_as_double(kg);
+    q[4] = __longlong_as_double(bf);
+    q[5] = __longlong_as_double(bg);
+    __threadfence();
+    last = atomicAdd(&sc->ticket[TK_INPUT], 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  v[0] = v[1] = 0.0;
+  kf = kg = ordered_key(INFINITY);
+  bf = bg = 0;
+  for (unsigned int b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+    const double* q = partials + (size_t)b * 6;
+    v[0] += __ldcg(q);
+    v[1] += __ldcg(q + 1);
+    kf = min(kf, __double_as_longlong(__ldcg(q + 2)));
+    kg = min(kg, __double_as_longlong(__ldcg(q + 3)));
+    bf += (int)__double_as_longlong(__ldcg(q + 4));
+    bg += (int)__double_as_longlong(__ldcg(q + 5));
+  }
+  input_reduce(v, kf, kg, bf, bg);
+  if (threadIdx.x == 0) {
+    const double fmin = key_value(kf), gmin = key_value(kg);
     sc->in_mean[0] = v[0] / (double)P;
     sc->in_mean[1] = v[1] / (double)P;
-    sc->in_min[0] = v[2];
-    sc->in_min[1] = v[3];
-    sc->in_nonfinite[0] = (int)v[4];
-    sc->in_nonfinite[1] = (int)v[5];
+    sc->in_min[0] = fmin;
+    sc->in_min[1] = gmin;
+    sc->in_nonfinite[0] = bf;
+    sc->in_nonfinite[1] = bg;
     // translated inputs must be positive after the translation, inputs used as given
     // (in_plain) as they are
     const double sf = sc->in_plain ? 0.0 : 1.0 - sc->in_mean[0];
     const double sg = sc->in_plain ? 0.0 : 1.0 - sc->in_mean[1];
-    bool bad = v[4] > 0 || v[5] > 0 || !(v[2] + sf > 0.0) || !(v[3] + sg > 0.0);
+    const bool bad = bf > 0 || bg > 0 || !(fmin + sf > 0.0) || !(gmin + sg > 0.0);
     sc->in_bad = bad ? 1 : 0;
     sc->ticket[TK_INPUT] = 0;
   }
@@ -230,7 +279,9 @@ __global__ void k_input_apply(const double* __restrict__ f, const double* __rest
   }
 }
 
-static int reduce_blocks() {
+// blocks of a grid reduction or an elementwise pass over P points: 1024 points each, at most two
+// blocks per SM
+static int reduce_blocks(long P) {
   static int nb = 0;
   if (nb == 0) {
     int dev = 0, sms = 0;
@@ -238,13 +289,13 @@ static int reduce_blocks() {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     nb = (sms > 0 ? sms : 148) * 2;
   }
-  return nb;
+  return (int)(P < 1024L * nb ? (P + 1023) / 1024 : nb);
 }
 
 cudaError_t launch_input_stats(const double* f, const double* g, int N, int M,
                                double* partials, DevScalars* sc, cudaStream_t st, Bat bat) {
-  k_input_stats<<<bgrid(dim3(reduce_blocks()), bat), 256, 0, st>>>(f, g, (long)N * M, partials,
-                                                                   sc, bat);
+  const long P = (long)N * M;
+  k_input_stats<<<bgrid(dim3(reduce_blocks(P)), bat), 256, 0, st>>>(f, g, P, partials, sc, bat);
   return cudaGetLastError();
 }
 
@@ -268,7 +319,7 @@ cudaError_t launch_translate_inputs(const double* f, const double* g, double* ft
                                     int N, int M, double* partials, DevScalars* sc,
                                     cudaStream_t st, Bat bat) {
   const long P = (long)N * M;
-  const dim3 nb = bgrid(dim3(reduce_blocks()), bat);
+  const dim3 nb = bgrid(dim3(reduce_blocks(P)), bat);
   k_input_stats<<<nb, 256, 0, st>>>(f, g, P, partials, sc, bat);
   k_input_apply<<<nb, 256, 0, st>>>(f, g, ft, gt, P, sc, bat);
   return cudaGetLastError();
@@ -411,7 +462,7 @@ __global__ void __launch_bounds__(8 * RTX, 3)
     while (gi >= N) gi -= N;
     while (gj < 0) gj += M;
     while (gj >= M) gj -= M;
-    tile[r][cc] = dd_from_double(u[(size_t)gi * M + gj]);
+    tile[r][cc] = dd_from_double_cvt(u[(size_t)gi * M + gj]);
   }
   __syncthreads();
   for (int idx = tid; idx < RTY * (RTX + 4); idx += blockDim.x) {
@@ -551,7 +602,7 @@ __global__ void __launch_bounds__(8 * RTX, 3)
     const dd fn = dd_mul(G, det);
     const size_t p = (size_t)i * M + j;
     const dd fr = dd_sub(ldd(fdd, p), fn);
-    Fraw[p] = dd_to_double(fr);
+    Fraw[p] = (double)fr.hi + (double)fr.lo;
     // coefficients of the linearisation (Jacobian only), FP32
     const float Gt = G.hi, dett = det.hi;
     const float a11 = Gt * (1.0f + uyy.hi), a12 = -Gt * uxy.hi, a22 = Gt * (1.0f + uxx.hi);
@@ -694,7 +745,7 @@ __global__ void k_sub(double* __restrict__ u, long P, const double* __restrict__
 
 cudaError_t launch_subtract_mean(double* u, int N, int M, double* partials, DevScalars* sc,
                                  double* mean_out, cudaStream_t st) {
-  const int nb = reduce_blocks();
+  const int nb = reduce_blocks((long)N * M);
   k_sum<<<nb, 256, 0, st>>>(u, (long)N * M, partials, sc, mean_out);
   k_sub<<<nb, 256, 0, st>>>(u, (long)N * M, mean_out);
   return cudaGetLastError();
@@ -729,7 +780,7 @@ __global__ void k_gmres_init(const double* __restrict__ Fraw, const T* __restric
     T bt;
     if constexpr (sizeof(T) == 4) {
       // the shifted residual in FP64 (one add), the rest in the vector precision
-      float b = __double2float_rn(Fraw[p] + s) * (float)inv_tau;  // h = (f - f~_n) / tau
+      float b = dd_from_double(Fraw[p] + s).hi * (float)inv_tau;  // h = (f - f~_n) / tau
       if (restart) b -= w[p];
       bt = b;
     } else {
@@ -1373,7 +1424,7 @@ __global__ void k_sub_sel(UPair up, double* __restrict__ out, long P,
 
 cudaError_t launch_final_gauge(UPair u, double* out, int N, int M, double* partials,
                                DevScalars* sc, double* mean_out, cudaStream_t st, Bat bat) {
-  const dim3 nb = bgrid(dim3(reduce_blocks()), bat);
+  const dim3 nb = bgrid(dim3(reduce_blocks((long)N * M)), bat);
   k_sum_sel<<<nb, 256, 0, st>>>(u, (long)N * M, partials, sc, mean_out, bat);
   k_sub_sel<<<nb, 256, 0, st>>>(u, out, (long)N * M, sc, mean_out, bat);
   return cudaGetLastError();
@@ -1406,7 +1457,7 @@ __global__ void k_grad4(const double* __restrict__ g, int N, int M, double* __re
 
 cudaError_t launch_grad4(const double* g, int N, int M, double* gx, double* gy, float* gx32,
                          float* gy32, cudaStream_t st) {
-  k_grad4<<<reduce_blocks(), 256, 0, st>>>(g, N, M, gx, gy, gx32, gy32);
+  k_grad4<<<reduce_blocks((long)N * M), 256, 0, st>>>(g, N, M, gx, gy, gx32, gy32);
   return cudaGetLastError();
 }
 
@@ -1452,7 +1503,7 @@ cudaError_t launch_set_step(DevScalars* sc, int j, cudaStream_t st) {
 
 cudaError_t launch_normalize(double* x, long P, double* partials, DevScalars* sc,
                              cudaStream_t st) {
-  const int nb = reduce_blocks();
+  const int nb = reduce_blocks(P);
   k_norm2<<<nb, 256, 0, st>>>(x, P, partials, sc);
   k_scale_by_norm<<<nb, 256, 0, st>>>(x, P, sc);
   return cudaGetLastError();
@@ -1481,13 +1532,13 @@ __global__ void k_scatter(const double* __restrict__ src, double* const* __restr
 
 cudaError_t launch_gather(const double* const* tab, double* dst, long P, Bat bat,
                           cudaStream_t st) {
-  k_gather<<<bgrid(dim3(reduce_blocks()), bat), 256, 0, st>>>(tab, dst, P, bat);
+  k_gather<<<bgrid(dim3(reduce_blocks(P)), bat), 256, 0, st>>>(tab, dst, P, bat);
   return cudaGetLastError();
 }
 
 cudaError_t launch_scatter(const double* src, double* const* tab, long P, const DevScalars* sc,
                            Bat bat, cudaStream_t st) {
-  k_scatter<<<bgrid(dim3(reduce_blocks()), bat), 256, 0, st>>>(src, tab, P, sc, bat);
+  k_scatter<<<bgrid(dim3(reduce_blocks(P)), bat), 256, 0, st>>>(src, tab, P, sc, bat);
   return cudaGetLastError();
 }
 
@@ -1501,7 +1552,7 @@ __global__ void k_convert(const TI* __restrict__ in, TO* __restrict__ out, long 
 template <typename T>
 cudaError_t launch_convert(const void* in, int in_d, void* out, int out_d, long n,
                            cudaStream_t st) {
-  const int nb = reduce_blocks();
+  const int nb = reduce_blocks(n);
   if (in_d && out_d)
     k_convert<double, double><<<nb, 256, 0, st>>>((const double*)in, (double*)out, n);
   else if (in_d)

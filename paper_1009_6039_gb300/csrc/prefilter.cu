@@ -57,7 +57,7 @@ template <> struct Ops<dd> {
   static __device__ __forceinline__ float2 mem(dd v) { return make_float2(v.hi, v.lo); }
   static __device__ __forceinline__ void store(long o, float2 r, float2* odd, double* out) {
     odd[o] = r;
-    if (out) out[o] = (double)r.x + (double)r.y;
+    if (out) out[o] = dd_to_double(dd{r.x, r.y});
   }
   static __device__ __forceinline__ dd zero() { return dd{0.f, 0.f}; }
   static __device__ __forceinline__ dd step(dd z, dd a, dd s) { return dd_add(dd_mul(z, a), s); }

@@ -1541,8 +1541,8 @@ __global__ void __launch_bounds__(256)
     const int n = t + e * TPT;
     const ddc z = buf[n];
     double2 a = ui ? ui[n] : make_double2(0.0, 0.0);
-    a.x += step * dd_to_double(z.x);
-    a.y += step * dd_to_double(z.y);
+    a.x = fma(step, dd_to_double(z.x), a.x);
+    a.y = fma(step, dd_to_double(z.y), a.y);
     uo[n] = a;
   }
 }

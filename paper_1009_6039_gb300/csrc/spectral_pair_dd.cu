@@ -372,10 +372,10 @@ __global__ void __launch_bounds__(pthreads<L>(), L <= 512 ? 4 : 2)
     dc_to(dld(A, swz(n)), za, zb);
     double2 a = uia ? uia[n] : make_double2(0.0, 0.0);
     double2 b = uib ? uib[n] : make_double2(0.0, 0.0);
-    a.x += step * dd_to_double(za.x);
-    a.y += step * dd_to_double(za.y);
-    b.x += step * dd_to_double(zb.x);
-    b.y += step * dd_to_double(zb.y);
+    a.x = fma(step, dd_to_double(za.x), a.x);
+    a.y = fma(step, dd_to_double(za.y), a.y);
+    b.x = fma(step, dd_to_double(zb.x), b.x);
+    b.y = fma(step, dd_to_double(zb.y), b.y);
     uoa[n] = a;
     uob[n] = b;
   }
