@@ -1160,9 +1160,21 @@ static int read_scalars(ot_plan* p) {
 }
 
 
+// p->f, p->g = f, g translated to mean 1; the mixed mode also leaves f as (hi, lo) floats, and the
+// learned start's source log f - log g in src when given
+static int run_translate(ot_plan* p, const double* f, const double* g, Bat bat = Bat(),
+                         float* src = nullptr) {
+  LAUNCH(p, OT_PROF_OTHER, -1, 2,
+         launch_translate_inputs(f, g, p->f, p->g, p->N, p->M, p->partials, p->sc, p->stream, bat,
+                                 p->precision ? p->fdd : nullptr, src));
+  return OT_OK;
+}
+
 // c = B-spline coefficients of g in FP64 (recursive filters along y and x; p->Fraw is free
 // scratch before the first residual); the mixed mode also keeps c and f as (hi, lo) floats
-static int run_prefilter(ot_plan* p, const double* g, double* c) {
+// (f_split: run_translate has left f's; c32: a copy of c's high parts, in the mixed mode)
+static int run_prefilter(ot_plan* p, const double* g, double* c, bool f_split = false,
+                         float* c32 = nullptr) {
   if (p->interp) {
     // nearest / bilinear: the grid values themselves and their gradient
     const long P = (long)p->N * p->M;
@@ -1171,14 +1183,15 @@ static int run_prefilter(ot_plan* p, const double* g, double* c) {
            launch_grad4(g, p->N, p->M, p->gxy, p->gxy + P, p->gxy32, p->gxy32 + P, p->stream));
     if (p->precision) {
       LAUNCH(p, OT_PROF_OTHER, -1, 1, launch_split_dd(c, p->cdd, P, p->stream));
-      LAUNCH(p, OT_PROF_OTHER, -1, 1, launch_split_dd(p->f, p->fdd, P, p->stream));
+      if (!f_split)
+        LAUNCH(p, OT_PROF_OTHER, -1, 1, launch_split_dd(p->f, p->fdd, P, p->stream));
     }
     return OT_OK;
   }
   LAUNCH(p, OT_PROF_OTHER, -1, 2,
          launch_prefilter(g, p->Fraw, c, p->precision ? p->cdd : nullptr, p->N, p->M,
-                          p->stream, btc(p)));
-  if (p->precision)
+                          p->stream, btc(p), c32));
+  if (p->precision && !f_split)
     LAUNCH(p, OT_PROF_OTHER, -1, 1,
            launch_split_dd(p->f, p->fdd, (long)p->N * p->M, p->stream, btc(p)));
   return OT_OK;
@@ -1450,9 +1463,12 @@ static int alloc_ws(ot_plan* p) {
 // u_add may be null.
 static int run_ws_poisson32(ot_plan* p, const float* src32, double* u, const double* u_add,
                             bool lp) {
+  SpecTables tb = p->tb32;
+  // (nothing tuned: the pair row pass, 8.8 -> 4 us at 512x512 with cold caches)
+  if (tb.var_r2c == VAR_DEFAULT) tb.var_r2c = VAR_PAIR;
   LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
          launch_row_r2c<float>(src32, 0, nullptr, nullptr, (C2<float>*)p->spec, p->N, p->M,
-                               p->tb32, nullptr, p->stream));
+                               tb, nullptr, p->stream));
   LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
          launch_col_lbarinv_dd((const float2*)p->spec, (ddc*)p->q64, p->N, p->M, p->tb32,
                                p->tbdd, nullptr, p->stream, lp ? COL_POISSON_LP : COL_POISSON));
@@ -1485,33 +1501,37 @@ static int run_ws_poisson(ot_plan* p, const double* src, double* u, bool lp = fa
   return OT_OK;
 }
 
-// ws_src = log f - log g, ws_h = P(ws_src), ws_X = features at ws_h (f, g, c: the plan's
-// translated densities and B-spline coefficients)
-static int run_ws_features(ot_plan* p) {
+// ws_src = log f - log g, ws_h = P(ws_src), X = features at ws_h (f, g, c: the plan's
+// translated densities and B-spline coefficients; have: what ws_prepare_inputs has left)
+enum { WS_HAVE_SOURCE = 1, WS_HAVE_C32 = 2 };
+static int run_ws_features(ot_plan* p, float* X, int have = 0) {
   RET(alloc_ws(p));
   const long P = (long)p->N * p->M;
   if (p->precision) {
     // mixed: the source in FP32 (in ws_s, which the network overwrites later)
-    LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
-           launch_ws_source32(p->f, p->g, p->ws_s, P, p->stream));
+    if (!(have & WS_HAVE_SOURCE))
+      LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
+             launch_ws_source32(p->f, p->g, p->ws_s, P, p->stream));
     RET(run_ws_poisson32(p, p->ws_s, p->ws_h, nullptr, false));
   } else {
     LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
            launch_ws_source(p->f, p->g, p->ws_src, P, p->stream));
     RET(run_ws_poisson(p, p->ws_src, p->ws_h));
   }
+  if (!(have & WS_HAVE_C32))
+    LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
+           launch_convert<float>(p->c, 1, p->ws_c32, 0, P, p->stream));
   LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
-         launch_convert<float>(p->c, 1, p->ws_c32, 0, P, p->stream));
-  LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
-         launch_ws_features(p->f, p->g, p->ws_c32, p->ws_h, p->N, p->M, p->ws_X, p->stream));
+         launch_ws_features(p->f, p->g, p->ws_c32, p->ws_h, p->N, p->M, X, p->stream));
   return OT_OK;
 }
 
 // u = alpha (h + P(G MLP(X))), G the Gaussian low-pass; alpha and the network's error flag
 // in sc (stall: the failure-path test hook of the network kernel)
-static int run_warmstart(ot_plan* p, double* u, int stall = 0) {
+static int run_warmstart(ot_plan* p, double* u, int stall = 0, int have = 0) {
   const long P = (long)p->N * p->M;
-  RET(run_ws_features(p));
+  RET(alloc_ws(p));
+  RET(run_ws_features(p, p->ws_X, have));
   LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
          launch_ws_mlp(p->ws_wpack, p->ws_params, p->ws_X, P, p->ws_s, &p->sc->ws_err, p->sms,
                        p->stream, stall));
@@ -1566,9 +1586,7 @@ static int solve_impl(ot_plan* p, const double* f_in, const double* g_in, double
   set_solver_scalars(p);
   CK(cudaMemcpyAsync(p->sc, p->hsc, sizeof(DevScalars), cudaMemcpyHostToDevice, p->stream));
   if (p->translate) {
-    LAUNCH(p, OT_PROF_OTHER, -1, 2,
-           launch_translate_inputs(f_in, g_in, p->f, p->g, N, M, p->partials, p->sc,
-                                   p->stream));
+    RET(run_translate(p, f_in, g_in));
     RET(read_scalars(p));
     if (p->hsc->in_bad) {
       st->status = OT_EINVAL;
@@ -1590,7 +1608,7 @@ static int solve_impl(ot_plan* p, const double* f_in, const double* g_in, double
       return OT_EINVAL;
     }
   }
-  RET(run_prefilter(p, p->g, p->c));
+  RET(run_prefilter(p, p->g, p->c, p->translate));
   if (p->warm_start == 1) {
     if (phi != p->u) CK(cudaMemcpyAsync(p->u, phi, P * 8, cudaMemcpyDeviceToDevice, p->stream));
   } else if (p->warm_start == 2) {
@@ -1766,13 +1784,11 @@ static int capture_solve(ot_plan* p) {
   long long k0 = p->launches;
   p->cur_mask = MASK_ALL;
   if (p->translate)
-    LAUNCH(p, OT_PROF_OTHER, -1, 2,
-           launch_translate_inputs(p->f, p->g, p->f, p->g, N, M, p->partials, p->sc,
-                                   p->stream, btc(p)));
+    RET(run_translate(p, p->f, p->g, btc(p)));
   else
     LAUNCH(p, OT_PROF_OTHER, -1, 1,
            launch_input_stats(p->f, p->g, N, M, p->partials, p->sc, p->stream, btc(p)));
-  RET(run_prefilter(p, p->g, p->c));
+  RET(run_prefilter(p, p->g, p->c, p->translate));
   if (p->warm_start == 2) RET(run_warmstart(p, p->u));
   LAUNCH(p, OT_PROF_RESIDUAL, -1, 1,
          residual_launch<T>(p, p->f, p->c, p->u, p->Fraw, p->ucand, 0));
@@ -2537,30 +2553,35 @@ extern "C" int ot_ws_save_weights(const char* path, const float* params_host, in
   return ok ? OT_OK : OT_EINVAL;
 }
 
-// translate (or copy) the inputs into the plan's f, g and prefilter g
-static int ws_prepare_inputs(ot_plan* p, const double* f, const double* g) {
+// translate (or copy) the inputs into the plan's f, g and prefilter g; *have (mixed mode, one
+// problem): what run_ws_features finds done, its source and the coefficients' FP32 copy
+static int ws_prepare_inputs(ot_plan* p, const double* f, const double* g, int* have) {
   const long P = (long)p->N * p->M;
+  RET(alloc_ws(p));
+  const bool one = p->precision && !p->slab_base;
+  float* src = one && p->translate ? p->ws_s : nullptr;
+  float* c32 = one && !p->interp ? p->ws_c32 : nullptr;
+  *have = (src ? WS_HAVE_SOURCE : 0) | (c32 ? WS_HAVE_C32 : 0);
   set_solver_scalars(p);
   CK(cudaMemcpyAsync(p->sc, p->hsc, sizeof(DevScalars), cudaMemcpyHostToDevice, p->stream));
   if (p->translate) {
-    LAUNCH(p, OT_PROF_OTHER, -1, 2,
-           launch_translate_inputs(f, g, p->f, p->g, p->N, p->M, p->partials, p->sc,
-                                   p->stream));
+    RET(run_translate(p, f, g, Bat(), src));
     RET(read_scalars(p));
     if (p->hsc->in_bad) return OT_EINVAL;
   } else {
     CK(cudaMemcpyAsync(p->f, f, P * 8, cudaMemcpyDeviceToDevice, p->stream));
     CK(cudaMemcpyAsync(p->g, g, P * 8, cudaMemcpyDeviceToDevice, p->stream));
   }
-  return run_prefilter(p, p->g, p->c);
+  return run_prefilter(p, p->g, p->c, p->translate, c32);
 }
 
 extern "C" int ot_ws_predict(ot_plan* p, const double* f, const double* g, double* phi0,
                              double* alpha_out) {
   if (!p || !p->ready || !f || !g || !phi0 || !p->ws_have) return OT_EINVAL;
   CK(cudaSetDevice(p->device));
-  RET(ws_prepare_inputs(p, f, g));
-  RET(run_warmstart(p, phi0));
+  int have = 0;
+  RET(ws_prepare_inputs(p, f, g, &have));
+  RET(run_warmstart(p, phi0, 0, have));
   RET(read_scalars(p));
   if (alpha_out) *alpha_out = p->hsc->ws_alpha;
   if (p->hsc->ws_err) {
@@ -2575,13 +2596,24 @@ extern "C" int ot_ws_features(ot_plan* p, const double* f, const double* g,
   if (!p || !p->ready || !f || !g || !X || (phi_star && !target)) return OT_EINVAL;
   CK(cudaSetDevice(p->device));
   const long P = (long)p->N * p->M;
-  RET(ws_prepare_inputs(p, f, g));
-  RET(run_ws_features(p));
-  CK(cudaMemcpyAsync(X, p->ws_X, P * OTGB_WS_K * sizeof(float), cudaMemcpyDeviceToDevice,
-                     p->stream));
-  if (phi_star)
-    LAUNCH(p, OT_PROF_WARMSTART, -1, 2,
-           launch_ws_target(phi_star, p->ws_h, p->N, p->M, p->ws_tmp, target, p->stream));
+  int have = 0;
+  RET(ws_prepare_inputs(p, f, g, &have));
+  // straight into the caller's rows when they can take 16-byte stores
+  const bool direct = ((uintptr_t)X & 15) == 0;
+  RET(run_ws_features(p, direct ? X : p->ws_X, have));
+  if (!direct)
+    CK(cudaMemcpyAsync(X, p->ws_X, P * OTGB_WS_K * sizeof(float), cudaMemcpyDeviceToDevice,
+                       p->stream));
+  if (phi_star) {
+    // (a target over the potential itself goes through a plane of the plan)
+    const bool apart = (const char*)(target + P) <= (const char*)phi_star ||
+                       (const char*)(phi_star + P) <= (const char*)target;
+    float* t = apart ? target : (float*)p->ws_tmp;
+    LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
+           launch_ws_target(phi_star, p->ws_h, p->N, p->M, t, p->stream));
+    if (!apart)
+      CK(cudaMemcpyAsync(target, t, P * sizeof(float), cudaMemcpyDeviceToDevice, p->stream));
+  }
   CK(cudaStreamSynchronize(p->stream));
   return OT_OK;
 }
@@ -3089,8 +3121,7 @@ static int inverse_radius_impl(ot_plan* p, const double* f, const double* g, con
   p->hsc->forcing = 0;
   CK(cudaMemcpyAsync(p->sc, p->hsc, sizeof(DevScalars), cudaMemcpyHostToDevice, p->stream));
   if (p->translate) {
-    LAUNCH(p, OT_PROF_OTHER, -1, 2,
-           launch_translate_inputs(f, g, p->f, p->g, N, M, p->partials, p->sc, p->stream));
+    RET(run_translate(p, f, g));
   } else {
     CK(cudaMemcpyAsync(p->f, f, P * 8, cudaMemcpyDeviceToDevice, p->stream));
     CK(cudaMemcpyAsync(p->g, g, P * 8, cudaMemcpyDeviceToDevice, p->stream));
@@ -3099,7 +3130,7 @@ static int inverse_radius_impl(ot_plan* p, const double* f, const double* g, con
   }
   RET(read_scalars(p));
   if (p->hsc->in_bad) return OT_EINVAL;
-  RET(run_prefilter(p, p->g, p->c));
+  RET(run_prefilter(p, p->g, p->c, p->translate));
   CK(cudaMemcpyAsync(p->u, phi, P * 8, cudaMemcpyDeviceToDevice, p->stream));
   LAUNCH(p, OT_PROF_RESIDUAL, -1, 1,
          residual_launch<T>(p, p->f, p->c, p->u, p->Fraw, nullptr, 0));

@@ -262,20 +262,44 @@ __global__ void k_input_stats(const double* __restrict__ f, const double* __rest
   }
 }
 
+// the translated inputs; in the mixed mode also f as (hi, lo) floats, and for the learned start's
+// features log f - log g with FP32 logarithms: one pass, where the two were passes of their own
+// over f and g (6.0 and 5.4 us at 512x512 beside 6.8 us, cold caches)
 __global__ void k_input_apply(const double* __restrict__ f, const double* __restrict__ g,
-                              double* __restrict__ ft, double* __restrict__ gt, long P,
+                              double* __restrict__ ft, double* __restrict__ gt,
+                              float2* __restrict__ fdd, float* __restrict__ src, long P,
                               const DevScalars* __restrict__ sc, Bat bat) {
   f = badv(f, bat);
   g = badv(g, bat);
   ft = badv(ft, bat);
   gt = badv(gt, bat);
+  fdd = badv(fdd, bat);
   sc = badv(sc, bat);
   if (bskip(sc, bat)) return;
   const double sf = 1.0 - sc->in_mean[0], sg = 1.0 - sc->in_mean[1];
-  for (long p = blockIdx.x * (long)blockDim.x + threadIdx.x; p < P;
-       p += (long)gridDim.x * blockDim.x) {
-    ft[p] = f[p] + sf;
-    gt[p] = g[p] + sg;
+  const long nth = (long)gridDim.x * blockDim.x;
+  for (long p = blockIdx.x * (long)blockDim.x + threadIdx.x; p < P; p += 4 * nth) {
+    double a[4], b[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const bool in = p + k * nth < P;
+      a[k] = in ? f[p + k * nth] : 0.0;
+      b[k] = in ? g[p + k * nth] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const long q = p + k * nth;
+      if (q >= P) break;
+      a[k] += sf;
+      b[k] += sg;
+      ft[q] = a[k];
+      gt[q] = b[k];
+      if (fdd) {
+        const dd v = dd_from_double(a[k]);
+        fdd[q] = make_float2(v.hi, v.lo);
+        if (src) src[q] = logf(v.hi) - logf(dd_from_double(b[k]).hi);
+      }
+    }
   }
 }
 
@@ -317,11 +341,11 @@ cudaError_t launch_stamp(DevScalars* sc, int cls, cudaStream_t st) {
 
 cudaError_t launch_translate_inputs(const double* f, const double* g, double* ft, double* gt,
                                     int N, int M, double* partials, DevScalars* sc,
-                                    cudaStream_t st, Bat bat) {
+                                    cudaStream_t st, Bat bat, float2* fdd, float* src) {
   const long P = (long)N * M;
   const dim3 nb = bgrid(dim3(reduce_blocks(P)), bat);
   k_input_stats<<<nb, 256, 0, st>>>(f, g, P, partials, sc, bat);
-  k_input_apply<<<nb, 256, 0, st>>>(f, g, ft, gt, P, sc, bat);
+  k_input_apply<<<nb, 256, 0, st>>>(f, g, ft, gt, fdd, src, P, sc, bat);
   return cudaGetLastError();
 }
 

@@ -307,10 +307,13 @@ cudaError_t launch_row_c2r_update_dd(const ddc* q, const double* u_in, double* u
 // c = cubic B-spline coefficients of g (periodic), by recursive filters along y then x
 // (scratch: N x M FP64); cdd (optional) also receives c as (hi, lo) float pairs
 cudaError_t launch_prefilter(const double* g, double* scratch, double* c, float2* cdd, int N,
-                             int M, cudaStream_t st, Bat bat = Bat());
+                             int M, cudaStream_t st, Bat bat = Bat(), float* c32 = nullptr);
+// fdd: f translated, as (hi, lo) floats (the mixed mode); src, with fdd and without a batch: the
+// learned start's source log f - log g
 cudaError_t launch_translate_inputs(const double* f, const double* g, double* ft, double* gt,
                                     int N, int M, double* partials, DevScalars* sc,
-                                    cudaStream_t st, Bat bat = Bat());
+                                    cudaStream_t st, Bat bat = Bat(), float2* fdd = nullptr,
+                                    float* src = nullptr);
 // the statistics of f and g alone (means, minima, non-finite counts) for inputs used as given
 // (sc->in_plain must be 1: then in_bad flags a non-positive or non-finite value)
 cudaError_t launch_input_stats(const double* f, const double* g, int N, int M,
@@ -454,8 +457,8 @@ cudaError_t launch_ws_source32(const double* f, const double* g, float* src, lon
 cudaError_t launch_ws_features(const double* f, const double* g, const float* c32,
                                const double* h, int N, int M, float* X, cudaStream_t st);
 // t = (D_xx + D_yy)(phi - h); scratch: N x M FP64
-cudaError_t launch_ws_target(const double* phi, const double* h, int N, int M, double* scratch,
-                             float* t, cudaStream_t st);
+cudaError_t launch_ws_target(const double* phi, const double* h, int N, int M, float* t,
+                             cudaStream_t st);
 // out = (double)s
 cudaError_t launch_ws_widen(const float* s, double* out, long P, cudaStream_t st);
 // u = h + t

@@ -39,7 +39,7 @@ template <> struct Ops<double> {
   }
   static __device__ __forceinline__ double val(double s) { return s; }
   static __device__ __forceinline__ double mem(double v) { return v; }
-  static __device__ __forceinline__ void store(long o, double r, float2*, double* out) {
+  static __device__ __forceinline__ void store(long o, double r, float2*, double* out, float*) {
     out[o] = r;
   }
   static __device__ __forceinline__ double zero() { return 0.0; }
@@ -55,8 +55,10 @@ template <> struct Ops<dd> {
   }
   static __device__ __forceinline__ dd val(float2 s) { return dd{s.x, s.y}; }
   static __device__ __forceinline__ float2 mem(dd v) { return make_float2(v.hi, v.lo); }
-  static __device__ __forceinline__ void store(long o, float2 r, float2* odd, double* out) {
+  static __device__ __forceinline__ void store(long o, float2 r, float2* odd, double* out,
+                                               float* o32) {
     odd[o] = r;
+    if (o32) o32[o] = r.x;
     if (out) out[o] = dd_to_double(dd{r.x, r.y});
   }
   static __device__ __forceinline__ dd zero() { return dd{0.f, 0.f}; }
@@ -67,12 +69,12 @@ template <> struct Ops<dd> {
 };
 
 // One axis.  XPASS: lines are rows (points along x), else columns.  Input: s64, or sdd when it is
-// null; output: out64 and / or odd.
+// null; output: out64 and / or odd, and with odd (without a batch) its high parts in out32.
 template <typename T, bool XPASS>
 __global__ void __launch_bounds__(256)
     k_prefilter(const double* __restrict__ s64, const float2* __restrict__ sdd,
-                float2* __restrict__ odd, double* __restrict__ out64, int N, int M, double z64,
-                double z8, double A64, Bat bat) {
+                float2* __restrict__ odd, double* __restrict__ out64, float* __restrict__ out32,
+                int N, int M, double z64, double z8, double A64, Bat bat) {
   using O = Ops<T>;
   __shared__ typename O::S x[EP][SW];  // [staged point][line]
   __shared__ typename O::S ep[NC][LN], ea[NC][LN];
@@ -136,14 +138,14 @@ __global__ void __launch_bounds__(256)
     const int k = XPASS ? e % TP : e / LN, l2 = XPASS ? e / TP : e % LN;
     if (line0 + l2 >= nlines || p0 + k >= L) continue;
     const typename O::S r = x[HALO + k][l2];
-    O::store((line0 + l2) * ls + (long)(p0 + k) * ps, r, odd, out64);
+    O::store((line0 + l2) * ls + (long)(p0 + k) * ps, r, odd, out64, out32);
   }
 }
 
 }  // namespace
 
 cudaError_t launch_prefilter(const double* g, double* scratch, double* c, float2* cdd, int N,
-                             int M, cudaStream_t st, Bat bat) {
+                             int M, cudaStream_t st, Bat bat, float* c32) {
   const double z = sqrt(3.0) - 2.0, z2 = z * z, z4 = z2 * z2, z8 = z4 * z4;
   const double A = 6.0 * z / (z2 - 1.0);
   // columns (along y), then rows (along x)
@@ -151,13 +153,14 @@ cudaError_t launch_prefilter(const double* g, double* scratch, double* c, float2
   const dim3 gx = bgrid(dim3((N + LN - 1) / LN, (M + TP - 1) / TP), bat);
   if (cdd) {
     float2* mid = reinterpret_cast<float2*>(scratch);
-    k_prefilter<dd, false><<<gy, 256, 0, st>>>(g, nullptr, mid, nullptr, N, M, z, z8, A, bat);
-    k_prefilter<dd, true><<<gx, 256, 0, st>>>(nullptr, mid, cdd, c, N, M, z, z8, A, bat);
+    k_prefilter<dd, false><<<gy, 256, 0, st>>>(g, nullptr, mid, nullptr, nullptr, N, M, z, z8, A,
+                                               bat);
+    k_prefilter<dd, true><<<gx, 256, 0, st>>>(nullptr, mid, cdd, c, c32, N, M, z, z8, A, bat);
   } else {
-    k_prefilter<double, false><<<gy, 256, 0, st>>>(g, nullptr, nullptr, scratch, N, M, z, z8, A,
-                                                   bat);
-    k_prefilter<double, true><<<gx, 256, 0, st>>>(scratch, nullptr, nullptr, c, N, M, z, z8, A,
-                                                  bat);
+    k_prefilter<double, false><<<gy, 256, 0, st>>>(g, nullptr, nullptr, scratch, nullptr, N, M, z, z8,
+                                                   A, bat);
+    k_prefilter<double, true><<<gx, 256, 0, st>>>(scratch, nullptr, nullptr, c, nullptr, N, M, z, z8,
+                                                  A, bat);
   }
   return cudaGetLastError();
 }

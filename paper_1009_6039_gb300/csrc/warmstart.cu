@@ -36,36 +36,6 @@ __device__ __forceinline__ int wrap_near(int a, int L) {
   return a < 0 ? a + L : (a >= L ? a - L : a);
 }
 
-// 4th-order centred stencils of a periodic FP64 field (spacing 1/M along j, 1/N along i),
-// at grid points 0 <= i < N, 0 <= j < M
-struct Stencil {
-  const double* u;
-  int N, M;
-  __device__ double at(int i, int j) const {
-    return u[(size_t)wrap_near(i, N) * M + wrap_near(j, M)];
-  }
-  __device__ double dx(int i, int j) const {
-    return (-at(i, j + 2) + 8.0 * at(i, j + 1) - 8.0 * at(i, j - 1) + at(i, j - 2)) *
-           (double)M / 12.0;
-  }
-  __device__ double dy(int i, int j) const {
-    return (-at(i + 2, j) + 8.0 * at(i + 1, j) - 8.0 * at(i - 1, j) + at(i - 2, j)) *
-           (double)N / 12.0;
-  }
-  __device__ double dxx(int i, int j) const {
-    return (-at(i, j + 2) + 16.0 * at(i, j + 1) - 30.0 * at(i, j) + 16.0 * at(i, j - 1) -
-            at(i, j - 2)) * (double)M * (double)M / 12.0;
-  }
-  __device__ double dyy(int i, int j) const {
-    return (-at(i + 2, j) + 16.0 * at(i + 1, j) - 30.0 * at(i, j) + 16.0 * at(i - 1, j) -
-            at(i - 2, j)) * (double)N * (double)N / 12.0;
-  }
-  __device__ double dxy(int i, int j) const {
-    return (-dy(i, j + 2) + 8.0 * dy(i, j + 1) - 8.0 * dy(i, j - 1) + dy(i, j - 2)) *
-           (double)M / 12.0;
-  }
-};
-
 // log f - log g with FP32 logarithms (h only seeds the features and the warm start)
 template <typename T>
 __global__ void k_ws_source(const double* __restrict__ f, const double* __restrict__ g,
@@ -76,28 +46,32 @@ __global__ void k_ws_source(const double* __restrict__ f, const double* __restri
 }
 
 // ---------------------------------------------------------------------------------------
-// Tiled stencils in double-float arithmetic: a block of 256 threads owns a 32 x 32 tile of
-// grid points (4 rows per thread) and stages the field with a halo of 2 (as dd) and its
+// Tiled stencils in double-float arithmetic: a block of 256 threads owns a tile of TH x 32
+// grid points (TH / 8 rows per thread) and stages the field with a halo of 2 (as dd) and its
 // unscaled y-differences in shared memory.
 // ---------------------------------------------------------------------------------------
-constexpr int TW = 32, TRPT = 4;
+constexpr int TW = 32;
+template <int TH>
 struct TileDD {
-  dd t[TW + 4][TW + 4];
-  dd dy[TW][TW + 4];
+  dd t[TH + 4][TW + 4];
+  dd dy[TH][TW + 4];
 };
 struct StencilK {
   dd Mh, Nh, Mh2, Nh2, MNh;  // M/12, N/12, M^2/12, N^2/12, MN/144
 };
 
-__device__ void tile_load_dd(TileDD& T, const double* __restrict__ u, int N, int M, int by,
+template <int TH>
+__device__ void tile_load_dd(TileDD<TH>& T, const double* __restrict__ u, int N, int M, int by,
                              int bx) {
-  for (int idx = threadIdx.x; idx < (TW + 4) * (TW + 4); idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < (TH + 4) * (TW + 4); idx += blockDim.x) {
     const int r = idx / (TW + 4), cc = idx - r * (TW + 4);
-    const int gi = wrap_near(by + r - 2, N), gj = wrap_near(bx + cc - 2, M);
+    int gi = wrap_near(by + r - 2, N), gj = wrap_near(bx + cc - 2, M);
+    if (gi >= N) gi %= N;  // (a grid smaller than the tile)
+    if (gj >= M) gj %= M;
     T.t[r][cc] = dd_from_double(u[(size_t)gi * M + gj]);
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < TW * (TW + 4); idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < TH * (TW + 4); idx += blockDim.x) {
     const int r = idx / (TW + 4), cc = idx - r * (TW + 4);
     T.dy[r][cc] = dd_sub(dd_scale2(dd_sub(T.t[r + 3][cc], T.t[r + 1][cc]), 8.0f),
                          dd_sub(T.t[r + 4][cc], T.t[r][cc]));
@@ -106,7 +80,8 @@ __device__ void tile_load_dd(TileDD& T, const double* __restrict__ u, int N, int
 }
 
 // 4th-order stencils at tile point (ty, tx)
-__device__ __forceinline__ void tile_stencils_dd(const TileDD& T, int ty, int tx,
+template <int TH>
+__device__ __forceinline__ void tile_stencils_dd(const TileDD<TH>& T, int ty, int tx,
                                                  const StencilK& K, dd* ux, dd* uy, dd* uxx,
                                                  dd* uyy, dd* uxy) {
   const int r = ty + 2, q = tx + 2;
@@ -158,18 +133,19 @@ __device__ __forceinline__ void cubic_bspline_f(float t, float w[4], float dw[4]
 //   10 hx, 10 hy, 0.1 Gx / Gc, 0.1 Gy / Gc, (Gx hx + Gy hy) / Gc, (hxx - hyy)^2 + 4 hxy^2,
 //   r (hxx + hyy), 0],   Gc = max(G, floor), lg = log Gc, ld = log max(det, floor),
 // G, Gx, Gy the interpolant of g at T = x + grad h, det = det(I + D^2 h).
+template <int TH>
 __global__ void __launch_bounds__(256)
     k_ws_features(const double* __restrict__ f, const double* __restrict__ g,
                   const float* __restrict__ c32, const double* __restrict__ h, int N, int M,
                   StencilK K, float* __restrict__ X) {
-  __shared__ TileDD T;
-  const int bx = blockIdx.x * TW, by = blockIdx.y * TW;
+  __shared__ TileDD<TH> T;
+  const int bx = blockIdx.x * TW, by = blockIdx.y * TH;
   tile_load_dd(T, h, N, M, by, bx);
   const int tx = threadIdx.x % TW, ty0 = threadIdx.x / TW;
   const int j = bx + tx;
 #pragma unroll 1
-  for (int rr = 0; rr < TRPT; ++rr) {
-    const int ty = ty0 + rr * (TW / TRPT);
+  for (int rr = 0; rr < TH / 8; ++rr) {
+    const int ty = ty0 + rr * 8;
     const int i = by + ty;
     if (i >= N || j >= M) continue;
     dd ux, uy, uxx, uyy, uxy;
@@ -227,20 +203,31 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// training target s* = (D_xx + D_yy)(phi - h)
-__global__ void k_ws_target(const double* __restrict__ phi, const double* __restrict__ h,
-                            int N, int M, double* __restrict__ diff, float* __restrict__ t,
-                            int stage) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = blockIdx.y;
-  if (j >= M) return;
-  const size_t p = (size_t)i * M + j;
-  if (stage == 0) {
-    diff[p] = phi[p] - h[p];
-  } else {
-    const Stencil S{diff, N, M};
-    t[p] = (float)(S.dxx(i, j) + S.dyy(i, j));
+// training target s* = (D_xx + D_yy)(phi - h), the difference staged per tile of 8 x 32 points (halo
+// 2): one pass, where the difference went through a plane of its own.  Bound by the FP64 pipe (12
+// instructions per point with the halo's differences)
+__global__ void __launch_bounds__(256)
+    k_ws_target(const double* __restrict__ phi, const double* __restrict__ h, int N, int M,
+                double kx, double ky, float* __restrict__ t) {  // kx = M^2 / 12, ky = N^2 / 12
+  __shared__ double d[8 + 4][TW + 4];
+  const int bx = blockIdx.x * TW, by = blockIdx.y * 8;
+  for (int idx = threadIdx.x; idx < 12 * (TW + 4); idx += 256) {
+    const int r = idx / (TW + 4), cc = idx - r * (TW + 4);
+    const size_t q = (size_t)wrapi(by + r - 2, N) * M + wrapi(bx + cc - 2, M);
+    d[r][cc] = phi[q] - h[q];
   }
+  __syncthreads();
+  const int tx = threadIdx.x % TW, ty = threadIdx.x / TW;
+  const int i = by + ty, j = bx + tx;
+  if (i >= N || j >= M) return;
+  const double* c = &d[ty + 2][tx + 2];
+  constexpr int S = TW + 4;
+  double r = -30.0 * (kx + ky) * c[0];
+  r = fma(16.0 * kx, c[1] + c[-1], r);
+  r = fma(-kx, c[2] + c[-2], r);
+  r = fma(16.0 * ky, c[S] + c[-S], r);
+  r = fma(-ky, c[2 * S] + c[-2 * S], r);
+  t[(size_t)i * M + j] = (float)r;
 }
 
 __global__ void k_ws_widen(const float* __restrict__ s, double* __restrict__ out, long P) {
@@ -263,7 +250,7 @@ __global__ void __launch_bounds__(256)
     k_ws_admissible(const double* __restrict__ u, int N, int M, StencilK K,
                     double* __restrict__ partials, unsigned int* ticket,
                     const int* __restrict__ err, double* alpha) {
-  __shared__ TileDD T;
+  __shared__ TileDD<32> T;
   __shared__ float red[4][8];
   __shared__ bool last;
   const int bx = blockIdx.x * TW, by = blockIdx.y * TW;
@@ -272,8 +259,8 @@ __global__ void __launch_bounds__(256)
   const int tx = threadIdx.x % TW, ty0 = threadIdx.x / TW;
   const int j = bx + tx;
 #pragma unroll 1
-  for (int rr = 0; rr < TRPT; ++rr) {
-    const int ty = ty0 + rr * (TW / TRPT);
+  for (int rr = 0; rr < 4; ++rr) {
+    const int ty = ty0 + rr * 8;
     const int i = by + ty;
     if (i >= N || j >= M) continue;
     dd ux, uy, uxx, uyy, uxy;
@@ -800,7 +787,6 @@ __global__ void k_ws_pack(const float* __restrict__ params, unsigned char* __res
   st_row8(base, row, k0, v);
 }
 
-inline dim3 grid2(int N, int M) { return dim3((M + 127) / 128, N); }
 inline int nblk(long P, int t = 256) {
   long b = (P + t - 1) / t;
   return (int)(b < 4096 ? (b > 0 ? b : 1) : 4096);
@@ -820,21 +806,22 @@ __device__ __forceinline__ dd warp_sum_dd(dd v) {
   return v;
 }
 
+template <int TH>
 __global__ void __launch_bounds__(256)
     k_transport(const double* __restrict__ f, const double* __restrict__ u, int N, int M,
                 StencilK K, double* __restrict__ div, float2* __restrict__ partials,
                 unsigned int* ticket, double* dist) {
-  __shared__ TileDD T;
+  __shared__ TileDD<TH> T;
   __shared__ float2 red[8];
   __shared__ bool last;
-  const int bx = blockIdx.x * TW, by = blockIdx.y * TW;
+  const int bx = blockIdx.x * TW, by = blockIdx.y * TH;
   tile_load_dd(T, u, N, M, by, bx);
   const int tx = threadIdx.x % TW, ty0 = threadIdx.x / TW;
   const int j = bx + tx;
   dd acc = dd{0.f, 0.f};
 #pragma unroll 1
-  for (int rr = 0; rr < TRPT; ++rr) {
-    const int ty = ty0 + rr * (TW / TRPT);
+  for (int rr = 0; rr < TH / 8; ++rr) {
+    const int ty = ty0 + rr * 8;
     const int i = by + ty;
     if (i >= N || j >= M) continue;
     dd ux, uy, uxx, uyy, uxy;
@@ -909,18 +896,28 @@ static StencilK stencil_consts(int N, int M) {
   return K;
 }
 
-static dim3 tiles(int N, int M) { return dim3((M + TW - 1) / TW, (N + TW - 1) / TW); }
+static dim3 tiles(int N, int M, int th) { return dim3((M + TW - 1) / TW, (N + th - 1) / th); }
+// fewer than n tiles of 32 x 32 points
+static bool small_grid(int N, int M, long n) {
+  const dim3 t = tiles(N, M, 32);
+  return (long)t.x * t.y < n;
+}
 
 cudaError_t launch_ws_features(const double* f, const double* g, const float* c32,
                                const double* h, int N, int M, float* X, cudaStream_t st) {
-  k_ws_features<<<tiles(N, M), 256, 0, st>>>(f, g, c32, h, N, M, stencil_consts(N, M), X);
+  // 8-row tiles while the 32-row ones give an SM less than two blocks (a thread's four points follow
+  // each other).  8 / 32 rows, us, one GB300: 5.6 / 11.6 at 128^2, 9.8 / 11.8 at 384^2, 14.5 / 16.1
+  // at 512^2 (256 tiles), 43.8 / 42.4 at 1024^2, 163 / 150 at 2048^2
+  const bool low = small_grid(N, M, 304);
+  auto k = low ? k_ws_features<8> : k_ws_features<32>;
+  k<<<tiles(N, M, low ? 8 : 32), 256, 0, st>>>(f, g, c32, h, N, M, stencil_consts(N, M), X);
   return cudaGetLastError();
 }
 
-cudaError_t launch_ws_target(const double* phi, const double* h, int N, int M, double* scratch,
-                             float* t, cudaStream_t st) {
-  k_ws_target<<<grid2(N, M), 128, 0, st>>>(phi, h, N, M, scratch, t, 0);
-  k_ws_target<<<grid2(N, M), 128, 0, st>>>(phi, h, N, M, scratch, t, 1);
+cudaError_t launch_ws_target(const double* phi, const double* h, int N, int M, float* t,
+                             cudaStream_t st) {
+  k_ws_target<<<tiles(N, M, 8), 256, 0, st>>>(phi, h, N, M, (double)M * M / 12.0,
+                                              (double)N * N / 12.0, t);
   return cudaGetLastError();
 }
 
@@ -939,7 +936,7 @@ int ws_admissible_blocks(int N, int M) { return ((M + TW - 1) / TW) * ((N + TW -
 cudaError_t launch_ws_admissible(double* u, int N, int M, double* partials,
                                  unsigned int* ticket, const int* err, double* alpha,
                                  cudaStream_t st) {
-  k_ws_admissible<<<tiles(N, M), 256, 0, st>>>(u, N, M, stencil_consts(N, M), partials, ticket,
+  k_ws_admissible<<<tiles(N, M, 32), 256, 0, st>>>(u, N, M, stencil_consts(N, M), partials, ticket,
                                                err, alpha);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -951,7 +948,11 @@ cudaError_t launch_ws_admissible(double* u, int N, int M, double* partials,
 cudaError_t launch_transport(const double* f, const double* u, int N, int M, double* div,
                              double* partials, unsigned int* ticket, double* dist,
                              cudaStream_t st) {
-  k_transport<<<tiles(N, M), 256, 0, st>>>(f, u, N, M, stencil_consts(N, M), div,
+  // 8 / 32-row tiles, us: 6.5 / 9.8 at 128^2, 9.2 / 10.0 at 384^2 (144 tiles), 11.9 / 11.7 at 512^2,
+  // 19.3 / 16.3 at 512x1024, 114 / 76 at 2048^2
+  const bool low = small_grid(N, M, 152);
+  auto k = low ? k_transport<8> : k_transport<32>;
+  k<<<tiles(N, M, low ? 8 : 32), 256, 0, st>>>(f, u, N, M, stencil_consts(N, M), div,
                                            reinterpret_cast<float2*>(partials), ticket, dist);
   return cudaGetLastError();
 }
