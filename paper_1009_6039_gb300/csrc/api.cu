@@ -1197,10 +1197,13 @@ static int run_prefilter(ot_plan* p, const double* g, double* c, bool f_split = 
   return OT_OK;
 }
 
-// w = L Lbar^{-1} x, x = V + (*jptr) P scaled by scale[*jptr] when jptr is given
+// w = L Lbar^{-1} x, x = V + (*jptr) P scaled by scale[*jptr] when jptr is given (coef: other
+// coefficient planes than the plan's)
 template <typename T>
 static int run_matvec(ot_plan* p, const T* x, const int* jptr, const double* scale, T* w,
-                      const int* skip, int tag, bool rows_done = false) {
+                      const int* skip, int tag, bool rows_done = false,
+                      const T* coef = nullptr) {
+  if (!coef) coef = (const T*)p->coef;
   const size_t P = (size_t)p->N * p->M;
   const SpecTables& tb = tables<T>(p);
   const DevScalars* msc = p->slab_base ? p->sc : nullptr;
@@ -1214,7 +1217,7 @@ static int run_matvec(ot_plan* p, const T* x, const int* jptr, const double* sca
                           (float2*)p->q2, p->N, p->M, tb, p->sc, skip, p->stream));
     LAUNCH(p, OT_PROF_ROW_C2R_COMBINE, tag, 1,
            launch_mvT_combine((const float2*)p->q0, (const float2*)p->q1,
-                              (const float2*)p->q2, (const float*)p->coef, (float*)w, p->N,
+                              (const float2*)p->q2, (const float*)coef, (float*)w, p->N,
                               p->M, tb, skip, p->stream));
     return OT_OK;
   }
@@ -1227,8 +1230,8 @@ static int run_matvec(ot_plan* p, const T* x, const int* jptr, const double* sca
                        (C2<T>*)p->q2, p->N, p->M, tb, p->sc, skip, p->stream, btc(p)));
   LAUNCH(p, OT_PROF_ROW_C2R_COMBINE, tag, 1,
          launch_row_c2r<T>(ROWINV_COMBINE, (C2<T>*)p->q0, (C2<T>*)p->q1, (C2<T>*)p->q2,
-                           (const T*)p->coef, w, nullptr, nullptr, 0.0, 1.0, p->N, p->M, tb,
-                           skip, p->stream, msc, btc(p)));
+                           coef, w, nullptr, nullptr, 0.0, 1.0, p->N, p->M, tb, skip, p->stream,
+                           msc, btc(p)));
   return OT_OK;
 }
 
@@ -1502,9 +1505,10 @@ static int run_ws_poisson(ot_plan* p, const double* src, double* u, bool lp = fa
 }
 
 // ws_src = log f - log g, ws_h = P(ws_src), X = features at ws_h (f, g, c: the plan's
-// translated densities and B-spline coefficients; have: what ws_prepare_inputs has left)
+// translated densities and B-spline coefficients; have: what ws_prepare_inputs has left; bad, when
+// given: X stays as it is where *bad)
 enum { WS_HAVE_SOURCE = 1, WS_HAVE_C32 = 2 };
-static int run_ws_features(ot_plan* p, float* X, int have = 0) {
+static int run_ws_features(ot_plan* p, float* X, int have = 0, const int* bad = nullptr) {
   RET(alloc_ws(p));
   const long P = (long)p->N * p->M;
   if (p->precision) {
@@ -1522,7 +1526,8 @@ static int run_ws_features(ot_plan* p, float* X, int have = 0) {
     LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
            launch_convert<float>(p->c, 1, p->ws_c32, 0, P, p->stream));
   LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
-         launch_ws_features(p->f, p->g, p->ws_c32, p->ws_h, p->N, p->M, X, p->stream));
+         launch_ws_features(p->f, p->g, p->ws_c32, p->ws_h, p->N, p->M, X, bad,
+                            p->stream));
   return OT_OK;
 }
 
@@ -2422,16 +2427,44 @@ static int upload_abar(ot_plan* p, const double* abar) {
   return OT_OK;
 }
 
+// The caller's planes as the passes' own operands.  In the FP64 mode a plane that can take 16-byte
+// accesses is read or written where it is (a plane copied in or out is 7 us of 172 at 384x768 and
+// 26 of 638 at 2048x2048, one GB300); else it goes through the plan's buffer `own`, as FP32 planes
+// do.  A pass reads its whole input before a later one writes a result, so in-place calls agree
+// (apart: a result clear of an input that the last pass still reads).
+template <typename T>
+static bool plane_direct(const void* x) {
+  return sizeof(T) == 8 && ((uintptr_t)x & 15) == 0;
+}
+template <typename T>
+static int plane_in(ot_plan* p, const double* x, long n, void* own, const T** in) {
+  *in = plane_direct<T>(x) ? (const T*)x : (const T*)own;
+  if (!plane_direct<T>(x)) CK(launch_convert<T>(x, 1, own, sizeof(T) == 8, n, p->stream));
+  return OT_OK;
+}
+template <typename T>
+static T* plane_out(double* x, void* own, bool apart = true) {
+  return plane_direct<T>(x) && apart ? (T*)x : (T*)own;
+}
+template <typename T>
+static int plane_done(ot_plan* p, const T* out, double* x, long n) {
+  if ((const void*)out != (const void*)x)
+    CK(launch_convert<T>(out, sizeof(T) == 8, x, 1, n, p->stream));
+  return OT_OK;
+}
+
 template <typename T>
 static int apply_op_impl(ot_plan* p, const double* coef, const double* abar,
                          const double* sigma, double* w) {
   const long P = (long)p->N * p->M;
   int rc = upload_abar(p, abar);
   if (rc) return rc;
-  CK(launch_convert<T>(coef, 1, p->coef, sizeof(T) == 8, 5 * P, p->stream));
-  CK(launch_convert<T>(sigma, 1, p->sigma, sizeof(T) == 8, P, p->stream));
-  RET(run_matvec<T>(p, (const T*)p->sigma, nullptr, nullptr, (T*)p->w, nullptr, -1));
-  CK(launch_convert<T>(p->w, sizeof(T) == 8, w, 1, P, p->stream));
+  const T *cf, *sg;
+  RET(plane_in<T>(p, coef, 5 * P, p->coef, &cf));
+  RET(plane_in<T>(p, sigma, P, p->sigma, &sg));
+  T* out = plane_out<T>(w, p->w, w + P <= coef || coef + 5 * P <= w);
+  RET(run_matvec<T>(p, sg, nullptr, nullptr, out, nullptr, -1, false, cf));
+  RET(plane_done<T>(p, out, w, P));
   CK(cudaStreamSynchronize(p->stream));
   return OT_OK;
 }
@@ -2449,9 +2482,11 @@ static int lbar_impl(ot_plan* p, const double* abar, const double* sigma, double
   const long P = (long)p->N * p->M;
   int rc = upload_abar(p, abar);
   if (rc) return rc;
-  CK(launch_convert<T>(sigma, 1, p->sigma, sizeof(T) == 8, P, p->stream));
-  RET(run_lbar_inv<T>(p, (const T*)p->sigma, nullptr, nullptr, 0.0, (T*)p->w));
-  CK(launch_convert<T>(p->w, sizeof(T) == 8, theta, 1, P, p->stream));
+  const T* sg;
+  RET(plane_in<T>(p, sigma, P, p->sigma, &sg));
+  T* out = plane_out<T>(theta, p->w);
+  RET(run_lbar_inv<T>(p, sg, nullptr, nullptr, 0.0, out));
+  RET(plane_done<T>(p, out, theta, P));
   CK(cudaStreamSynchronize(p->stream));
   return OT_OK;
 }
@@ -2468,12 +2503,14 @@ template <typename T>
 static int fft_fwd_impl(ot_plan* p, const double* x, double* spec) {
   const long P = (long)p->N * p->M;
   const SpecTables& tb = tables<T>(p);
-  CK(launch_convert<T>(x, 1, p->sigma, sizeof(T) == 8, P, p->stream));
-  CK(launch_row_r2c<T>((const T*)p->sigma, 0, nullptr, nullptr, (C2<T>*)p->spec, p->N, p->M,
-                       tb, nullptr, p->stream));
-  CK(launch_col<T>(COL_FWD, (C2<T>*)p->spec, (C2<T>*)p->q0, nullptr, nullptr, p->N, p->M, tb,
+  const T* in;
+  RET(plane_in<T>(p, x, P, p->sigma, &in));
+  T* out = plane_out<T>(spec, p->q0);
+  CK(launch_row_r2c<T>(in, 0, nullptr, nullptr, (C2<T>*)p->spec, p->N, p->M, tb, nullptr,
+                       p->stream));
+  CK(launch_col<T>(COL_FWD, (C2<T>*)p->spec, (C2<T>*)out, nullptr, nullptr, p->N, p->M, tb,
                    nullptr, nullptr, p->stream));
-  CK(launch_convert<T>(p->q0, sizeof(T) == 8, spec, 1, P, p->stream));
+  RET(plane_done<T>(p, out, spec, P));
   CK(cudaStreamSynchronize(p->stream));
   return OT_OK;
 }
@@ -2482,12 +2519,14 @@ template <typename T>
 static int fft_inv_impl(ot_plan* p, const double* spec, double* x) {
   const long P = (long)p->N * p->M;
   const SpecTables& tb = tables<T>(p);
-  CK(launch_convert<T>(spec, 1, p->spec, sizeof(T) == 8, P, p->stream));
-  CK(launch_col<T>(COL_INV, (C2<T>*)p->spec, (C2<T>*)p->q0, nullptr, nullptr, p->N, p->M, tb,
+  const T* in;
+  RET(plane_in<T>(p, spec, P, p->spec, &in));
+  T* out = plane_out<T>(x, p->w);
+  CK(launch_col<T>(COL_INV, (const C2<T>*)in, (C2<T>*)p->q0, nullptr, nullptr, p->N, p->M, tb,
                    nullptr, nullptr, p->stream));
-  CK(launch_row_c2r<T>(ROWINV_PLAIN, (C2<T>*)p->q0, nullptr, nullptr, nullptr, (T*)p->w,
-                       nullptr, nullptr, 0.0, 1.0, p->N, p->M, tb, nullptr, p->stream));
-  CK(launch_convert<T>(p->w, sizeof(T) == 8, x, 1, P, p->stream));
+  CK(launch_row_c2r<T>(ROWINV_PLAIN, (C2<T>*)p->q0, nullptr, nullptr, nullptr, out, nullptr,
+                       nullptr, 0.0, 1.0, p->N, p->M, tb, nullptr, p->stream));
+  RET(plane_done<T>(p, out, x, P));
   CK(cudaStreamSynchronize(p->stream));
   return OT_OK;
 }
@@ -2555,7 +2594,9 @@ extern "C" int ot_ws_save_weights(const char* path, const float* params_host, in
 
 // translate (or copy) the inputs into the plan's f, g and prefilter g; *have (mixed mode, one
 // problem): what run_ws_features finds done, its source and the coefficients' FP32 copy
-static int ws_prepare_inputs(ot_plan* p, const double* f, const double* g, int* have) {
+// (late: the caller reads the verdict on the inputs itself)
+static int ws_prepare_inputs(ot_plan* p, const double* f, const double* g, int* have,
+                             bool late = false) {
   const long P = (long)p->N * p->M;
   RET(alloc_ws(p));
   const bool one = p->precision && !p->slab_base;
@@ -2566,8 +2607,10 @@ static int ws_prepare_inputs(ot_plan* p, const double* f, const double* g, int* 
   CK(cudaMemcpyAsync(p->sc, p->hsc, sizeof(DevScalars), cudaMemcpyHostToDevice, p->stream));
   if (p->translate) {
     RET(run_translate(p, f, g, Bat(), src));
-    RET(read_scalars(p));
-    if (p->hsc->in_bad) return OT_EINVAL;
+    if (!late) {
+      RET(read_scalars(p));
+      if (p->hsc->in_bad) return OT_EINVAL;
+    }
   } else {
     CK(cudaMemcpyAsync(p->f, f, P * 8, cudaMemcpyDeviceToDevice, p->stream));
     CK(cudaMemcpyAsync(p->g, g, P * 8, cudaMemcpyDeviceToDevice, p->stream));
@@ -2596,23 +2639,31 @@ extern "C" int ot_ws_features(ot_plan* p, const double* f, const double* g,
   if (!p || !p->ready || !f || !g || !X || (phi_star && !target)) return OT_EINVAL;
   CK(cudaSetDevice(p->device));
   const long P = (long)p->N * p->M;
-  int have = 0;
-  RET(ws_prepare_inputs(p, f, g, &have));
-  // straight into the caller's rows when they can take 16-byte stores
+  // Straight into the caller's rows when they can take 16-byte stores, and a target over the
+  // potential itself through a plane of the plan.  With no copy of either, the verdict on the
+  // inputs is read at the end (one wait instead of two): the kernels leave X and target alone
+  // when the inputs were refused.
   const bool direct = ((uintptr_t)X & 15) == 0;
-  RET(run_ws_features(p, direct ? X : p->ws_X, have));
+  const bool apart = !phi_star || (const char*)(target + P) <= (const char*)phi_star ||
+                     (const char*)(phi_star + P) <= (const char*)target;
+  const bool late = direct && apart && p->translate;
+  const int* bad = late ? &p->sc->in_bad : nullptr;
+  int have = 0;
+  RET(ws_prepare_inputs(p, f, g, &have, late));
+  RET(run_ws_features(p, direct ? X : p->ws_X, have, bad));
   if (!direct)
     CK(cudaMemcpyAsync(X, p->ws_X, P * OTGB_WS_K * sizeof(float), cudaMemcpyDeviceToDevice,
                        p->stream));
   if (phi_star) {
-    // (a target over the potential itself goes through a plane of the plan)
-    const bool apart = (const char*)(target + P) <= (const char*)phi_star ||
-                       (const char*)(phi_star + P) <= (const char*)target;
     float* t = apart ? target : (float*)p->ws_tmp;
     LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
-           launch_ws_target(phi_star, p->ws_h, p->N, p->M, t, p->stream));
+           launch_ws_target(phi_star, p->ws_h, p->N, p->M, t, bad, p->stream));
     if (!apart)
       CK(cudaMemcpyAsync(target, t, P * sizeof(float), cudaMemcpyDeviceToDevice, p->stream));
+  }
+  if (late) {
+    RET(read_scalars(p));
+    return p->hsc->in_bad ? OT_EINVAL : OT_OK;
   }
   CK(cudaStreamSynchronize(p->stream));
   return OT_OK;
@@ -2622,16 +2673,14 @@ extern "C" int ot_ws_mlp_forward(ot_plan* p, const float* X, int64_t rows, float
   if (!p || !p->ready || !p->ws_have || rows < 0 || (rows > 0 && (!X || !out)))
     return OT_EINVAL;
   CK(cudaSetDevice(p->device));
-  CK(cudaMemsetAsync(&p->sc->ws_err, 0, sizeof(int), p->stream));
+  p->hsc->ws_err = 0;  // (pinned: the kernel writes it through, and only when a wait runs out)
   const int stall = p->ws_stall;
   p->ws_stall = 0;
   LAUNCH(p, OT_PROF_WARMSTART, -1, 1,
-         launch_ws_mlp(p->ws_wpack, p->ws_params, X, rows, out, &p->sc->ws_err, p->sms,
+         launch_ws_mlp(p->ws_wpack, p->ws_params, X, rows, out, &p->hsc->ws_err, p->sms,
                        p->stream, stall));
-  int err = 0;
-  CK(cudaMemcpyAsync(&err, &p->sc->ws_err, sizeof(int), cudaMemcpyDeviceToHost, p->stream));
   CK(cudaStreamSynchronize(p->stream));
-  if (err) {
+  if (p->hsc->ws_err) {
     record_kernel_error("tensor-core network: bounded mbarrier wait ran out", __LINE__);
     return OT_ETIMEOUT;
   }
@@ -2644,9 +2693,9 @@ extern "C" int ot_transport_outputs(ot_plan* p, const double* f, const double* p
   CK(cudaSetDevice(p->device));
   LAUNCH(p, OT_PROF_OTHER, -1, 1,
          launch_transport(f, phi, p->N, p->M, div_out, p->partials,
-                          &p->sc->ticket[TK_TRANSPORT], &p->sc->dist, p->stream));
-  CK(cudaMemcpyAsync(dist, &p->sc->dist, sizeof(double), cudaMemcpyDeviceToHost, p->stream));
+                          &p->sc->ticket[TK_TRANSPORT], &p->hsc->dist, p->stream));
   CK(cudaStreamSynchronize(p->stream));
+  *dist = p->hsc->dist;  // (pinned: the kernel writes it through)
   return OT_OK;
 }
 
@@ -2664,6 +2713,7 @@ struct ot_ws_trainer {
   cudaStream_t stream = 0;
   float *params = nullptr, *m = nullptr, *v = nullptr;
   WsTrainBuffers b{};
+  char* host = nullptr;  // pinned: a loss, and a gradient 16 bytes on
   std::vector<void*> allocs;
 };
 
@@ -2671,6 +2721,7 @@ extern "C" void ot_ws_trainer_destroy(ot_ws_trainer* tr) {
   if (!tr) return;
   cudaSetDevice(tr->device);
   for (void* q : tr->allocs) cudaFree(q);
+  if (tr->host) cudaFreeHost(tr->host);
   delete tr;
 }
 
@@ -2701,6 +2752,7 @@ extern "C" int ot_ws_trainer_create(ot_ws_trainer** out, int32_t batch,
   tr->v = (float*)get(n * 4);
   WsTrainBuffers& b = tr->b;
   b.grad = (float*)get(n * 4);
+  if (cudaMallocHost(&tr->host, 16 + n * 4) != cudaSuccess) failed = true;
   b.sms = 0;
   cudaDeviceGetAttribute(&b.sms, cudaDevAttrMultiProcessorCount, tr->device);
   if (b.sms < 1) b.sms = 148;
@@ -2733,13 +2785,14 @@ extern "C" int ot_ws_trainer_grad(ot_ws_trainer* tr, const float* X, const float
                                   const int64_t* idx, float* grad_host, double* loss_host) {
   if (!tr || !X || !t || !idx) return OT_EINVAL;
   CK(cudaSetDevice(tr->device));
-  CK(launch_ws_grad(tr->params, X, t, (const long long*)idx, tr->B, tr->b, tr->stream));
-  if (grad_host)
-    CK(cudaMemcpyAsync(grad_host, tr->b.grad, ws_param_count() * 4, cudaMemcpyDeviceToHost,
-                       tr->stream));
-  if (loss_host)
-    CK(cudaMemcpyAsync(loss_host, tr->b.loss, 8, cudaMemcpyDeviceToHost, tr->stream));
+  // the sums go straight to pinned memory
+  WsTrainBuffers b = tr->b;
+  b.loss = (double*)tr->host;
+  b.grad = (float*)(tr->host + 16);
+  CK(launch_ws_grad(tr->params, X, t, (const long long*)idx, tr->B, b, tr->stream));
   CK(cudaStreamSynchronize(tr->stream));
+  if (grad_host) memcpy(grad_host, b.grad, ws_param_count() * 4);
+  if (loss_host) *loss_host = *b.loss;
   return OT_OK;
 }
 
@@ -2747,13 +2800,15 @@ extern "C" int ot_ws_trainer_step(ot_ws_trainer* tr, const float* X, const float
                                   const int64_t* idx, float lr, double* loss_host) {
   if (!tr || !X || !t || !idx || !(lr > 0.f)) return OT_EINVAL;
   CK(cudaSetDevice(tr->device));
-  CK(launch_ws_grad(tr->params, X, t, (const long long*)idx, tr->B, tr->b, tr->stream));
+  WsTrainBuffers b = tr->b;
+  if (loss_host) b.loss = (double*)tr->host;  // (else nothing waits for the step)
+  CK(launch_ws_grad(tr->params, X, t, (const long long*)idx, tr->B, b, tr->stream));
   tr->t += 1;
   CK(launch_ws_adam(tr->params, tr->m, tr->v, tr->b.grad, ws_param_count(), lr, tr->t,
                     tr->stream));
   if (loss_host) {
-    CK(cudaMemcpyAsync(loss_host, tr->b.loss, 8, cudaMemcpyDeviceToHost, tr->stream));
     CK(cudaStreamSynchronize(tr->stream));
+    *loss_host = *b.loss;
   }
   return OT_OK;
 }

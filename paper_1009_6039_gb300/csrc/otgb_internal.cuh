@@ -455,10 +455,11 @@ cudaError_t launch_ws_source32(const double* f, const double* g, float* src, lon
                                cudaStream_t st);
 // c32: FP32 copy of the B-spline coefficients of g
 cudaError_t launch_ws_features(const double* f, const double* g, const float* c32,
-                               const double* h, int N, int M, float* X, cudaStream_t st);
-// t = (D_xx + D_yy)(phi - h); scratch: N x M FP64
+                               const double* h, int N, int M, float* X, const int* bad,
+                               cudaStream_t st);
+// t = (D_xx + D_yy)(phi - h); this and the features write nothing where bad is given and *bad set
 cudaError_t launch_ws_target(const double* phi, const double* h, int N, int M, float* t,
-                             cudaStream_t st);
+                             const int* bad, cudaStream_t st);
 // out = (double)s
 cudaError_t launch_ws_widen(const float* s, double* out, long P, cudaStream_t st);
 // u = h + t

@@ -137,7 +137,8 @@ template <int TH>
 __global__ void __launch_bounds__(256)
     k_ws_features(const double* __restrict__ f, const double* __restrict__ g,
                   const float* __restrict__ c32, const double* __restrict__ h, int N, int M,
-                  StencilK K, float* __restrict__ X) {
+                  StencilK K, float* __restrict__ X, const int* __restrict__ bad) {
+  if (bad && *bad) return;
   __shared__ TileDD<TH> T;
   const int bx = blockIdx.x * TW, by = blockIdx.y * TH;
   tile_load_dd(T, h, N, M, by, bx);
@@ -208,7 +209,9 @@ __global__ void __launch_bounds__(256)
 // instructions per point with the halo's differences)
 __global__ void __launch_bounds__(256)
     k_ws_target(const double* __restrict__ phi, const double* __restrict__ h, int N, int M,
-                double kx, double ky, float* __restrict__ t) {  // kx = M^2 / 12, ky = N^2 / 12
+                double kx, double ky, float* __restrict__ t,  // kx = M^2 / 12, ky = N^2 / 12
+                const int* __restrict__ bad) {
+  if (bad && *bad) return;
   __shared__ double d[8 + 4][TW + 4];
   const int bx = blockIdx.x * TW, by = blockIdx.y * 8;
   for (int idx = threadIdx.x; idx < 12 * (TW + 4); idx += 256) {
@@ -726,7 +729,7 @@ __global__ void __launch_bounds__(128 * WS_CH, 1)
     }
   }
   if (!ok) {
-    if (r == 0 && err) atomicExch(err, 1);
+    if (r == 0 && err) *(volatile int*)err = 1;  // (may be pinned host memory)
     // let an MMA group still in flight finish before its TMEM goes away (bounded; with
     // `stall` nothing is in flight and this wait runs out too)
     if (inflight) bar_wait(bar, phase);
@@ -904,20 +907,22 @@ static bool small_grid(int N, int M, long n) {
 }
 
 cudaError_t launch_ws_features(const double* f, const double* g, const float* c32,
-                               const double* h, int N, int M, float* X, cudaStream_t st) {
+                               const double* h, int N, int M, float* X, const int* bad,
+                               cudaStream_t st) {
   // 8-row tiles while the 32-row ones give an SM less than two blocks (a thread's four points follow
   // each other).  8 / 32 rows, us, one GB300: 5.6 / 11.6 at 128^2, 9.8 / 11.8 at 384^2, 14.5 / 16.1
   // at 512^2 (256 tiles), 43.8 / 42.4 at 1024^2, 163 / 150 at 2048^2
   const bool low = small_grid(N, M, 304);
   auto k = low ? k_ws_features<8> : k_ws_features<32>;
-  k<<<tiles(N, M, low ? 8 : 32), 256, 0, st>>>(f, g, c32, h, N, M, stencil_consts(N, M), X);
+  k<<<tiles(N, M, low ? 8 : 32), 256, 0, st>>>(f, g, c32, h, N, M, stencil_consts(N, M), X,
+                                                   bad);
   return cudaGetLastError();
 }
 
 cudaError_t launch_ws_target(const double* phi, const double* h, int N, int M, float* t,
-                             cudaStream_t st) {
+                             const int* bad, cudaStream_t st) {
   k_ws_target<<<tiles(N, M, 8), 256, 0, st>>>(phi, h, N, M, (double)M * M / 12.0,
-                                              (double)N * N / 12.0, t);
+                                              (double)N * N / 12.0, t, bad);
   return cudaGetLastError();
 }
 
