@@ -12,13 +12,15 @@
 // A plan set's classes run these passes too (Bat), and sizes with a factor 3 ran the generic
 // kernels of 12 elements per thread before.  us per launch, one GB300, 5 problems, generic ->
 // pairs:             row r2c     column       combine      theta column  theta row
-//   128^2            4.6 -> 3.9  13.2 -> 5.5  14.2 -> 5.8   8.2 ->  8.3   6.8 ->  7.1
-//   192^2            7.6 -> 3.6  24.0 -> 6.5  25.2 -> 6.1  17.3 -> 10.2  18.6 ->  6.9
-//   384^2            8.1 -> 4.6  28.6 -> 14.7 30.7 -> 13.9 27.3 -> 24.3  28.0 -> 13.1
-//   512^2            6.7 -> 5.7  28.1 -> 22.1 32.2 -> 18.2 34.2 -> 32.4  19.2 -> 18.4
-// and for a single 384^2 or 1536^2 problem: column 15.2 -> 7.1, 71 -> 46; combine 11.3 -> 5.7,
-// 67 -> 35; theta column 20.7 -> 10.2, 83 -> 73.  Bound by latency below about 10 us, above by
-// shared-memory traffic (a stage reads and writes every element).
+//   128^2            4.6 -> 3.4  13.2 -> 4.6  14.2 -> 4.1   8.2 ->  6.8   6.8 ->  7.2
+//   192^2            7.6 -> 3.2  24.0 -> 4.9  25.2 -> 5.0  17.3 ->  7.6  18.6 ->  7.5
+//   384^2            8.1 -> 4.2  28.6 -> 9.8  30.7 -> 10.7 27.3 -> 17.8  28.0 -> 14.7
+//   512^2            6.7 -> 5.1  28.1 -> 16.0 32.2 -> 12.8 34.2 -> 28.8  19.2 -> 18.1
+// and for a single 384^2 or 1536^2 problem: column 15.2 -> 6.1, 71 -> 41; combine 11.3 -> 5.0,
+// 67 -> 29; theta column 20.7 -> 9.8, 83 -> 71.  Bound by latency below about 10 us, above by
+// shared-memory traffic (a stage reads and writes every element; the first and the last stage keep
+// to registers where values are loaded, computed or stored: at 1024^2 column 17.7 -> 15.9,
+// combine 14.3 -> 11.7, theta column 27.6 -> 25.6 us).
 #pragma once
 #include "f32x2.cuh"
 #include "spectral.cuh"
@@ -114,83 +116,128 @@ __host__ __device__ constexpr int pstage_count() {
     return 0;
 }
 
-// One stage of radix R (span Ns) on NP transform pairs of length L;
-// tw: the stage-ordered twiddles as (w.x, w.x, w.y, w.y) words.  Out of place (one barrier)
-// or in place (INPLACE: the stores wait for every thread's loads).
+// radix of the last stage
+template <int REM> __host__ __device__ constexpr int plast() {
+  if constexpr (REM == pradix<REM>())
+    return REM;
+  else
+    return plast<REM / pradix<REM>()>();
+}
+
+// A stage of radix R (span Ns) on NP transform pairs of length L, in three steps: a thread's slots
+// into registers (R == 3: one butterfly, else 4 / R), their twiddles (tw: the stage-ordered
+// twiddles as (w.x, w.x, w.y, w.y) words) and butterflies, and the results into shared memory.
+// The first stage's slot e is element t + e L / 4 (L / 3 for radix 3), the last stage's slot s
+// ends as element pout(t, s) (sx: see k_col_pair): the first stage can take its values from where they are loaded or
+// computed and the last one leave them to where they are used, without shared memory between.
+template <int R> __host__ __device__ constexpr int pslots() { return R == 3 ? 3 : 4; }
+template <int R, int L> __device__ __forceinline__ bool pactive(int t) {
+  return L % 3 != 0 || R == 3 || t < L / 4;
+}
+template <int R, int L> __device__ __forceinline__ int pout(int t, int s) {
+  return t + (s / R) * (L / 4) + (s % R) * (L / R);
+}
+template <int R, int L, int NP>
+__device__ __forceinline__ void pload(PC* const (&in)[NP], PC (&v)[NP][pslots<R>()], int t,
+                                      int sx = 0) {
+  constexpr int T = R == 3 ? L / 3 : L / 4, LR = L / R;
+#pragma unroll
+  for (int s = 0; s < pslots<R>(); ++s) {
+    const int src = swz(t + (s / R) * T + (s % R) * LR) ^ sx;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) v[q][s] = in[q][src];
+  }
+}
+template <int R, int SIGN, int L, int Ns, int NP>
+__device__ __forceinline__ void pbfly(PC (&v)[NP][pslots<R>()], int t,
+                                      const ulonglong2* __restrict__ tw) {
+  constexpr int T = R == 3 ? L / 3 : L / 4;
+#pragma unroll
+  for (int b = 0; b < pslots<R>() / R; ++b) {
+    if (Ns > 1) {
+      const int k = (int)((unsigned)(t + b * T) % (unsigned)Ns);
+#pragma unroll
+      for (int r = 1; r < R; ++r) {
+        const ulonglong2 w = tw[(Ns - 1) + (r - 1) * Ns + k];
+        const u64 nwy = sub2(0ull, w.y);  // (0, 0) - (w.y, w.y)
+#pragma unroll
+        for (int q = 0; q < NP; ++q)
+          v[q][b * R + r] = cmulp<SIGN>(v[q][b * R + r], w.x, w.y, nwy);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NP; ++q) BflyP<R, SIGN>::run(&v[q][b * R]);
+  }
+}
+template <int R, int L, int Ns, int NP>
+__device__ __forceinline__ void pstore(PC* const (&out)[NP], const PC (&v)[NP][pslots<R>()],
+                                       int t, int sx = 0) {
+  constexpr int T = R == 3 ? L / 3 : L / 4;
+#pragma unroll
+  for (int s = 0; s < pslots<R>(); ++s) {
+    const int j = t + (s / R) * T;
+    const int qd = (int)((unsigned)j / (unsigned)Ns);
+    const int dst = swz(qd * (Ns * R) + (j - qd * Ns) + (s % R) * Ns) ^ sx;
+#pragma unroll
+    for (int q = 0; q < NP; ++q) out[q][dst] = v[q][s];
+  }
+}
+
+// a whole stage: out of place (one barrier), or in place (the stores wait for every thread's loads)
 template <int R, int SIGN, int L, int Ns, int NP, bool INPLACE = false>
 __device__ __forceinline__ void pstage(PC* const (&in)[NP], PC* const (&out)[NP], int t,
-                                       const ulonglong2* __restrict__ tw) {
-  constexpr int NB = R == 3 ? 1 : 4 / R;  // butterflies per thread
-  constexpr int T = R == 3 ? L / 3 : L / 4, LR = L / R;
-  const bool active = L % 3 != 0 || R == 3 || t < T;
-  PC v[NP][NB * R];
-  if (active) {
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      const int j = t + b * T;
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int src = swz(j + r * LR);
-#pragma unroll
-        for (int q = 0; q < NP; ++q) v[q][b * R + r] = in[q][src];
-      }
-    }
-  }
+                                       const ulonglong2* __restrict__ tw, int sx = 0) {
+  const bool active = pactive<R, L>(t);
+  PC v[NP][pslots<R>()];
+  if (active) pload<R, L, NP>(in, v, t, sx);
   if (INPLACE) __syncthreads();
   if (active) {
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      const int j = t + b * T;
-      const int qd = (int)((unsigned)j / (unsigned)Ns);
-      const int k = j - qd * Ns;
-      if (Ns > 1) {
-#pragma unroll
-        for (int r = 1; r < R; ++r) {
-          const ulonglong2 w = tw[(Ns - 1) + (r - 1) * Ns + k];
-          const u64 nwy = sub2(0ull, w.y);  // (0, 0) - (w.y, w.y)
-#pragma unroll
-          for (int q = 0; q < NP; ++q)
-            v[q][b * R + r] = cmulp<SIGN>(v[q][b * R + r], w.x, w.y, nwy);
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < NP; ++q) BflyP<R, SIGN>::run(&v[q][b * R]);
-      const int d = qd * (Ns * R) + k;
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int dst = swz(d + r * Ns);
-#pragma unroll
-        for (int q = 0; q < NP; ++q) out[q][dst] = v[q][b * R + r];
-      }
-    }
+    pbfly<R, SIGN, L, Ns, NP>(v, t, tw);
+    pstore<R, L, Ns, NP>(out, v, t, sx);
   }
   __syncthreads();
 }
 
-// the transform: stages alternating between a and b, starting from a; the result ends in a
-// for an even number of stages, in b for an odd one
-template <int SIGN, int L, int Ns, int REM, int NP, bool FROM_A>
+// the transform's stages behind the first one: alternating between a and b, starting from a; with
+// LAST the last one too, else it is left to the caller (plast_regs)
+template <int SIGN, int L, int Ns, int REM, int NP, bool FROM_A, bool LAST>
 __device__ __forceinline__ void pfft_rec(PC* const (&a)[NP], PC* const (&b)[NP], int t,
-                                         const ulonglong2* __restrict__ tw) {
-  if constexpr (REM > 1) {
-    constexpr int R = pradix<REM>();
+                                         const ulonglong2* __restrict__ tw, int sx = 0) {
+  constexpr int R = pradix<REM>();
+  if constexpr (REM > (LAST ? 1 : R)) {
     if constexpr (FROM_A)
-      pstage<R, SIGN, L, Ns, NP>(a, b, t, tw);
+      pstage<R, SIGN, L, Ns, NP>(a, b, t, tw, sx);
     else
-      pstage<R, SIGN, L, Ns, NP>(b, a, t, tw);
-    pfft_rec<SIGN, L, Ns * R, REM / R, NP, !FROM_A>(a, b, t, tw);
+      pstage<R, SIGN, L, Ns, NP>(b, a, t, tw, sx);
+    pfft_rec<SIGN, L, Ns * R, REM / R, NP, !FROM_A, LAST>(a, b, t, tw, sx);
   }
 }
-
-// the same transform in place
+// the same in place, without the last stage
 template <int SIGN, int L, int Ns, int REM, int NP>
 __device__ __forceinline__ void pfft_inplace(PC* const (&a)[NP], int t,
                                              const ulonglong2* __restrict__ tw) {
-  if constexpr (REM > 1) {
-    constexpr int R = pradix<REM>();
+  constexpr int R = pradix<REM>();
+  if constexpr (REM > R) {
     pstage<R, SIGN, L, Ns, NP, true>(a, a, t, tw);
     pfft_inplace<SIGN, L, Ns * R, REM / R, NP>(a, t, tw);
   }
+}
+// first stage of the values in v, into out (a barrier)
+template <int SIGN, int L, int NP>
+__device__ __forceinline__ void pfirst_regs(PC (&v)[NP][pelems<L>()], PC* const (&out)[NP], int t,
+                                            int sx = 0) {
+  constexpr int R = pradix<L>();
+  pbfly<R, SIGN, L, 1, NP>(v, t, nullptr);
+  pstore<R, L, 1, NP>(out, v, t, sx);
+  __syncthreads();
+}
+// last stage from shared memory into registers (threads below L / 4 only: pactive)
+template <int SIGN, int L, int NP>
+__device__ __forceinline__ void plast_regs(PC* const (&in)[NP], PC (&v)[NP][4], int t,
+                                           const ulonglong2* __restrict__ tw, int sx = 0) {
+  constexpr int R = plast<L>();
+  pload<R, L, NP>(in, v, t, sx);
+  pbfly<R, SIGN, L, L / R, NP>(v, t, tw);
 }
 
 // the stage table behind the base table of length L
@@ -208,6 +255,15 @@ __device__ __forceinline__ void load_tw4(ulonglong2* tw4, const float2* __restri
     const float2 w = st[i];
     tw4[i] = make_ulonglong2(pk(w.x, w.x), pk(w.y, w.y));
   }
+}
+
+// A column pass takes two column pairs per block where one each would give SMs a second block: half
+// the blocks with whole sectors (k_col_pair) then, else every SM counts.  Column pass, us, one /
+// two pairs per block, one GB300: 512^2 (128 pairs) 7.4 / 8.4, 1024x512 10.9 / 12.9; five of 128^2
+// (160) 5.1 / 4.6, 768^2 (192) 12.5 / 11.0, 512x1024 (256) 9.7 / 8.5; theta's column pass 10.1 / 13.3
+// at 512^2, 23.5 / 17.9 at 768^2, 25.6 / 22.2 at 1024^2.
+inline bool two_pairs(int M, const Bat& bat) {
+  return (long)(M / 4) * (bat.on ? bat.n : 1) > 152;
 }
 
 // the lengths of the pair passes: rows (M / 2) and columns

@@ -25,21 +25,22 @@ __device__ __forceinline__ void st_pair(float2* outa, float2* outb, int k, PC v)
   outb[k] = b;
 }
 
-// the row pair's transform (from P0, scratch P1; buf: where it ends) and its split into the
-// two rows' half spectra: X_k = E + W_M^k O, X_(L-k) = conj(E - W_M^k O) with
+// the row pair's transform of the thread's values v (in P0 and P1) and its split into the two rows' half spectra: X_k = E + W_M^k O, X_(L-k) = conj(E - W_M^k O) with
 // E = (Z_k + conj Z_(L-k)) / 2, O = -i (Z_k - conj Z_(L-k)) / 2, X_0 packed as (X_0, X_L)
 template <int L>
-__device__ __forceinline__ void r2c_pair_transform_split(PC* P0, PC* P1, float2* outa,
-                                                         float2* outb, int t,
+__device__ __forceinline__ void r2c_pair_transform_split(PC (&v)[1][pelems<L>()], PC* P0, PC* P1,
+                                                         float2* outa, float2* outb, int t,
                                                          const ulonglong2* __restrict__ tw4,
                                                          const float2* __restrict__ twM) {
   constexpr int TPT = pthreads<L>();
   {
     PC* const a[1] = {P0};
     PC* const b[1] = {P1};
-    pfft_rec<-1, L, 1, L, 1, true>(a, b, t, tw4);
+    constexpr int R0 = pradix<L>();
+    pfirst_regs<-1, L, 1>(v, a, t);
+    pfft_rec<-1, L, R0, L / R0, 1, true, true>(a, b, t, tw4);
   }
-  const PC* buf = pstage_count<L>() % 2 == 1 ? P1 : P0;
+  const PC* buf = pstage_count<L>() % 2 == 0 ? P1 : P0;
   const u64 half = pk(0.5f, 0.5f), nhalf = pk(-0.5f, -0.5f);
   for (int k = t; k <= L / 2; k += TPT) {
     if (k == 0) {
@@ -104,17 +105,15 @@ __global__ void __launch_bounds__(pthreads<L>())
   load_tw4<L>(tw4, twL, t, TPT);
   const float2* xa = reinterpret_cast<const float2*>(x + (size_t)r0 * M);
   const float2* xb = xa + L;
+  PC v[1][E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int n = t + e * TPT;
     const float2 za = xa[n], zb = xb[n];
-    PC v;
-    v.re = pk(za.x * s, zb.x * s);
-    v.im = pk(za.y * s, zb.y * s);
-    P0[swz(n)] = v;
+    v[0][e].re = pk(za.x * s, zb.x * s);
+    v[0][e].im = pk(za.y * s, zb.y * s);
   }
-  __syncthreads();
-  r2c_pair_transform_split<L>(P0, P1, spec + (size_t)r0 * L, spec + (size_t)(r0 + 1) * L, t,
+  r2c_pair_transform_split<L>(v, P0, P1, spec + (size_t)r0 * L, spec + (size_t)(r0 + 1) * L, t,
                               tw4, twM);
 }
 
@@ -148,6 +147,7 @@ __device__ __forceinline__ void update_r2c_pair_j(float* __restrict__ V,
   const float s = (float)inv_hn;  // the row pass's (float) scale[j + 1]
   const bool next = J < sc->m;    // a next product (block-uniform)
   if (next) load_tw4<L>(tw4, twL, t, TPT);
+  PC v[1][E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int n = t + e * TPT;
@@ -165,16 +165,11 @@ __device__ __forceinline__ void update_r2c_pair_j(float* __restrict__ V,
       reinterpret_cast<float2*>(V + (size_t)(j + 1) * P + ro)[n] = x;
       xr[h] = x;
     }
-    if (next) {
-      PC v;
-      v.re = pk(xr[0].x * s, xr[1].x * s);
-      v.im = pk(xr[0].y * s, xr[1].y * s);
-      P0[swz(n)] = v;
-    }
+    v[0][e].re = pk(xr[0].x * s, xr[1].x * s);
+    v[0][e].im = pk(xr[0].y * s, xr[1].y * s);
   }
   if (!next) return;  // the cycle's last step: no next product
-  __syncthreads();
-  r2c_pair_transform_split<L>(P0, P1, spec + (size_t)r0 * L, spec + (size_t)(r0 + 1) * L, t,
+  r2c_pair_transform_split<L>(v, P0, P1, spec + (size_t)r0 * L, spec + (size_t)(r0 + 1) * L, t,
                               tw4, twM);
 }
 

@@ -11,8 +11,11 @@
 // multiply-adds per part, with the twiddle broadcast to both lanes; the multiplication by
 // +-i exchanges the parts and costs nothing.  A thread holds 4 elements (radix-4 stages,
 // one radix-2 stage for odd powers of two), the length is fixed at compile time
-// (256 ... 2048), and the stages run out of place between two buffer sets (one barrier a
-// stage).  Shared memory is addressed through an XOR swizzle of the 16-byte element index,
+// (96 ... 2048), and the stages run out of place between two buffer sets (one barrier a
+// stage).  The loaded column enters the first stage in registers, the last forward stage's
+// results take the symbols and enter the first inverse stage there (a factor 3 exchanges them
+// once, and columns 0 and M/2 their mirrored entries), and the last stage stores to global
+// memory: 8 passes through shared memory where there were 13.  Shared memory is addressed through an XOR swizzle of the 16-byte element index,
 // i ^ ((i >> 2) & 7), under which every stage's reads and writes of a quarter warp fall in
 // distinct bank groups.  The symbol multiplies are the scalar operations of k_col.
 // (In place on three buffers -- 64 N instead of 112 N bytes, two barriers a stage -- measured the
@@ -24,8 +27,14 @@ namespace {
 
 using namespace pair;
 
-template <int N>
-__global__ void __launch_bounds__(pthreads<N>(), N <= 1024 ? 2 : 1)
+// G column pairs per block, a pair per group of every G-th thread, so that a row's G pairs are read
+// and written by neighbouring threads (G == 2: whole 32-byte sectors; one pair's 16 bytes are half
+// of one, and the kernel waited for them: 1024^2 15.9 -> 12.9 us, 5 problems of 512^2 19.2 -> 16.0).
+// The groups have their own buffers, the second one's swizzled by 4 elements more (sx): the four
+// elements of either group that a quarter warp accesses then lie in distinct bank groups.
+// (G == 4 is no better: 5 of 512^2 18.6 us, 16 of 384^2 24.0 against 25.3.)
+template <int N, int G>
+__global__ void __launch_bounds__(pthreads<N>() * G, N * G <= 1024 ? 2 : 1)
     k_col_pair(const float2* __restrict__ spec, float2* __restrict__ out0,
                float2* __restrict__ out1, float2* __restrict__ out2, int M, float inv,
                const float2* __restrict__ twN, const DevScalars* __restrict__ sc,
@@ -39,14 +48,14 @@ __global__ void __launch_bounds__(pthreads<N>(), N <= 1024 ? 2 : 1)
   skip = badv(skip, bat);
   if ((skip && *skip) || (bat.on && bskip(sc, bat))) return;
   constexpr int TPT = pthreads<N>(), E = pelems<N>();
-  constexpr bool ODD = pstage_count<N>() % 2 == 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ulonglong2* tw4 = reinterpret_cast<ulonglong2*>(smem_raw);
-  PC* pb = reinterpret_cast<PC*>(smem_raw + (size_t)N * sizeof(ulonglong2));
+  const int grp = G == 1 ? 0 : threadIdx.x % G, sx = 8 / G * grp;
+  PC* pb = reinterpret_cast<PC*>(smem_raw + (size_t)N * sizeof(ulonglong2)) + (size_t)grp * 6 * N;
   PC* const P[6] = {pb, pb + N, pb + 2 * N, pb + 3 * N, pb + 4 * N, pb + 5 * N};
   const int Lc = M / 2;
-  const int c0 = 2 * blockIdx.x;
-  const int t = threadIdx.x;
+  const int c0 = 2 * (G * blockIdx.x + grp);
+  const int t = threadIdx.x / G;
 
   // the column pair: one 16-byte load per row, issued before the twiddle table is built so
   // that both sets of loads are in flight together, then regrouped into (re, im) pairs
@@ -54,89 +63,107 @@ __global__ void __launch_bounds__(pthreads<N>(), N <= 1024 ? 2 : 1)
 #pragma unroll
   for (int e = 0; e < E; ++e)
     xs[e] = *reinterpret_cast<const float4*>(spec + (size_t)(t + e * TPT) * Lc + c0);
-  load_tw4<N>(tw4, twN, t, TPT);
+  float2 sy[E];
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    PC v;
-    v.re = pk(xs[e].x, xs[e].z);
-    v.im = pk(xs[e].y, xs[e].w);
-    P[0][swz(t + e * TPT)] = v;
-  }
-  __syncthreads();
-
-  // forward column transforms of both columns (from P0, scratch P3)
-  {
-    PC* const a[1] = {P[0]};
-    PC* const b[1] = {P[3]};
-    pfft_rec<-1, N, 1, N, 1, true>(a, b, t, tw4);
-  }
-  PC* const F = ODD ? P[3] : P[0];
-  // the inverse transforms start in the set that does not hold F
-  PC* const I0 = ODD ? P[0] : P[3];
-  PC* const I1 = ODD ? P[1] : P[4];
-  PC* const I2 = ODD ? P[2] : P[5];
-
+  for (int e = 0; e < E; ++e) sy[e] = symy[t + e * TPT];
+  const float2 sxa = symx[c0], sxb = symx[c0 + 1];
   float ab[5];
 #pragma unroll
   for (int q = 0; q < 5; ++q) ab[q] = sc ? (float)sc->abar[q] : 0.f;
-  const float2 sxa = symx[c0], sxb = symx[c0 + 1];
+  load_tw4<N>(tw4, twN, threadIdx.x, TPT * G);
+
+  // forward column transforms of both columns (in P0 and P3)
+  constexpr int R0 = pradix<N>(), RL = plast<N>();
+  constexpr bool FLIP = pstage_count<N>() % 2 == 1;  // the stages between end in P3
+  const bool last = pactive<RL, N>(t);
+  PC z[1][E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    z[0][e].re = pk(xs[e].x, xs[e].z);
+    z[0][e].im = pk(xs[e].y, xs[e].w);
+  }
+  {
+    PC* const a[1] = {P[0]};
+    PC* const b[1] = {P[3]};
+    pfirst_regs<-1, N, 1>(z, a, t, sx);
+    pfft_rec<-1, N, R0, N / R0, 1, true, false>(a, b, t, tw4, sx);
+  }
+  PC* const F[1] = {FLIP ? P[3] : P[0]};
+  // the exchange of the transformed columns (a set apart from F and from the inverse
+  // transforms' first one): where a thread's slots of the last stage are not those of the first
+  // (a factor 3), and for the mirrored entries of columns 0 and M / 2
+  PC* const X = FLIP ? P[4] : P[1];
+  PC f[1][4];
+  if (last) plast_regs<-1, N, 1>(F, f, t, tw4, sx);
+  if (N % 3 == 0 || blockIdx.x == 0) {
+    if (last) {
+#pragma unroll
+      for (int s = 0; s < 4; ++s) X[swz(pout<RL, N>(t, s)) ^ sx] = f[0][s];
+    }
+    __syncthreads();
+  }
+
+  PC v[3][E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int k = t + e * TPT;
-    const PC z = F[swz(k)];
+    PC zk;
+    if constexpr (N % 3 == 0)
+      zk = X[swz(k) ^ sx];
+    else  // slot s = b RL + r is element t + (b + r 4 / RL) N / 4
+      zk = f[0][RL == 4 ? e : (e & 1) * 2 + (e >> 1)];
     float2 za, zb;
-    upk(z.re, za.x, zb.x);
-    upk(z.im, za.y, zb.y);
-    const float2 sy = symy[k];
+    upk(zk.re, za.x, zb.x);
+    upk(zk.im, za.y, zb.y);
     float2 sa, s0a;
     if (c0 == 0) {
       // the two real columns k1 = 0 and k1 = M/2 carried as X0 + i XL (as in k_col)
-      const PC pz = F[swz((N - k) % N)];
+      const PC pz = X[swz((N - k) % N) ^ sx];
       float2 p, pbv;
       upk(pz.re, p.x, pbv.x);
       upk(pz.im, p.y, pbv.y);
       float2 A = mk2<float>(0.5f * (za.x + p.x), 0.5f * (za.y - p.y));
       float2 B = mk2<float>(0.5f * (za.y + p.y), -0.5f * (za.x - p.x));
-      A = cmul<float>(rho_bar<float>(ab, symx[0], sy), A);
-      B = cmul<float>(rho_bar<float>(ab, symx[M / 2], sy), B);
+      A = cmul<float>(rho_bar<float>(ab, symx[0], sy[e]), A);
+      B = cmul<float>(rho_bar<float>(ab, symx[M / 2], sy[e]), B);
       const float2 Bn = cscale<float>(B, symx[M / 2].y);
       s0a = cscale<float>(mk2<float>(A.x - Bn.y, A.y + Bn.x), inv);
       sa = cscale<float>(mk2<float>(A.x - B.y, A.y + B.x), inv);
     } else {
-      sa = cscale<float>(cmul<float>(rho_bar<float>(ab, sxa, sy), za), inv);
+      sa = cscale<float>(cmul<float>(rho_bar<float>(ab, sxa, sy[e]), za), inv);
       s0a = sa;
     }
-    const float2 sb = cscale<float>(cmul<float>(rho_bar<float>(ab, sxb, sy), zb), inv);
-    const int d = swz(k);
-    PC q;
-    q.re = pk(s0a.x, sb.x);
-    q.im = pk(s0a.y, sb.y);
-    I0[d] = q;
-    q.re = pk(-sy.x * sa.y, -sy.x * sb.y);
-    q.im = pk(sy.x * sa.x, sy.x * sb.x);
-    I1[d] = q;
-    q.re = pk(sa.x * sy.y, sb.x * sy.y);
-    q.im = pk(sa.y * sy.y, sb.y * sy.y);
-    I2[d] = q;
+    const float2 sb = cscale<float>(cmul<float>(rho_bar<float>(ab, sxb, sy[e]), zb), inv);
+    v[0][e].re = pk(s0a.x, sb.x);
+    v[0][e].im = pk(s0a.y, sb.y);
+    v[1][e].re = pk(-sy[e].x * sa.y, -sy[e].x * sb.y);
+    v[1][e].im = pk(sy[e].x * sa.x, sy[e].x * sb.x);
+    v[2][e].re = pk(sa.x * sy[e].y, sb.x * sy[e].y);
+    v[2][e].im = pk(sa.y * sy[e].y, sb.y * sy[e].y);
   }
-  __syncthreads();
 
-  // the three inverse transforms interleaved
-  PC* const ia[3] = {I0, I1, I2};
-  PC* const ib[3] = {ODD ? P[3] : P[0], ODD ? P[4] : P[1], ODD ? P[5] : P[2]};
-  pfft_rec<+1, N, 1, N, 3, true>(ia, ib, t, tw4);
-  PC* const* res = ODD ? ib : ia;
-  float2* const outs[3] = {out0, out1, out2};
+  // the three inverse transforms interleaved, first in the set that does not hold F
+  {
+    PC* const a[3] = {FLIP ? P[0] : P[3], FLIP ? P[1] : P[4], FLIP ? P[2] : P[5]};
+    PC* const b[3] = {FLIP ? P[3] : P[0], FLIP ? P[4] : P[1], FLIP ? P[5] : P[2]};
+    pfirst_regs<+1, N, 3>(v, a, t, sx);
+    pfft_rec<+1, N, R0, N / R0, 3, true, false>(a, b, t, tw4, sx);
+    if (!last) return;
+    PC r[3][4];
+    if constexpr (FLIP)
+      plast_regs<+1, N, 3>(b, r, t, tw4, sx);
+    else
+      plast_regs<+1, N, 3>(a, r, t, tw4, sx);
+    float2* const outs[3] = {out0, out1, out2};
 #pragma unroll
-  for (int o = 0; o < 3; ++o) {
+    for (int o = 0; o < 3; ++o) {
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      const int n = t + e * TPT;
-      const PC v = res[o][swz(n)];
-      float4 x;
-      upk(v.re, x.x, x.z);
-      upk(v.im, x.y, x.w);
-      *reinterpret_cast<float4*>(outs[o] + (size_t)n * Lc + c0) = x;
+      for (int s = 0; s < 4; ++s) {
+        float4 x;
+        upk(r[o][s].re, x.x, x.z);
+        upk(r[o][s].im, x.y, x.w);
+        *reinterpret_cast<float4*>(outs[o] + (size_t)pout<RL, N>(t, s) * Lc + c0) = x;
+      }
     }
   }
 }
@@ -146,8 +173,9 @@ __global__ void __launch_bounds__(pthreads<N>(), N <= 1024 ? 2 : 1)
 // row transforms d_xx Q0, d_x Q0, d_x Q1, Q1, Q2 of two neighbouring rows r0 = 2b and
 // r0 + 1, held side by side as in k_col_pair, weighted by a11, b1, 2 a12, b2, a22 and summed
 // into w = L Lbar^{-1} sigma.  The row symbols, the complex-to-real pre-processing, the
-// transforms and the weighting all run on the packed pairs; the stages run in place (two
-// barriers a stage), which keeps a block at 48 KB of shared memory at length 512, so that
+// transforms and the weighting all run on the packed pairs, the terms, the pre-processing and the
+// first stage in registers, the last stage and the weighting too; the stages between run in place
+// (two barriers a stage), which keeps a block at 48 KB of shared memory at length 512, so that
 // the N / 2 blocks of a 1024 x 1024 grid run in one wave.
 // ---------------------------------------------------------------------------------------
 template <int L>
@@ -203,71 +231,79 @@ __global__ void __launch_bounds__(pthreads<L>(), L <= 512 ? 4 : 2)
     x1.im = pk(a1.y, b1.y);
     x2.re = pk(a2.x, b2.x);
     x2.im = pk(a2.y, b2.y);
-    PC dxx, dx0, dx1;
-    if (k == 0) {
-      dxx.re = 0ull;
-      dxx.im = x0.im;
-      dx0.re = dx0.im = dx1.re = dx1.im = 0ull;
-    } else {
-      const float2 sx = symx[k];
-      const u64 s2 = pk(sx.y, sx.y), s1 = pk(sx.x, sx.x), ns1 = pk(-sx.x, -sx.x);
-      dxx.re = mul2(x0.re, s2);
-      dxx.im = mul2(x0.im, s2);
-      dx0.re = mul2(x0.im, ns1);
-      dx0.im = mul2(x0.re, s1);
-      dx1.re = mul2(x1.im, ns1);
-      dx1.im = mul2(x1.re, s1);
-    }
     const int d = swz(k);
-    B[0][d] = dxx;
-    B[1][d] = dx0;
-    B[2][d] = dx1;
-    B[3][d] = x1;
-    B[4][d] = x2;
+    B[0][d] = x0;
+    B[1][d] = x1;
+    B[2][d] = x2;
   }
   __syncthreads();
 
-  // complex-to-real pre-processing: Z_k = (X_k + conj X_(L-k)) + i (X_k - conj X_(L-k))
-  // conj(W_M^k), Z_(L-k) likewise, each pair (k, L - k) by one thread
-  for (int k = t; k <= L / 2; k += TPT) {
-    if (k == 0) {
-      const int d = swz(0);
+  // The five terms and their complex-to-real pre-processing: Z_k = (X_k + conj X_(L-k)) +
+  // i (X_k - conj X_(L-k)) conj(W_M^k) of each, from the thread's own entries k and the mirrored
+  // ones (both ends of a pair do it: 26 instructions an entry more, and three words read where
+  // the terms themselves were written, read, written and read again)
+  PC z[5][E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int k = t + e * TPT;
+    const int dk = swz(k), dm = swz(e == 0 && t == 0 ? 0 : L - k);
+    PC xk[5], xm[5];
+    xk[0] = B[0][dk];
+    xk[3] = B[1][dk];
+    xk[4] = B[2][dk];
+    xm[0] = B[0][dm];
+    xm[3] = B[1][dm];
+    xm[4] = B[2][dm];
+    if (e == 0 && t == 0) {
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
-        const PC x = B[q][d];
-        PC z;
-        z.re = add2(x.re, x.im);
-        z.im = sub2(x.re, x.im);
-        B[q][d] = z;
+        PC x;
+        if (q < 3) {
+          x.re = 0ull;
+          x.im = q == 0 ? xk[0].im : 0ull;
+        } else {
+          x = xk[q];
+        }
+        z[q][e].re = add2(x.re, x.im);
+        z[q][e].im = sub2(x.re, x.im);
       }
     } else {
-      const float2 w = twM[k];
+      const float2 w = twM[k], sk = symx[k], sm = symx[L - k];
       const u64 wx = pk(w.x, w.x), wy = pk(w.y, w.y), nwy = pk(-w.y, -w.y);
-      const int dk = swz(k), dm = swz(L - k);
+      const u64 k1 = pk(sk.x, sk.x), nk1 = pk(-sk.x, -sk.x), k2 = pk(sk.y, sk.y);
+      const u64 m1 = pk(sm.x, sm.x), nm1 = pk(-sm.x, -sm.x), m2 = pk(sm.y, sm.y);
+      xk[1].re = mul2(xk[0].im, nk1);
+      xk[1].im = mul2(xk[0].re, k1);
+      xm[1].re = mul2(xm[0].im, nm1);
+      xm[1].im = mul2(xm[0].re, m1);
+      xk[2].re = mul2(xk[3].im, nk1);
+      xk[2].im = mul2(xk[3].re, k1);
+      xm[2].re = mul2(xm[3].im, nm1);
+      xm[2].im = mul2(xm[3].re, m1);
+      xk[0].re = mul2(xk[0].re, k2);
+      xk[0].im = mul2(xk[0].im, k2);
+      xm[0].re = mul2(xm[0].re, m2);
+      xm[0].im = mul2(xm[0].im, m2);
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
-        const PC xk = B[q][dk], xm = B[q][dm];
         PC S, D;
-        S.re = add2(xk.re, xm.re);
-        S.im = sub2(xk.im, xm.im);
-        D.re = sub2(xk.re, xm.re);
-        D.im = add2(xk.im, xm.im);
+        S.re = add2(xk[q].re, xm[q].re);
+        S.im = sub2(xk[q].im, xm[q].im);
+        D.re = sub2(xk[q].re, xm[q].re);
+        D.im = add2(xk[q].im, xm[q].im);
         const PC O = cmulp<+1>(D, wx, wy, nwy);
-        PC zk;
-        zk.re = sub2(S.re, O.im);
-        zk.im = add2(S.im, O.re);
-        B[q][dk] = zk;
-        if (2 * k != L) {
-          PC zm;
-          zm.re = add2(S.re, O.im);
-          zm.im = sub2(O.re, S.im);
-          B[q][dm] = zm;
-        }
+        z[q][e].re = sub2(S.re, O.im);
+        z[q][e].im = add2(S.im, O.re);
       }
     }
   }
   __syncthreads();
-  pfft_inplace<+1, L, 1, L, 5>(B, t, tw4);
+  constexpr int R0 = pradix<L>(), RL = plast<L>();
+  pfirst_regs<+1, L, 5>(z, B, t);
+  pfft_inplace<+1, L, R0, L / R0, 5>(B, t, tw4);
+  if (!pactive<RL, L>(t)) return;
+  PC y[5][4];
+  plast_regs<+1, L, 5>(B, y, t, tw4);
 
   // w = a11 y0 + b1 y1 + 2 a12 y2 + b2 y3 + a22 y4 on both rows (the coefficient planes a11,
   // a12, a22, b1, b2 in that order)
@@ -281,14 +317,13 @@ __global__ void __launch_bounds__(pthreads<L>(), L <= 512 ? 4 : 2)
   float2* ov = reinterpret_cast<float2*>(out);
   const u64 two = pk(2.f, 2.f);
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int n = t + e * TPT;
-    const int d = swz(n);
+  for (int e = 0; e < 4; ++e) {
+    const int n = pout<RL, L>(t, e);
     const size_t ia = ra / 2 + n, ib = rb / 2 + n;
     const float2 a11a = c0[ia], a11b = c0[ib], a12a = c1[ia], a12b = c1[ib];
     const float2 a22a = c2[ia], a22b = c2[ib], b1a = c3[ia], b1b = c3[ib];
     const float2 b2a = c4[ia], b2b = c4[ib];
-    const PC y0 = B[0][d], y1 = B[1][d], y2 = B[2][d], y3 = B[3][d], y4 = B[4][d];
+    const PC y0 = y[0][e], y1 = y[1][e], y2 = y[2][e], y3 = y[3][e], y4 = y[4][e];
     u64 rr = mul2(pk(a11a.x, a11b.x), y0.re);
     rr = fma2(pk(b1a.x, b1b.x), y1.re, rr);
     rr = fma2(mul2(two, pk(a12a.x, a12b.x)), y2.re, rr);
@@ -320,17 +355,27 @@ cudaError_t comb_pair_L(const float2* q0, const float2* q1, const float2* q2, co
   return cudaGetLastError();
 }
 
+template <int N, int G>
+cudaError_t col_pair_G(const float2* spec, float2* o0, float2* o1, float2* o2, int M,
+                       const SpecTables& tb, const DevScalars* sc, const int* skip,
+                       cudaStream_t st, Bat bat) {
+  const size_t sm = (size_t)N * sizeof(ulonglong2) + 6 * (size_t)N * G * sizeof(PC);
+  cudaError_t e = prepare_launch(k_col_pair<N, G>, pthreads<N>() * G, sm);
+  if (e != cudaSuccess) return e;
+  k_col_pair<N, G><<<bgrid(dim3(M / 4 / G), bat), pthreads<N>() * G, sm, st>>>(
+      spec, o0, o1, o2, M, (float)(1.0 / ((double)N * (double)M)), (const float2*)tb.twN, sc,
+      skip, (const float2*)tb.symx, (const float2*)tb.symy, bat);
+  return cudaGetLastError();
+}
+
 template <int N>
 cudaError_t col_pair_N(const float2* spec, float2* o0, float2* o1, float2* o2, int M,
                        const SpecTables& tb, const DevScalars* sc, const int* skip,
                        cudaStream_t st, Bat bat) {
-  const size_t sm = (size_t)N * sizeof(ulonglong2) + 6 * (size_t)N * sizeof(PC);
-  cudaError_t e = prepare_launch(k_col_pair<N>, pthreads<N>(), sm);
-  if (e != cudaSuccess) return e;
-  k_col_pair<N><<<bgrid(dim3(M / 4), bat), pthreads<N>(), sm, st>>>(
-      spec, o0, o1, o2, M, (float)(1.0 / ((double)N * (double)M)), (const float2*)tb.twN, sc,
-      skip, (const float2*)tb.symx, (const float2*)tb.symy, bat);
-  return cudaGetLastError();
+  if constexpr (N <= 1024) {  // (shared memory: 208 N bytes)
+    if (two_pairs(M, bat)) return col_pair_G<N, 2>(spec, o0, o1, o2, M, tb, sc, skip, st, bat);
+  }
+  return col_pair_G<N, 1>(spec, o0, o1, o2, M, tb, sc, skip, st, bat);
 }
 
 }  // namespace

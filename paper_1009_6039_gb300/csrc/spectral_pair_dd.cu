@@ -110,65 +110,76 @@ __device__ __forceinline__ void load_twdd(ulonglong2* th, ulonglong2* tl,
   }
 }
 
-// one double-float stage of radix R (span Ns), in -> out (in place: the stores wait for every
-// thread's loads); the threads as in pstage
+// a double-float stage of radix R (span Ns), in pload, pbfly and pstore's three steps and with their
+// slots
+template <int R, int L>
+__device__ __forceinline__ void dload(DBuf in, DC (&v)[pslots<R>()], int t, int sx = 0) {
+  constexpr int T = R == 3 ? L / 3 : L / 4, LR = L / R;
+#pragma unroll
+  for (int s = 0; s < pslots<R>(); ++s) v[s] = dld(in, swz(t + (s / R) * T + (s % R) * LR) ^ sx);
+}
+template <int R, int SIGN, int L, int Ns>
+__device__ __forceinline__ void dbfly(DC (&v)[pslots<R>()], int t,
+                                      const ulonglong2* __restrict__ th,
+                                      const ulonglong2* __restrict__ tl) {
+  constexpr int T = R == 3 ? L / 3 : L / 4;
+#pragma unroll
+  for (int b = 0; b < pslots<R>() / R; ++b) {
+    if (Ns > 1) {
+      const int k = (int)((unsigned)(t + b * T) % (unsigned)Ns);
+#pragma unroll
+      for (int r = 1; r < R; ++r) {
+        const int ti = (Ns - 1) + (r - 1) * Ns + k;
+        const ulonglong2 wh = th[ti], wl = tl[ti];
+        const D2 wx{wh.x, wl.x};
+        D2 wy{wh.y, wl.y};
+        if (SIGN > 0) wy = d2_neg(wy);
+        v[b * R + r] = dc_mul(v[b * R + r], wx, wy);
+      }
+    }
+    BflyDC<R, SIGN>::run(&v[b * R]);
+  }
+}
+template <int R, int L, int Ns>
+__device__ __forceinline__ void dstore(DBuf out, const DC (&v)[pslots<R>()], int t, int sx = 0) {
+  constexpr int T = R == 3 ? L / 3 : L / 4;
+#pragma unroll
+  for (int s = 0; s < pslots<R>(); ++s) {
+    const int j = t + (s / R) * T;
+    const int qd = (int)((unsigned)j / (unsigned)Ns);
+    dst(out, swz(qd * (Ns * R) + (j - qd * Ns) + (s % R) * Ns) ^ sx, v[s]);
+  }
+}
+// in -> out (in place: the stores wait for every thread's loads)
 template <int R, int SIGN, int L, int Ns, bool INPLACE>
 __device__ __forceinline__ void dstage(DBuf in, DBuf out, int t,
                                        const ulonglong2* __restrict__ th,
-                                       const ulonglong2* __restrict__ tl) {
-  constexpr int NB = R == 3 ? 1 : 4 / R;
-  constexpr int T = R == 3 ? L / 3 : L / 4, LR = L / R;
-  const bool active = L % 3 != 0 || R == 3 || t < T;
-  DC v[NB * R];
-  if (active) {
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      const int j = t + b * T;
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[b * R + r] = dld(in, swz(j + r * LR));
-    }
-  }
+                                       const ulonglong2* __restrict__ tl, int sx = 0) {
+  const bool active = pactive<R, L>(t);
+  DC v[pslots<R>()];
+  if (active) dload<R, L>(in, v, t, sx);
   if (INPLACE) __syncthreads();
   if (active) {
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      const int j = t + b * T;
-      const int qd = (int)((unsigned)j / (unsigned)Ns);
-      const int k = j - qd * Ns;
-      if (Ns > 1) {
-#pragma unroll
-        for (int r = 1; r < R; ++r) {
-          const int ti = (Ns - 1) + (r - 1) * Ns + k;
-          const ulonglong2 wh = th[ti], wl = tl[ti];
-          const D2 wx{wh.x, wl.x};
-          D2 wy{wh.y, wl.y};
-          if (SIGN > 0) wy = d2_neg(wy);
-          v[b * R + r] = dc_mul(v[b * R + r], wx, wy);
-        }
-      }
-      BflyDC<R, SIGN>::run(&v[b * R]);
-      const int d = qd * (Ns * R) + k;
-#pragma unroll
-      for (int r = 0; r < R; ++r) dst(out, swz(d + r * Ns), v[b * R + r]);
-    }
+    dbfly<R, SIGN, L, Ns>(v, t, th, tl);
+    dstore<R, L, Ns>(out, v, t, sx);
   }
   __syncthreads();
 }
 
-// the inverse transform: in place (INPLACE), or alternating between a and b from a (the
-// result ends in a for an even number of stages, in b for an odd one)
+// the inverse transform's stages from span Ns on, without the last one: in place (INPLACE), or
+// alternating between a and b from a
 template <int SIGN, int L, int Ns, int REM, bool INPLACE, bool FROM_A>
 __device__ __forceinline__ void dfft(DBuf a, DBuf b, int t, const ulonglong2* __restrict__ th,
-                                     const ulonglong2* __restrict__ tl) {
-  if constexpr (REM > 1) {
-    constexpr int R = pradix<REM>();
+                                     const ulonglong2* __restrict__ tl, int sx = 0) {
+  constexpr int R = pradix<REM>();
+  if constexpr (REM > R) {
     if constexpr (INPLACE)
-      dstage<R, SIGN, L, Ns, true>(a, a, t, th, tl);
+      dstage<R, SIGN, L, Ns, true>(a, a, t, th, tl, sx);
     else if constexpr (FROM_A)
-      dstage<R, SIGN, L, Ns, false>(a, b, t, th, tl);
+      dstage<R, SIGN, L, Ns, false>(a, b, t, th, tl, sx);
     else
-      dstage<R, SIGN, L, Ns, false>(b, a, t, th, tl);
-    dfft<SIGN, L, Ns * R, REM / R, INPLACE, !FROM_A>(a, b, t, th, tl);
+      dstage<R, SIGN, L, Ns, false>(b, a, t, th, tl, sx);
+    dfft<SIGN, L, Ns * R, REM / R, INPLACE, !FROM_A>(a, b, t, th, tl, sx);
   }
 }
 
@@ -181,8 +192,8 @@ __device__ __forceinline__ float lowpass_of(int mode, int k1, int k2, int M, int
 // eigenvalues, zero mode -> 0, _LP with the Gaussian low-pass) on column pairs: the FP32
 // forward column transform, the scalar symbol step of k_col_lbarinv_dd per column, the
 // double-float inverse column transform (out of place), ddc output
-template <int N, bool POISSON>
-__global__ void __launch_bounds__(pthreads<N>(), N <= 1024 ? 2 : 1)
+template <int N, bool POISSON, int G>
+__global__ void __launch_bounds__(pthreads<N>() * G, N * G <= 1024 ? 2 : 1)
     k_col_lbarinv_pair(const float2* __restrict__ spec, ddc* __restrict__ out, int M, int mode,
                        float inv, const float2* __restrict__ twN32,
                        const float2* __restrict__ twM32, const ddc* __restrict__ twNdd,
@@ -193,48 +204,65 @@ __global__ void __launch_bounds__(pthreads<N>(), N <= 1024 ? 2 : 1)
   sc = badv(sc, bat);
   if (bat.on && bskip(sc, bat)) return;
   constexpr int TPT = pthreads<N>(), E = pelems<N>();
-  constexpr bool FODD = pstage_count<N>() % 2 == 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ulonglong2* tw4 = reinterpret_cast<ulonglong2*>(smem_raw);
   ulonglong2* th = tw4 + N;
   ulonglong2* tl = th + N;
-  ulonglong2* base = tl + N;
+  const int grp = G == 1 ? 0 : threadIdx.x % G, sx = 8 / G * grp;  // as in k_col_pair
+  ulonglong2* base = tl + N + (size_t)grp * 4 * N;
   // double-float buffers A (h, l) and B (h, l); the FP32 forward ping-pongs inside A
   const DBuf A{base, base + N}, B{base + 2 * N, base + 3 * N};
   PC* const F0 = reinterpret_cast<PC*>(A.h);
   PC* const F1 = reinterpret_cast<PC*>(A.l);
   const int Lc = M / 2;
-  const int c0 = 2 * blockIdx.x;
-  const int t = threadIdx.x;
+  const int c0 = 2 * (G * blockIdx.x + grp);
+  const int t = threadIdx.x / G;
   // the column pair's loads first, so that they are in flight with the twiddle tables' loads
   float4 xs[E];
 #pragma unroll
   for (int e = 0; e < E; ++e)
     xs[e] = *reinterpret_cast<const float4*>(spec + (size_t)(t + e * TPT) * Lc + c0);
-  load_tw4<N>(tw4, twN32, t, TPT);
-  load_twdd<N>(th, tl, twNdd, t, TPT);
+  load_tw4<N>(tw4, twN32, threadIdx.x, TPT * G);
+  load_twdd<N>(th, tl, twNdd, threadIdx.x, TPT * G);
+  constexpr int R0 = pradix<N>(), RL = plast<N>();
+  constexpr bool FLIP = pstage_count<N>() % 2 == 1;  // the stages between end in the second buffer
+  const bool last = pactive<RL, N>(t);
+  PC zf[1][E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
-    PC v;
-    v.re = pk(xs[e].x, xs[e].z);
-    v.im = pk(xs[e].y, xs[e].w);
-    F0[swz(t + e * TPT)] = v;
+    zf[0][e].re = pk(xs[e].x, xs[e].z);
+    zf[0][e].im = pk(xs[e].y, xs[e].w);
   }
-  __syncthreads();
   {
     PC* const a[1] = {F0};
     PC* const b[1] = {F1};
-    pfft_rec<-1, N, 1, N, 1, true>(a, b, t, tw4);
+    pfirst_regs<-1, N, 1>(zf, a, t, sx);
+    pfft_rec<-1, N, R0, N / R0, 1, true, false>(a, b, t, tw4, sx);
   }
-  const PC* const F = FODD ? F1 : F0;
+  PC* const F[1] = {FLIP ? F1 : F0};
+  PC* const X = FLIP ? F0 : F1;  // the exchange, as in k_col_pair
+  PC f[1][4];
+  if (last) plast_regs<-1, N, 1>(F, f, t, tw4, sx);
+  if (N % 3 == 0 || blockIdx.x == 0) {
+    if (last) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) X[swz(pout<RL, N>(t, q)) ^ sx] = f[0][q];
+    }
+    __syncthreads();
+  }
 
   float ab[5];
 #pragma unroll
   for (int q = 0; q < 5; ++q) ab[q] = !POISSON ? (float)sc->abar_n[q] : 0.f;
+  DC v[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int k = t + e * TPT;
-    const PC z2 = F[swz(k)];
+    PC z2;
+    if constexpr (N % 3 == 0)
+      z2 = X[swz(k) ^ sx];
+    else
+      z2 = f[0][RL == 4 ? e : (e & 1) * 2 + (e >> 1)];
     float2 zc[2];
     upk(z2.re, zc[0].x, zc[1].x);
     upk(z2.im, zc[0].y, zc[1].y);
@@ -245,7 +273,7 @@ __global__ void __launch_bounds__(pthreads<N>(), N <= 1024 ? 2 : 1)
       const float2 z = zc[h];
       float2 r;
       if (col == 0) {
-        const PC p2 = F[swz((N - k) % N)];
+        const PC p2 = X[swz((N - k) % N) ^ sx];
         float2 pz, pother;
         upk(p2.re, pz.x, pother.x);
         upk(p2.im, pz.y, pother.y);
@@ -275,21 +303,23 @@ __global__ void __launch_bounds__(pthreads<N>(), N <= 1024 ? 2 : 1)
       }
       s[h] = mk2<float>(r.x * inv, r.y * inv);
     }
-    DC v;
-    v.re = D2{pk(s[0].x, s[1].x), 0ull};
-    v.im = D2{pk(s[0].y, s[1].y), 0ull};
-    dst(B, swz(k), v);
+    v[e].re = D2{pk(s[0].x, s[1].x), 0ull};
+    v[e].im = D2{pk(s[0].y, s[1].y), 0ull};
   }
+  // inverse in double-float from B (scratch A, behind the first stage's barrier)
+  dbfly<R0, +1, N, 1>(v, t, th, tl);
+  dstore<R0, N, 1>(B, v, t, sx);
   __syncthreads();
-  // inverse in double-float from B (scratch A)
-  dfft<+1, N, 1, N, false, true>(B, A, t, th, tl);
-  const DBuf res = FODD ? A : B;
+  dfft<+1, N, R0, N / R0, false, true>(B, A, t, th, tl, sx);
+  if (!last) return;
+  DC r[4];
+  dload<RL, N>(FLIP ? A : B, r, t, sx);
+  dbfly<RL, +1, N, N / RL>(r, t, th, tl);
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int n = t + e * TPT;
+  for (int q = 0; q < 4; ++q) {
     ddc a, b;
-    dc_to(dld(res, swz(n)), a, b);
-    ddc* o = out + (size_t)n * Lc + c0;
+    dc_to(r[q], a, b);
+    ddc* o = out + (size_t)pout<RL, N>(t, q) * Lc + c0;
     o[0] = a;
     o[1] = b;
   }
@@ -360,16 +390,22 @@ __global__ void __launch_bounds__(pthreads<L>(), L <= 512 ? 4 : 2)
     }
   }
   __syncthreads();
-  dfft<+1, L, 1, L, true, true>(A, A, t, th, tl);
+  constexpr int R0 = pradix<L>(), RL = plast<L>();
+  dstage<R0, +1, L, 1, true>(A, A, t, th, tl);
+  dfft<+1, L, R0, L / R0, true, true>(A, A, t, th, tl);
+  if (!pactive<RL, L>(t)) return;
+  DC r[4];
+  dload<RL, L>(A, r, t);
+  dbfly<RL, +1, L, L / RL>(r, t, th, tl);
   const double2* uia = u_in ? reinterpret_cast<const double2*>(u_in + (size_t)r0 * M) : nullptr;
   const double2* uib = u_in ? uia + L : nullptr;
   double2* uoa = reinterpret_cast<double2*>(u_out + (size_t)r0 * M);
   double2* uob = uoa + L;
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int n = t + e * TPT;
+  for (int e = 0; e < 4; ++e) {
+    const int n = pout<RL, L>(t, e);
     ddc za, zb;
-    dc_to(dld(A, swz(n)), za, zb);
+    dc_to(r[e], za, zb);
     double2 a = uia ? uia[n] : make_double2(0.0, 0.0);
     double2 b = uib ? uib[n] : make_double2(0.0, 0.0);
     a.x = fma(step, dd_to_double(za.x), a.x);
@@ -381,14 +417,14 @@ __global__ void __launch_bounds__(pthreads<L>(), L <= 512 ? 4 : 2)
   }
 }
 
-template <int N, bool POISSON>
+template <int N, bool POISSON, int G>
 cudaError_t col_lbarinv_pair_launch(const float2* spec, ddc* out, int M, const SpecTables& tb32,
                                const SpecTables& tbdd, const DevScalars* sc, cudaStream_t st,
                                int mode, Bat bat) {
-  const size_t sm = 7 * (size_t)N * sizeof(ulonglong2);
-  cudaError_t e = prepare_launch(k_col_lbarinv_pair<N, POISSON>, pthreads<N>(), sm);
+  const size_t sm = (3 + 4 * G) * (size_t)N * sizeof(ulonglong2);
+  cudaError_t e = prepare_launch(k_col_lbarinv_pair<N, POISSON, G>, pthreads<N>() * G, sm);
   if (e != cudaSuccess) return e;
-  k_col_lbarinv_pair<N, POISSON><<<bgrid(dim3(M / 4), bat), pthreads<N>(), sm, st>>>(
+  k_col_lbarinv_pair<N, POISSON, G><<<bgrid(dim3(M / 4 / G), bat), pthreads<N>() * G, sm, st>>>(
       spec, out, M, mode, (float)(1.0 / ((double)N * (double)M)), (const float2*)tb32.twN,
       (const float2*)tb32.twM, (const ddc*)tbdd.twN, sc, (const float2*)tb32.symx,
       (const float2*)tb32.symy, bat);
@@ -399,9 +435,16 @@ template <int N>
 cudaError_t col_lbarinv_pair_N(const float2* spec, ddc* out, int M, const SpecTables& tb32,
                                const SpecTables& tbdd, const DevScalars* sc, cudaStream_t st,
                                int mode, Bat bat) {
+  if constexpr (N <= 1024) {
+    if (two_pairs(M, bat)) {
+      if (mode == COL_LBARINV)
+        return col_lbarinv_pair_launch<N, false, 2>(spec, out, M, tb32, tbdd, sc, st, mode, bat);
+      return col_lbarinv_pair_launch<N, true, 2>(spec, out, M, tb32, tbdd, sc, st, mode, bat);
+    }
+  }
   if (mode == COL_LBARINV)
-    return col_lbarinv_pair_launch<N, false>(spec, out, M, tb32, tbdd, sc, st, mode, bat);
-  return col_lbarinv_pair_launch<N, true>(spec, out, M, tb32, tbdd, sc, st, mode, bat);
+    return col_lbarinv_pair_launch<N, false, 1>(spec, out, M, tb32, tbdd, sc, st, mode, bat);
+  return col_lbarinv_pair_launch<N, true, 1>(spec, out, M, tb32, tbdd, sc, st, mode, bat);
 }
 
 template <int L>

@@ -97,3 +97,11 @@ def test_solves_on_pairs_fused_and_batched(ot, N, M):
     assert torch.equal(phis[0], phis[2])
     assert float((phis[0] - u).abs().max()) <= 1e-6
     ps.close()
+
+
+@pytest.mark.parametrize("N,M", [(96, 768), (128, 1024), (192, 768), (256, 1024), (384, 768),
+                                 (512, 768), (768, 768), (1024, 768)])
+def test_two_column_pairs_per_block(ot, N, M):
+    # more than 152 column pairs: blocks of two (the same bounds)
+    test_operator_on_pairs(ot, N, M)
+    test_poisson_on_pairs(ot, N, M, False)
