@@ -598,7 +598,9 @@ static int alloc_buffers(ot_plan* p) {
   RET(alloc_tables(p));
   if (p->interp) RET(alloc_grad_planes(p));
   if (p->linsolver) RET(alloc_fd_planes(p));
-  size_t np = (size_t)residual_partial_blocks(p->N, p->M) * 10;
+  // (an 8-row tile's ten partials per block at most)
+  size_t np = std::max((size_t)residual_partial_blocks(p->N, p->M),
+                       (size_t)((p->M + 31) / 32) * ((p->N + 7) / 8)) * 10;
   size_t nk = (size_t)p->sms * kMaxKrylovBlocksPerSm * OTGB_MAXM;  // any OT_OPT_KRYLOV_BLOCKS
   if (nk > np) np = nk;
   CK(cudaMalloc(&p->partials, np * 8));
@@ -643,7 +645,9 @@ static int alloc_batch(ot_plan* p, int B) {
   // GMRES vector kernels: blocks per pair by its size (the pairs fill the GPU together)
   long kb = (long)(P / 2048);
   p->kblocks = (int)std::min<long>(std::max<long>(kb, 8), p->sms);
-  size_t np = (size_t)residual_partial_blocks(p->N, p->M) * 10;
+  // (an 8-row tile's ten partials per block at most)
+  size_t np = std::max((size_t)residual_partial_blocks(p->N, p->M),
+                       (size_t)((p->M + 31) / 32) * ((p->N + 7) / 8)) * 10;
   np = std::max(np, (size_t)p->kblocks * OTGB_MAXM);
   np = std::max(np, (size_t)2 * p->sms * 8);  // the 2-blocks-per-SM grid reductions
   struct Item {

@@ -366,21 +366,6 @@ __device__ __forceinline__ int wrap_near(int a, int L) {  // a in [-L, 2L)
   return a < 0 ? a + L : (a >= L ? a - L : a);
 }
 
-template <typename G>
-__device__ __forceinline__ void bspline_w(G t, G w[4], G dw[4]) {
-  const G s = (G)1 - t;
-  const G t2 = t * t, t3 = t2 * t;
-  const G sixth = (G)(1.0 / 6.0);
-  w[0] = s * s * s * sixth;
-  w[1] = ((G)3 * t3 - (G)6 * t2 + (G)4) * sixth;
-  w[2] = ((G)-3 * t3 + (G)3 * t2 + (G)3 * t + (G)1) * sixth;
-  w[3] = t3 * sixth;
-  dw[0] = (G)-0.5 * s * s;
-  dw[1] = (G)0.5 * ((G)3 * t2 - (G)4 * t);
-  dw[2] = (G)0.5 * ((G)-3 * t2 + (G)2 * t + (G)1);
-  dw[3] = (G)0.5 * t2;
-}
-
 // ---------------------------------------------------------------------------------------
 // Mixed-mode residual: the same evaluation with every FP64-accuracy quantity (the stencils
 // of u, the displaced point, the B-spline value gather, det, f_n and F) in double-float
@@ -404,40 +389,35 @@ __device__ __forceinline__ dd ldd(const float2* __restrict__ a, size_t i) {
   return dd{v.x, v.y};
 }
 
-// 6 x the cubic B-spline value weights at t in [0, 1) (taps -1, 0, 1, 2): s^3,
+// 6 x the cubic B-spline value weights at t in [0, 1) (taps -1, 0, 1, 2) for two positions: s^3,
 // 3 t^3 - 6 t^2 + 4, 6 - (the other three), t^3, with s = 1 - t; all coefficients exact
-__device__ __forceinline__ void bspline6_dd(dd t, dd w[4]) {
-  const dd s = dd_add_f(dd_neg(t), 1.0f);
-  const dd t2 = dd_mul(t, t), t3 = dd_mul(t2, t);
-  w[0] = dd_mul(dd_mul(s, s), s);
-  w[1] = dd_add_f(dd_sub(dd_mul_f(t3, 3.0f), dd_mul_f(t2, 6.0f)), 4.0f);
-  w[3] = t3;
-  w[2] = dd_add_f(dd_neg(dd_add(dd_add(w[0], w[1]), w[3])), 6.0f);
-}
-
-// the same weights for two positions at once (t.h, t.l: the lanes' high and low words), each
-// lane bit for bit bspline6_dd's
 __device__ __forceinline__ void bspline6_dd2(pair::D2 t, pair::D2 w[4]) {
   using namespace pair;
-  const u64 one = pk(1.0f, 1.0f);
-  // dd_add_f(a, b) = fast_two_sum(s.hi, s.lo + a.lo) with s = two_sum(a.hi, b)
-  auto add_f = [](D2 a, u64 b) {
-    const D2 s = two_sum2(a.h, b);
-    return fast_two_sum2(s.h, add2(s.l, a.l));
-  };
-  // dd_mul_f(a, b) = fast_two_sum(p, fma(a.lo, b, fma(a.hi, b, -p))) with p = a.hi b
-  auto mul_f = [](D2 a, u64 b) {
-    const u64 p = mul2(a.h, b);
-    u64 e = fma2(a.h, b, neg2(p));
-    e = fma2(a.l, b, e);
-    return fast_two_sum2(p, e);
-  };
-  const D2 s = add_f(d2_neg(t), one);
-  const D2 t2 = d2_mul(t, t), t3 = d2_mul(t2, t);
-  w[0] = d2_mul(d2_mul(s, s), s);
-  w[1] = add_f(d2_sub(mul_f(t3, pk(3.0f, 3.0f)), mul_f(t2, pk(6.0f, 6.0f))), pk(4.0f, 4.0f));
+  const D2 s = d2_sub(D2{pk(1.0f, 1.0f), 0ull}, t);
+  const u64 nt = neg2(t.h);
+  const D2 t2 = d2_mul_n(t, t, nt), t3 = d2_mul_n(t2, t, nt);
+  const u64 ns = neg2(s.h);
+  w[0] = d2_mul_n(d2_mul_n(s, s, ns), s, ns);
+  w[1] = d2_add_f(d2_sub(d2_mul_f(t3, pk(3.0f, 3.0f)), d2_mul_f(t2, pk(6.0f, 6.0f))),
+                  pk(4.0f, 4.0f));
   w[3] = t3;
-  w[2] = add_f(d2_neg(d2_add(d2_add(w[0], w[1]), w[3])), pk(6.0f, 6.0f));
+  w[2] = d2_sub(D2{pk(6.0f, 6.0f), 0ull}, d2_add(d2_add(w[0], w[1]), w[3]));
+}
+// the FP32 weights and their derivatives for two positions (the Jacobian's)
+__device__ __forceinline__ void bspline_w2(pair::u64 t, pair::u64 w[4], pair::u64 dw[4]) {
+  using namespace pair;
+  auto c = [](float x) { return pk(x, x); };
+  const u64 s = sub2(c(1.0f), t), t2 = mul2(t, t), s2 = mul2(s, s);
+  const float sixth = 1.0f / 6.0f;
+  w[0] = mul2(mul2(s2, s), c(sixth));
+  w[1] = fma2(t2, fma2(t, c(0.5f), c(-1.0f)), c(4.0f * sixth));
+  w[2] = fma2(t, fma2(t, fma2(t, c(-0.5f), c(0.5f)), c(0.5f)), c(sixth));
+  w[3] = mul2(mul2(t2, t), c(sixth));
+  dw[0] = mul2(s2, c(-0.5f));
+  dw[1] = mul2(c(0.5f), fma2(c(3.0f), t2, mul2(c(-4.0f), t)));
+  dw[3] = mul2(t2, c(0.5f));
+  // (their sum is zero: a rounding error of it enters G_x times M)
+  dw[2] = neg2(add2(add2(dw[0], dw[3]), dw[1]));
 }
 
 // floor of a dd position p (|p| < 2^23): integer part k and fraction t in [0, 1) as dd.
@@ -457,7 +437,24 @@ __device__ __forceinline__ int dd_floor(dd p, dd* t) {
   return (int)fl;
 }
 
-// A block covers 32 columns x 8 RPT rows, RPT rows per thread.
+// the scalars of a residual from its ten totals
+__device__ __forceinline__ void residual_close(DevScalars* sc, const double (&v)[10], int N,
+                                               int M) {
+  const double Pd = (double)N * (double)M;
+  const double mean_fn = v[0] / Pd;
+  const double shift = mean_fn - 1.0;
+  sc->mean_fn = mean_fn;
+  sc->shift = shift;
+  sc->res_inf = fmax(fabs(v[6] + shift), fabs(v[7] + shift));
+  for (int a = 0; a < 5; ++a) sc->abar[a] = v[1 + a];
+  sc->min_det = v[8];
+  sc->k1_nonfinite = (int)v[9];
+  sc->admissible = (v[9] == 0.0 && isfinite(sc->res_inf) && v[8] > 0.0) ? 1 : 0;
+  sc->ticket[TK_RESID] = 0;
+}
+
+// Nearest-node and bilinear interpolation (a block covers 32 columns x 8 RPT rows, RPT rows per
+// thread)
 template <int RPT>
 __global__ void __launch_bounds__(8 * RTX, 3)
     k_residual_dd(const float2* __restrict__ fdd, const float2* __restrict__ cdd,
@@ -554,7 +551,7 @@ __global__ void __launch_bounds__(8 * RTX, 3)
       G = ldd(cdd, q);
       Gx = __ldg(K.gx + q);
       Gy = __ldg(K.gy + q);
-    } else if (K.interp == 1) {  // bilinear on the cell (i0, j0) .. (i0 + 1, j0 + 1)
+    } else {  // bilinear on the cell (i0, j0) .. (i0 + 1, j0 + 1)
       const dd sx = dd_add_f(dd{-tx_.hi, -tx_.lo}, 1.0f), sy = dd_add_f(dd{-ty_.hi, -ty_.lo}, 1.0f);
       const size_t q00 = (size_t)ii[1] * M + jj[1], q01 = (size_t)ii[1] * M + jj[2];
       const size_t q10 = (size_t)ii[2] * M + jj[1], q11 = (size_t)ii[2] * M + jj[2];
@@ -568,59 +565,6 @@ __global__ void __launch_bounds__(8 * RTX, 3)
            w11 * __ldg(K.gx + q11);
       Gy = w00 * __ldg(K.gy + q00) + w01 * __ldg(K.gy + q01) + w10 * __ldg(K.gy + q10) +
            w11 * __ldg(K.gy + q11);
-    } else {
-      // packed pairs (dd2.cuh): the x and y value weights in the two lanes of one call, then
-      // the 16-tap gather over row pairs (b, b + 2), each lane a row's double-float sum in the
-      // scalar order; the two lanes' partial sums of G (rows 0, 1 and rows 2, 3) are added last
-      using namespace pair;
-      dd wxs[4], wys[4];
-      bspline6_dd(tx_, wxs);
-      bspline6_dd(ty_, wys);
-      D2 wv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) wv[a] = D2{pk(wxs[a].hi, wys[a].hi), pk(wxs[a].lo, wys[a].lo)};
-      // gradient weights in FP32 (Jacobian only)
-      float wxf[4], dwx[4], wyf[4], dwy[4];
-      bspline_w<float>(tx_.hi, wxf, dwx);
-      bspline_w<float>(ty_.hi, wyf, dwy);
-      D2 G36p{0ull, 0ull};
-      u64 gxp = 0ull, gyp = 0ull;
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const size_t ra = (size_t)ii[b] * M, rb = (size_t)ii[b + 2] * M;
-        D2 sv{0ull, 0ull};
-        u64 svf = 0ull, sdf = 0ull;
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          const float2 ca = __ldg(cdd + ra + jj[a]), cb = __ldg(cdd + rb + jj[a]);
-          const D2 cv{pk(ca.x, cb.x), pk(ca.y, cb.y)};
-          float xh, xl, yh, yl;  // the x weight, broadcast to both lanes
-          upk(wv[a].h, xh, yh);
-          upk(wv[a].l, xl, yl);
-          sv = d2_add(d2_mul(cv, D2{pk(xh, xh), pk(xl, xl)}), sv);
-          svf = fma2(cv.h, pk(wxf[a], wxf[a]), svf);
-          sdf = fma2(cv.h, pk(dwx[a], dwx[a]), sdf);
-        }
-        float xh0, yh0, xl0, yl0, xh2, yh2, xl2, yl2;  // the y weights of rows b and b + 2
-        upk(wv[b].h, xh0, yh0);
-        upk(wv[b].l, xl0, yl0);
-        upk(wv[b + 2].h, xh2, yh2);
-        upk(wv[b + 2].l, xl2, yl2);
-        const D2 wyp{pk(yh0, yh2), pk(yl0, yl2)};
-        G36p = d2_add(d2_mul(sv, wyp), G36p);
-        gxp = fma2(sdf, pk(wyf[b], wyf[b + 2]), gxp);
-        gyp = fma2(svf, pk(dwy[b], dwy[b + 2]), gyp);
-      }
-      dd g01, g23;
-      upk(G36p.h, g01.hi, g23.hi);
-      upk(G36p.l, g01.lo, g23.lo);
-      const dd G36 = dd_add(g01, g23);
-      float gx01, gx23, gy01, gy23;
-      upk(gxp, gx01, gx23);
-      upk(gyp, gy01, gy23);
-      G = dd_mul(G36, K.inv36);
-      Gx = (gx01 + gx23) * K.M;
-      Gy = (gy01 + gy23) * K.N;
     }
     const dd det = dd_sub(dd_mul(dd_add_f(uxx, 1.0f), dd_add_f(uyy, 1.0f)), dd_mul(uxy, uxy));
     const dd fn = dd_mul(G, det);
@@ -668,17 +612,351 @@ __global__ void __launch_bounds__(8 * RTX, 3)
   if (threadIdx.x == 0) {
     double v[10];
     for (int a = 0; a < 10; ++a) v[a] = (double)r[a].hi + (double)r[a].lo;
-    const double Pd = (double)N * (double)M;
-    const double mean_fn = v[0] / Pd;
-    const double shift = mean_fn - 1.0;
-    sc->mean_fn = mean_fn;
-    sc->shift = shift;
-    sc->res_inf = fmax(fabs(v[6] + shift), fabs(v[7] + shift));
-    for (int a = 0; a < 5; ++a) sc->abar[a] = v[1 + a];
-    sc->min_det = v[8];
-    sc->k1_nonfinite = (int)v[9];
-    sc->admissible = (v[9] == 0.0 && isfinite(sc->res_inf) && v[8] > 0.0) ? 1 : 0;
-    sc->ticket[TK_RESID] = 0;
+    residual_close(sc, v, N, M);
+  }
+}
+
+// ---------------------------------------------------------------------------------------
+// The cubic-spline residual on two points per thread, rows ty and ty + RB of a tile of 2 RB RT x 32
+// points, held in the two lanes of packed FP32 pairs (dd2.cuh): every double-float operation is one
+// packed instruction for both points.  The kernel is bound by instruction issue and the latency of
+// the double-float chains (16 warps per SM: a point pair fills 128 registers), not by its 52 bytes
+// a point: with one point per thread 1650 instructions a point, 1120 here, a tenth of the former
+// the block sums' shuffle trees.  These are folded: eight values' halves change lanes together, and
+// maxima and minima go as ordered integers through the warp reduction instructions.  1024^2: 75.5
+// -> 63.6 us, 256^2 15.1 -> 11.0.  (80 registers for 24 warps per SM: 79 us, spills.)
+// ---------------------------------------------------------------------------------------
+struct ResidSums {
+  dd s[6];            // sum of f_n, the five Simpson sums
+  dd fmax, fmin, dmin;
+  int bad;
+};
+__device__ __forceinline__ int ordered32(float x) {
+  const int b = __float_as_int(x);
+  return b ^ ((b >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float unordered32(int k) {
+  return __int_as_float(k ^ ((k >> 31) & 0x7fffffff));
+}
+// smallest dd of the lanes in mask (largest: of the negated one; no lane holds a NaN)
+__device__ __forceinline__ dd warp_min_dd(dd v, unsigned mask) {
+  const int h = ordered32(v.hi), m = __reduce_min_sync(mask, h);
+  const int l = __reduce_min_sync(mask, h == m ? ordered32(v.lo) : 0x7fffffff);
+  return dd{unordered32(m), unordered32(l)};
+}
+// the block's ten values to dst (the order of k_residual_dd's partials); NW (4 or 8) warps
+template <int NW>
+__device__ __forceinline__ void resid_block_sums(const ResidSums& r, float2* dst) {
+  __shared__ float2 ws[NW][8], we[3][NW];
+  __shared__ int wb[NW];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  auto shfl = [](dd v, int o) {
+    return dd{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+  };
+  dd x[8];
+#pragma unroll
+  for (int a = 0; a < 8; ++a) x[a] = a < 6 ? r.s[a] : dd{0.f, 0.f};
+  int o = 16;
+#pragma unroll
+  for (int h = 4; h > 0; h /= 2, o /= 2) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int a = 0; a < h; ++a)
+      x[a] = dd_add(up ? x[a + h] : x[a], shfl(up ? x[a] : x[a + h], o));
+  }
+  x[0] = dd_add(x[0], shfl(x[0], 2));
+  x[0] = dd_add(x[0], shfl(x[0], 1));
+  const dd mx = warp_min_dd(dd_neg(r.fmax), 0xffffffffu), mn = warp_min_dd(r.fmin, 0xffffffffu),
+           md = warp_min_dd(r.dmin, 0xffffffffu);
+  const int nb = __reduce_add_sync(0xffffffffu, r.bad);
+  if (lane % 4 == 0) ws[wid][lane / 4] = make_float2(x[0].hi, x[0].lo);
+  if (lane == 0) {
+    we[0][wid] = make_float2(mx.hi, mx.lo);
+    we[1][wid] = make_float2(mn.hi, mn.lo);
+    we[2][wid] = make_float2(md.hi, md.lo);
+    wb[wid] = nb;
+  }
+  __syncthreads();
+  if (threadIdx.x < 8 * NW) {  // (groups of NW lanes: value threadIdx.x / NW)
+    const int a = threadIdx.x / NW;
+    const float2 q = ws[threadIdx.x % NW][a];
+    dd s = dd{q.x, q.y};
+#pragma unroll
+    for (int m = NW / 2; m > 0; m /= 2) s = dd_add(s, shfl(s, m));
+    if (threadIdx.x % NW == 0 && a < 6) dst[a] = make_float2(s.hi, s.lo);
+  } else if (wid == NW - 1 && lane < NW) {
+    constexpr unsigned mask = (1u << NW) - 1;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const float2 q = we[a][lane];
+      dd m = warp_min_dd(dd{q.x, q.y}, mask);
+      if (a == 0) m = dd_neg(m);
+      if (lane == 0) dst[6 + a] = make_float2(m.hi, m.lo);
+    }
+    const int n = __reduce_add_sync(mask, wb[lane]);
+    if (lane == 0) dst[9] = make_float2((float)n, 0.f);
+  }
+}
+
+template <int RB, int RT, int BPS>
+__global__ void __launch_bounds__(RB * RTX, BPS)
+    k_residual_dd2(const float2* __restrict__ fdd, const float2* __restrict__ cdd,
+                   const double* __restrict__ ua, const double* __restrict__ ub, int sel, int N,
+                   int M, ResidConstsDD K, double* __restrict__ Fraw, float* __restrict__ coef,
+                   double* partials, DevScalars* sc, Bat bat) {
+  using namespace pair;
+  constexpr int RTY = 2 * RB * RT, W = RTX + 4;
+  __shared__ float th[RTY + 4][W], tl[RTY + 4][W];  // u with a halo of 2, high and low words
+  __shared__ float yh[RTY][W], yl[RTY][W];          // its unscaled y-difference
+  fdd = badv(fdd, bat);
+  cdd = badv(cdd, bat);
+  ua = badv(ua, bat);
+  ub = badv(ub, bat);
+  Fraw = badv(Fraw, bat);
+  coef = badv(coef, bat);
+  partials = badv(partials, bat);
+  sc = badv(sc, bat);
+  if (bskip(sc, bat)) return;
+  const double* __restrict__ u = (ub && ((sc->upar ^ sel) & 1)) ? ub : ua;
+  const int bx = blockIdx.x * RTX, by = blockIdx.y * RTY;
+  const int tid = threadIdx.x;
+  for (int idx = tid; idx < (RTY + 4) * W; idx += RB * RTX) {
+    const int r = idx / W, cc = idx - r * W;
+    int gi = wrap_near(by + r - 2, N), gj = wrap_near(bx + cc - 2, M);
+    if (gi >= N) gi %= N;  // (a grid smaller than the tile)
+    if (gj >= M) gj %= M;
+    const dd v = dd_from_double_cvt(u[(size_t)gi * M + gj]);
+    th[r][cc] = v.hi;
+    tl[r][cc] = v.lo;
+  }
+  __syncthreads();
+  for (int idx = tid; idx < RTY / 2 * W; idx += RB * RTX) {  // rows r and r + RTY / 2
+    constexpr int H = RTY / 2;
+    const int r = idx / W, c = idx - r * W;
+    auto T = [&](int d) {
+      return D2{pk(th[r + d][c], th[r + H + d][c]), pk(tl[r + d][c], tl[r + H + d][c])};
+    };
+    const D2 v = d2_sub(d2_scale2(d2_sub(T(3), T(1)), 8.0f), d2_sub(T(4), T(0)));
+    upk(v.h, yh[r][c], yh[r + H][c]);
+    upk(v.l, yl[r][c], yl[r + H][c]);
+  }
+  __syncthreads();
+  ResidSums acc;
+  acc.fmax = dd{-INFINITY, 0.f};
+  acc.fmin = acc.dmin = dd{INFINITY, 0.f};
+  acc.bad = 0;
+  D2 sfn{0ull, 0ull};
+  float simp[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+  const int tx = tid % RTX, ty0 = tid / RTX;
+  const int j = bx + tx;
+  const size_t P = (size_t)N * M;
+  const float wx = ((j & 1) ? 4.0f : 2.0f) * K.w3M;
+  const u64 one = pk(1.0f, 1.0f);
+  auto bc = [](dd c) { return D2{pk(c.hi, c.hi), pk(c.lo, c.lo)}; };
+#pragma unroll 1
+  for (int rr = 0; rr < RT; ++rr) {
+    const int ty = ty0 + 2 * RB * rr;
+    const int i = by + ty;
+    if (i >= N || j >= M) continue;
+    const bool two = i + RB < N;  // (a missing second row is computed on the wrapped rows)
+    const int q = tx + 2;
+    auto T = [&](int dr, int dc) {
+      const int r = ty + 2 + dr;
+      return D2{pk(th[r][q + dc], th[r + RB][q + dc]), pk(tl[r][q + dc], tl[r + RB][q + dc])};
+    };
+    auto Y = [&](int dc) {
+      return D2{pk(yh[ty][q + dc], yh[ty + RB][q + dc]), pk(yl[ty][q + dc], yl[ty + RB][q + dc])};
+    };
+    D2 ux, uxx, uyy;
+    {
+      const D2 c30 = d2_mul_f(T(0, 0), pk(30.0f, 30.0f));
+      const D2 xp1 = T(0, 1), xm1 = T(0, -1), xp2 = T(0, 2), xm2 = T(0, -2);
+      ux = d2_mul(d2_sub(d2_scale2(d2_sub(xp1, xm1), 8.0f), d2_sub(xp2, xm2)), bc(K.Mh));
+      uxx = d2_mul(d2_sub(d2_sub(d2_scale2(d2_add(xp1, xm1), 16.0f), d2_add(xp2, xm2)), c30),
+                   bc(K.Mh2));
+      uyy = d2_mul(d2_sub(d2_sub(d2_scale2(d2_add(T(1, 0), T(-1, 0)), 16.0f),
+                                 d2_add(T(2, 0), T(-2, 0))),
+                          c30),
+                   bc(K.Nh2));
+    }
+    const D2 uy = d2_mul(Y(0), bc(K.Nh));
+    const D2 uxy =
+        d2_mul(d2_sub(d2_scale2(d2_sub(Y(1), Y(-1)), 8.0f), d2_sub(Y(2), Y(-2))), bc(K.MNh));
+    // the displaced points in grid units: cells and fractions (dd_floor per lane)
+    int fa, fb;
+    auto split = [&](D2 p, D2* t) {
+      float pa, pb, ra, rb;
+      upk(p.h, pa, pb);
+      pa = floorf(pa);
+      pb = floorf(pb);
+      D2 f = d2_sub(p, D2{pk(pa, pb), 0ull});
+      upk(f.h, ra, rb);
+      if (ra < 0.f || ra >= 1.f || rb < 0.f || rb >= 1.f) {
+        const float da = ra < 0.f ? 1.f : (ra >= 1.f ? -1.f : 0.f);
+        const float db = rb < 0.f ? 1.f : (rb >= 1.f ? -1.f : 0.f);
+        pa -= da;
+        pb -= db;
+        f = d2_add_f(f, pk(da, db));
+      }
+      *t = f;
+      fa = (int)pa;
+      fb = (int)pb;
+    };
+    D2 tX, tY;
+    split(d2_add_f(d2_mul_f(ux, pk(K.M, K.M)), pk((float)j, (float)j)), &tX);
+    auto wrap = [](int a, int L) { return (unsigned)a < (unsigned)L ? a : wrapi(a, L); };
+    int ja[4], jb[4];
+    ja[1] = wrap(fa, M);
+    jb[1] = wrap(fb, M);
+    split(d2_add_f(d2_mul_f(uy, pk(K.N, K.N)), pk((float)i, (float)(i + RB))), &tY);
+    int ia[4], ib[4];
+    ia[1] = wrap(fa, N);
+    ib[1] = wrap(fb, N);
+    auto taps = [](int (&k)[4], int L) {
+      k[0] = k[1] == 0 ? L - 1 : k[1] - 1;
+      k[2] = wrap_near(k[1] + 1, L);
+      k[3] = wrap_near(k[1] + 2, L);
+    };
+    taps(ja, M);
+    taps(jb, M);
+    taps(ia, N);
+    taps(ib, N);
+    // the 16-tap gather, rows 0, 1 and rows 2, 3 summed apart; value weights in double-float, the gradient's in FP32 (Jacobian only)
+    D2 wv[4];
+    bspline6_dd2(tX, wv);
+    u64 nw[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) nw[a] = neg2(wv[a].h);
+    u64 wxf[4], dwx[4];
+    bspline_w2(tX.h, wxf, dwx);
+    D2 wy[4];
+    bspline6_dd2(tY, wy);
+    u64 wyf[4], dwy[4];
+    bspline_w2(tY.h, wyf, dwy);
+    D2 Gr[2];
+    u64 gx = 0ull, gy = 0ull;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const float2* ra = cdd + (size_t)ia[b] * M;
+      const float2* rb = cdd + (size_t)ib[b] * M;
+      D2 sv;
+      u64 svf = 0ull, sdf = 0ull;
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        const float2 ca = __ldg(ra + ja[a]), cb = __ldg(rb + jb[a]);
+        const D2 cv{pk(ca.x, cb.x), pk(ca.y, cb.y)};
+        const D2 m = d2_mul_n(cv, wv[a], nw[a]);
+        sv = a == 0 ? m : d2_add(m, sv);
+        svf = a == 0 ? mul2(cv.h, wxf[0]) : fma2(cv.h, wxf[a], svf);
+        sdf = a == 0 ? mul2(cv.h, dwx[0]) : fma2(cv.h, dwx[a], sdf);
+      }
+      const D2 m = d2_mul(sv, wy[b]);
+      Gr[b / 2] = b % 2 == 0 ? m : d2_add(m, Gr[b / 2]);
+      gx = b == 0 ? mul2(sdf, wyf[0]) : fma2(sdf, wyf[b], gx);
+      gy = b == 0 ? mul2(svf, dwy[0]) : fma2(svf, dwy[b], gy);
+    }
+    const D2 G = d2_mul(d2_add(Gr[0], Gr[1]), bc(K.inv36));
+    const D2 det = d2_sub(d2_mul(d2_add_f(uxx, one), d2_add_f(uyy, one)), d2_mul(uxy, uxy));
+    const D2 fn = d2_mul(G, det);
+    const size_t p = (size_t)i * M + j, pb = two ? p + (size_t)RB * M : p;
+    const float2 f0 = __ldg(fdd + p), f1 = __ldg(fdd + pb);
+    const D2 fr = d2_sub(D2{pk(f0.x, f1.x), pk(f0.y, f1.y)}, fn);
+    dd ra, rb, na, nb, da, db;
+    upk(fr.h, ra.hi, rb.hi);
+    upk(fr.l, ra.lo, rb.lo);
+    upk(fn.h, na.hi, nb.hi);
+    upk(fn.l, na.lo, nb.lo);
+    upk(det.h, da.hi, db.hi);
+    upk(det.l, da.lo, db.lo);
+    // coefficients of the linearisation (Jacobian only), FP32
+    u64 cf[5];
+    cf[0] = mul2(G.h, add2(one, uyy.h));
+    cf[1] = neg2(mul2(G.h, uxy.h));
+    cf[2] = mul2(G.h, add2(one, uxx.h));
+    cf[3] = K.nob ? 0ull : mul2(det.h, mul2(gx, pk(K.M, K.M)));
+    cf[4] = K.nob ? 0ull : mul2(det.h, mul2(gy, pk(K.N, K.N)));
+    Fraw[p] = (double)ra.hi + (double)ra.lo;
+    if (two) Fraw[pb] = (double)rb.hi + (double)rb.lo;
+    const float w = ((i & 1) ? 4.0f : 2.0f) * K.w3N * wx;  // (rows i and i + RB alike)
+#pragma unroll
+    for (int a = 0; a < 5; ++a) {
+      float x, y;
+      upk(cf[a], x, y);
+      coef[a * P + p] = x;
+      simp[a] = fmaf(w, x, simp[a]);
+      if (two) {
+        coef[a * P + pb] = y;
+        simp[a] = fmaf(w, y, simp[a]);
+      }
+    }
+    auto finite = [](dd v) { return fabsf(v.hi) < INFINITY && fabsf(v.lo) < INFINITY; };
+    if (finite(na)) {
+      if (dd_gt(ra, acc.fmax)) acc.fmax = ra;
+      if (dd_gt(acc.fmin, ra)) acc.fmin = ra;
+    } else {
+      na = dd{0.f, 0.f};
+      ++acc.bad;
+    }
+    if (dd_gt(acc.dmin, da)) acc.dmin = da;
+    if (two) {
+      if (finite(nb)) {
+        if (dd_gt(rb, acc.fmax)) acc.fmax = rb;
+        if (dd_gt(acc.fmin, rb)) acc.fmin = rb;
+      } else {
+        nb = dd{0.f, 0.f};
+        ++acc.bad;
+      }
+      if (dd_gt(acc.dmin, db)) acc.dmin = db;
+    } else {
+      nb = dd{0.f, 0.f};
+    }
+    sfn = d2_add(sfn, D2{pk(na.hi, nb.hi), pk(na.lo, nb.lo)});
+  }
+  {
+    dd a, b;
+    upk(sfn.h, a.hi, b.hi);
+    upk(sfn.l, a.lo, b.lo);
+    acc.s[0] = dd_add(a, b);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) acc.s[1 + k] = dd{simp[k], 0.f};
+  }
+  // grid reductions: a block's ten values, then those of all blocks in the last one
+  __shared__ bool last;
+  __shared__ float2 tot[10];
+  float2* pf = reinterpret_cast<float2*>(partials);
+  const unsigned int nblk = gridDim.x * gridDim.y;
+  resid_block_sums<RB>(acc, pf + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 10);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = atomicAdd(&sc->ticket[TK_RESID], 1u) == nblk - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  acc.fmax = dd{-INFINITY, 0.f};
+  acc.fmin = acc.dmin = dd{INFINITY, 0.f};
+  acc.bad = 0;
+#pragma unroll
+  for (int a = 0; a < 6; ++a) acc.s[a] = dd{0.f, 0.f};
+  for (unsigned int b = tid; b < nblk; b += RB * RTX) {
+    dd v[10];
+#pragma unroll
+    for (int a = 0; a < 10; ++a) {
+      const float2 t = __ldcg(pf + (size_t)b * 10 + a);
+      v[a] = dd{t.x, t.y};
+    }
+#pragma unroll
+    for (int a = 0; a < 6; ++a) acc.s[a] = dd_add(acc.s[a], v[a]);
+    if (dd_gt(v[6], acc.fmax)) acc.fmax = v[6];
+    if (dd_gt(acc.fmin, v[7])) acc.fmin = v[7];
+    if (dd_gt(acc.dmin, v[8])) acc.dmin = v[8];
+    acc.bad += (int)v[9].hi;
+  }
+  resid_block_sums<RB>(acc, tot);
+  __syncthreads();
+  if (tid == 0) {
+    double v[10];
+    for (int a = 0; a < 10; ++a) v[a] = (double)tot[a].x + (double)tot[a].y;
+    residual_close(sc, v, N, M);
   }
 }
 
@@ -729,16 +1007,33 @@ cudaError_t launch_residual_dd(const float2* fdd, const float2* cdd, const doubl
   K.gx = ip.gx32;
   K.gy = ip.gy32;
   if (ip.mode && !(ip.gx32 && ip.gy32)) return cudaErrorInvalidValue;
-  // 32-row tiles (four points per thread), 8-row tiles on the smallest grids: a thread's four
-  // points follow each other, 20 us however few the blocks.  32-row / 8-row tiles, us: 20.5 / 12.1
-  // at 16 tiles (128^2), 21.3 / 15.9 at 64 (256^2), 20.9 / 17.0 at 80 (five of 128^2), but
-  // 22.3 / 24.9 at 144 (384^2) and 29.2 / 36.6 at 256 (512^2), where the block sums weigh more.
   const int mx = (M + RTX - 1) / RTX;
-  if ((long)mx * ((N + 31) / 32) * (bat.on ? bat.n : 1) > 96)
-    k_residual_dd<4><<<bgrid(dim3(mx, (N + 31) / 32), bat), 8 * RTX, 0, st>>>(
+  const long tiles = (long)mx * ((N + 31) / 32) * (bat.on ? bat.n : 1);
+  if (ip.mode) {
+    // 32-row tiles (four points per thread), 8-row tiles on the smallest grids, where a thread's
+    // four points in a row are the time
+    if (tiles > 96)
+      k_residual_dd<4><<<bgrid(dim3(mx, (N + 31) / 32), bat), 8 * RTX, 0, st>>>(
+          fdd, cdd, ua, ub, sel, N, M, K, Fraw, coef, partials, sc, bat);
+    else
+      k_residual_dd<1><<<bgrid(dim3(mx, (N + 7) / 8), bat), 8 * RTX, 0, st>>>(
+          fdd, cdd, ua, ub, sel, N, M, K, Fraw, coef, partials, sc, bat);
+    return cudaGetLastError();
+  }
+  // 16-row tiles by 256 threads (a pair of points each) while few blocks have to finish soon, by
+  // 128 threads (two pairs) on middling grids, 32-row tiles by 128 (four pairs: least halo and
+  // block sums) on large ones.  us, one GB300, in this order: 128^2 (16 tiles) 10.8 / 13.4 / 20.0,
+  // 384^2 (144) 16.3 / 17.9 / 22.0, 512^2 (256) 24.2 / 24.4 / 25.5, five of 256^2 (320) 29.7 / 29.4 /
+  // 31.8, five of 384^2 (720) 51.2 / 47.8 / 49.1, 1024^2 (1024) 71.1 / 67.0 / 63.6, 16 of 512^2
+  // (4096) 268 / 238 / 226; one point per thread took 11.4, 22.2, 28.2, 37.6, 55.5, 75.5 and 258.
+  if (tiles <= 256)
+    k_residual_dd2<8, 1, 2><<<bgrid(dim3(mx, (N + 15) / 16), bat), 8 * RTX, 0, st>>>(
+        fdd, cdd, ua, ub, sel, N, M, K, Fraw, coef, partials, sc, bat);
+  else if (tiles < 1000)
+    k_residual_dd2<4, 2, 4><<<bgrid(dim3(mx, (N + 15) / 16), bat), 4 * RTX, 0, st>>>(
         fdd, cdd, ua, ub, sel, N, M, K, Fraw, coef, partials, sc, bat);
   else
-    k_residual_dd<1><<<bgrid(dim3(mx, (N + 7) / 8), bat), 8 * RTX, 0, st>>>(
+    k_residual_dd2<4, 4, 4><<<bgrid(dim3(mx, (N + 31) / 32), bat), 4 * RTX, 0, st>>>(
         fdd, cdd, ua, ub, sel, N, M, K, Fraw, coef, partials, sc, bat);
   return cudaGetLastError();
 }
