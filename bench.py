@@ -794,7 +794,7 @@ def run_ours(args):
         "frac_of_bf16_peak": net_flops / (net_ms / 1000.0) / 1e12 / bf16_peak,
         "ms_through_ot_ws_mlp_forward": api_ms,
         "note": "ms_per_launch: graph-replayed back-to-back launches (CUDA events); the API "
-                "call adds a 4-byte flag reset and a synchronising read per call"}
+                "call adds a wait for the stream per call"}
     ws_info["ms_per_solve"] = prof["warmstart"][0]
     ws_info["launches_per_solve"] = prof["warmstart"][1]
     ws_info["alpha"] = stats[0]["ws_alpha"]
