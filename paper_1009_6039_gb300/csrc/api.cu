@@ -642,9 +642,14 @@ static int alloc_batch(ot_plan* p, int B) {
   if (!p->precision || B < 1 || B > 1024) return OT_EINVAL;
   const size_t P = (size_t)p->N * p->M;
   RET(alloc_tables(p));
-  // GMRES vector kernels: blocks per pair by its size (the pairs fill the GPU together)
-  long kb = (long)(P / 2048);
-  p->kblocks = (int)std::min<long>(std::max<long>(kb, 8), p->sms);
+  // GMRES vector kernels: three blocks per two SMs over all pairs, so that one wave streams the
+  // vectors (every update block finishes the multi-dot's sums of its pair first), but a block has
+  // 2048 to 16384 points of its pair.  Multi-dot + update at step 4, us, P / 2048 blocks per pair / this
+  // rule, one GB300: 5 pairs of 512^2 18.2 / 11.3, 16 of 512^2 68 / 40, 16 of 256^2 15.1 / 11.0, 100 of
+  // 128^2 33 / 21; 100 of 512^2 269 / 267 (with 2 blocks per pair 359).
+  const long each = std::max<long>(3L * p->sms / 2 / B, (long)(P / 16384));
+  p->kblocks = (int)std::min<long>(
+      std::max<long>(std::min<long>(each, std::max<long>((long)(P / 2048), 8)), 2), p->sms);
   // (an 8-row tile's ten partials per block at most)
   size_t np = std::max((size_t)residual_partial_blocks(p->N, p->M),
                        (size_t)((p->M + 31) / 32) * ((p->N + 7) / 8)) * 10;
