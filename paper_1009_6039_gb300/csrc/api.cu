@@ -131,8 +131,9 @@ static Bat btc(const ot_plan* p) {
   // The Arnoldi step's close in the update while the class has at most 2048 update blocks (each
   // finishes the multi-dot's sums, with FP64 scalars by one thread, which for hundreds of pairs
   // costs more than the close in the multi-dot's last block).  Multi-dot + update at step 4, us,
-  // close in the multi-dot / in the update: 5 pairs of 128^2 7.7 + 3.8 / 3.6 + 4.7, 5 of 512^2
-  // 14.0 + 9.1 / 8.5 + 10.4, 16 of 512^2 (2048 blocks) 41.4 + 35.7 / 32.8 + 37.8.
+  // close in the multi-dot / in the update, with P / 2048 blocks per pair: 5 pairs of 128^2 7.7 +
+  // 3.8 / 3.6 + 4.7, 5 of 512^2 14.0 + 9.1 / 8.5 + 10.4, 16 of 512^2 (2048 blocks) 41.4 + 35.7 /
+  // 32.8 + 37.8.
   b.split = b.on && (long)p->kblocks * p->batch <= 2048;
   return b;
 }
