@@ -262,8 +262,10 @@ __global__ void __launch_bounds__(TWX * (TH < 8 ? TH : 8), TH == 32 ? 3 : 4)
     red.s[5] += b2;
     if (finite_key(fn)) {
       red.s[0] += fn;
-      red.kmax = max(red.kmax, ordered_key(fr));
-      red.kmin = min(red.kmin, ordered_key(fr));
+      if (!nan_key(fr)) {  // (a NaN in f: the other points' extremes stand)
+        red.kmax = max(red.kmax, ordered_key(fr));
+        red.kmin = min(red.kmin, ordered_key(fr));
+      }
     } else {
       red.bad += 1;
     }
