@@ -57,6 +57,11 @@ __device__ __forceinline__ int floor_frac(double x, double* t) {
   return k;
 }
 
+// the result of an operation is NaN (a quiet one: its high word tells)
+__device__ __forceinline__ bool nan_result(double x) {
+  return (__double2hiint(x) & 0x7fffffff) > 0x7ff00000;
+}
+
 // sums of six values, a maximum, two minima and a count over the block; the block's results are
 // in the first lanes of warp 0: lane v < 6 holds sum v in s[0], lane 0 the others
 struct Red {
@@ -262,7 +267,7 @@ __global__ void __launch_bounds__(TWX * (TH < 8 ? TH : 8), TH == 32 ? 3 : 4)
     red.s[5] += b2;
     if (finite_key(fn)) {
       red.s[0] += fn;
-      if (!nan_key(fr)) {  // (a NaN in f: the other points' extremes stand)
+      if (!nan_result(fr)) {  // (a NaN in f: the other points' extremes stand)
         red.kmax = max(red.kmax, ordered_key(fr));
         red.kmin = min(red.kmin, ordered_key(fr));
       }
