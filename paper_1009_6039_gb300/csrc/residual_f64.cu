@@ -30,7 +30,7 @@ struct ResidK {
   double MM, NN, MNh;  // M^2/12, N^2/12, M N / 144
   double Mg, Ng;       // M/12, N/12 (of the 6 w, 2 w' weights)
   double w3;           // 1/(9 M N): Simpson weights (2 or 4 per axis) x this
-  double Md, Nd;       // M, N
+  double Md, Nd, iM, iN;  // M, N, 1/M, 1/N
   int nob;             // 1: the simplified operator (b = 0, Sec. 3.3 remark)
   // interpolation of g (Sec. 4 intro; Sec. 5.2, 5.3): 0 cubic B-spline of the coefficients c;
   // 1 bilinear, 2 nearest node of the grid values (then c = g) and of the grid gradient gx, gy
@@ -44,7 +44,7 @@ __device__ __forceinline__ int wrap_any(int a, int L) {
   return r < 0 ? r + L : r;
 }
 
-// floor of x and the fraction t = x - floor(x) in [0, 1] (for any x: the index is wrapped later)
+// floor of x and the fraction t = x - floor(x) in [0, 1], |x| < 2^30
 __device__ __forceinline__ int floor_frac(double x, double* t) {
   const double m = x + 6755399441055744.0;  // 1.5 x 2^52: the nearest integer in the low bits
   int k = __double2loint(m);
@@ -55,6 +55,24 @@ __device__ __forceinline__ int floor_frac(double x, double* t) {
   }
   *t = r;
   return k;
+}
+// displaced by 2^30 cells or more, or not finite
+__device__ __forceinline__ bool far(double x) {
+  return (__double2hiint(x) & 0x7fffffff) >= 0x41d00000;
+}
+// cell of the position n + x, in [0, L), and the fraction, for any x (Ld = L, iL = 1 / L).  A far
+// position (a diverging iterate's) is reduced first: each x - floor(x / L) L is exact, two leave less
+// than 2^30 of any |x| < 2^100, and beyond, where neighbouring doubles are 2^47 cells apart, node 0
+// is taken.
+__device__ __forceinline__ int cell(int n, double x, int L, double Ld, double iL, double* t) {
+  if (far(x)) {
+    x = __dadd_rn((double)n, x);
+    n = 0;
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) x = fma(-floor(x * iL), Ld, x);
+    if (far(x)) x *= 0.0;  // (NaN stays NaN, infinity becomes NaN)
+  }
+  return wrap_any(n + floor_frac(x, t), L);
 }
 
 // the result of an operation is NaN (a quiet one: its high word tells)
@@ -189,7 +207,7 @@ __global__ void __launch_bounds__(TWX * (TH < 8 ? TH : 8), TH == 32 ? 3 : 4)
     const double det = fma(axx, ayy, -(uxy * uxy));
     // g at the displaced point x + grad u, in grid units, periodic cubic B-spline
     double t, s;
-    const int j0 = wrap_any(j + floor_frac(dx, &t), M), i0 = wrap_any(i + floor_frac(dy, &s), N);
+    const int j0 = cell(j, dx, M, K.Md, K.iM, &t), i0 = cell(i, dy, N, K.Nd, K.iN, &s);
     int jj[4], ii[4];
     jj[0] = j0 == 0 ? M - 1 : j0 - 1;
     jj[1] = j0;
@@ -389,6 +407,8 @@ cudaError_t launch_residual(const double* f, const double* c, const double* ua, 
   ResidK K;
   K.Md = (double)M;
   K.Nd = (double)N;
+  K.iM = 1.0 / K.Md;
+  K.iN = 1.0 / K.Nd;
   K.MM = (double)M * (double)M / 12.0;
   K.NN = (double)N * (double)N / 12.0;
   K.MNh = (double)M * (double)N / 144.0;
