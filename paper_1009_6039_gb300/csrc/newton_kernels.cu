@@ -1129,9 +1129,7 @@ __global__ void k_gmres_init(const double* __restrict__ Fraw, const T* __restric
       sc->iters = 0;
       sc->cycles = 0;
       sc->converged = (beta == 0.0);
-      sc->relres = 0.0;
     } else {
-      sc->relres = sc->bnorm > 0.0 ? beta / sc->bnorm : 0.0;
       if (beta <= sc->eta * sc->bnorm) sc->converged = 1;
     }
     sc->beta = beta;
@@ -1196,7 +1194,6 @@ __device__ void arnoldi_close(DevScalars* sc, int j, double hn, bool weak) {
   sc->gv[j] = sc->cs[j] * sc->gv[j];
   sc->iters += 1;
   sc->jend = j + 1;
-  sc->relres = fabs(sc->gv[j + 1]) / sc->bnorm;
   if (weak) {
     sc->cycle_done = 1;
   } else if (fabs(sc->gv[j + 1]) <= sc->eta * sc->bnorm || hn == 0.0) {

@@ -45,7 +45,6 @@ struct DevScalars {
   double scale[OTGB_MAXM + 1];  // V_i is stored unnormalised; v_i = scale[i] * V_i
   double h2[OTGB_MAXM];         // second Gram-Schmidt pass (reorthogonalisation)
   double hcol[OTGB_MAXM];       // column j of H before the rotations (the update's weights)
-  double relres;
   int j, jend, m, cycle_done, converged, iters, cycles;
   int jd;  // FP32 single-reduction step: the step index of the last multi-dot (for the update)
   double eta, tau;
