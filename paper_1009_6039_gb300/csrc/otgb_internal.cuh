@@ -45,6 +45,9 @@ struct DevScalars {
   double scale[OTGB_MAXM + 1];  // V_i is stored unnormalised; v_i = scale[i] * V_i
   double h2[OTGB_MAXM];         // second Gram-Schmidt pass (reorthogonalisation)
   double hcol[OTGB_MAXM];       // column j of H before the rotations (the update's weights)
+  // 2-norm of the last vector normalised by launch_normalize (here, so that the step's integers below
+  // lie 24 bytes past a 32-byte sector's start: 16 bytes past it plan sets take 1 % longer)
+  double pw_norm;
   int j, jend, m, cycle_done, converged, iters, cycles;
   int jd;  // FP32 single-reduction step: the step index of the last multi-dot (for the update)
   double eta, tau;
@@ -84,7 +87,6 @@ struct DevScalars {
   int active, in_cycle, halve;
   int excluded;       // the pair sits out this launch of the batched graph (a retry of others)
   double gauge_mean;  // mean removed by the final gauge of a batched solve
-  double pw_norm;     // 2-norm of the last vector normalised by launch_normalize
   // BiCG on the finite-difference system (Sec. 4.1): rho = (r, r*), alpha, beta, ||b||^2,
   // ||r||^2, the sums of p and p* (the all-ones part of A~ = A + 1 1^T); status 0 converged,
   // 1 iteration cap, 2 breakdown; done stops the self-skipping iteration kernels
