@@ -172,12 +172,12 @@ extern "C" {
                                    next step's product (the update forms v_(j+1) row by row
                                    and transforms it in place of a separate row pass); 0: two
                                    launches.  Same arithmetic either way (bit for bit) */
-#define OT_OPT_THETA_PAIRS 32   /* mixed mode, double-float theta (OT_OPT_THETA_FP64 = 2),
-                                   single problem: 1 (default) runs theta's column and row
+#define OT_OPT_THETA_PAIRS 32   /* mixed mode, double-float theta (OT_OPT_THETA_FP64 = 2):
+                                   1 (default) runs theta's column and row
                                    passes and the learned start's Poisson solves on column /
                                    row pairs with packed FP32 arithmetic where the sizes allow
-                                   (N a power of two in 256..2048 and M a multiple of 4 for the
-                                   column pass, M/2 a power of two in 256..1024 and N even for
+                                   (N = 2^a or 3 2^a in 96..2048 and M a multiple of 4 for the
+                                   column pass, M/2 = 2^a or 3 2^a in 64..1024 and N even for
                                    the row pass); 0: one column / row per thread group.  The
                                    double-float inverse transforms are the same arithmetic per
                                    column either way; the FP32 forward column transform
@@ -190,11 +190,12 @@ extern "C" {
                                    thread (where the size allows, else a variant that does);
                                    + 64: the generic column pass with 4 columns per block;
                                    + 256: the column pass on column pairs with packed FP32
-                                   arithmetic (N a power of two in 256..2048, M a multiple
+                                   arithmetic (N = 2^a or 3 2^a in 96..2048, M a multiple
                                    of 4; elsewhere c = 3); + 512: the combine pass on row
-                                   pairs (M/2 a power of two in 256..1024, N even; elsewhere
+                                   pairs (M/2 = 2^a or 3 2^a in 64..1024, N even; elsewhere
                                    b = 3); + 1024: the row R2C pass and the fused Arnoldi
-                                   update on row pairs (the same sizes; elsewhere r = 3);
+                                   update on row pairs (as the combine pass, M/2 >= 96;
+                                   elsewhere r = 3);
                                    turns OT_OPT_AUTOTUNE off */
 
 /* Kernel classes of the profile (ot_plan_get_profile). */

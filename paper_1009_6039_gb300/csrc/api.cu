@@ -128,12 +128,14 @@ static Bat btc(const ot_plan* p) {
   b.n = p->batch;
   b.slab = p->slab;
   b.mask = b.on ? p->cur_mask : MASK_ALL;
-  // The Arnoldi step's close in the update while the class has at most 2048 update blocks (each
-  // finishes the multi-dot's sums, with FP64 scalars by one thread, which for hundreds of pairs
-  // costs more than the close in the multi-dot's last block).  Multi-dot + update at step 4, us,
-  // close in the multi-dot / in the update, with P / 2048 blocks per pair: 5 pairs of 128^2 7.7 +
-  // 3.8 / 3.6 + 4.7, 5 of 512^2 14.0 + 9.1 / 8.5 + 10.4, 16 of 512^2 (2048 blocks) 41.4 + 35.7 /
-  // 32.8 + 37.8.
+  // The Arnoldi step's close in the update while the class has at most 2048 update blocks, each of
+  // which finishes the multi-dot's sums first (FP64 scalars by one thread); the first one only closes
+  // the step.  Multi-dot + update at step 4 with alloc_batch's blocks, us, close in the multi-dot / in
+  // the update, one GB300: 5 pairs of 128^2 12.2 / 8.3, of 256^2 12.7 / 8.7, of 512^2 15.6 / 11.2; 16 of
+  // them 12.2 / 8.3, 15.3 / 10.4, 47.6 / 42.8; 100 of 128^2 (2 blocks a pair: one worker) 18.2 / 17.0, of
+  // 256^2 82 / 73, of 512^2 249 / 237; 1024 of 128^2 (2048 blocks) 184 / 171.  The other way round
+  // only at 192^2 with 2 blocks a pair: 100 pairs 40 / 47, 300 pairs 113 / 115.  Above the line the
+  // two are within 3 %: 300 of 512^2 672 / 661, 1024 of 256^2 586 / 571.
   b.split = b.on && (long)p->kblocks * p->batch <= 2048;
   return b;
 }
@@ -644,10 +646,12 @@ static int alloc_batch(ot_plan* p, int B) {
   const size_t P = (size_t)p->N * p->M;
   RET(alloc_tables(p));
   // GMRES vector kernels: three blocks per two SMs over all pairs, so that one wave streams the
-  // vectors (every update block finishes the multi-dot's sums of its pair first), but a block has
-  // 2048 to 16384 points of its pair.  Multi-dot + update at step 4, us, P / 2048 blocks per pair / this
-  // rule, one GB300: 5 pairs of 512^2 18.2 / 11.3, 16 of 512^2 68 / 40, 16 of 256^2 15.1 / 11.0, 100 of
-  // 128^2 33 / 21; 100 of 512^2 269 / 267 (with 2 blocks per pair 359).
+  // vectors (every update block finishes the multi-dot's sums of its pair first).  Clamps, per pair:
+  // a block per 16384 points at least, a block per 2048 points at most (8 blocks on grids below
+  // 128^2), and in any case 2 blocks (the split close's first one works on no points) to one per SM.
+  // Multi-dot + update at step 4 with the split close, us, P / 2048 blocks per pair / this rule,
+  // one GB300: 5 pairs of 512^2 17.7 / 11.2, 16 of 512^2 62 / 43, 16 of 256^2 14.7 / 10.4, 100 of 128^2
+  // 21.5 / 17.0, 100 of 256^2 102 / 73, 100 of 512^2 354 / 237.
   const long each = std::max<long>(3L * p->sms / 2 / B, (long)(P / 16384));
   p->kblocks = (int)std::min<long>(
       std::max<long>(std::min<long>(each, std::max<long>((long)(P / 2048), 8)), 2), p->sms);
@@ -1359,8 +1363,9 @@ static int run_arnoldi_step(ot_plan* p, int j, const int* skip) {
            launch_gmres_update_r2c((float*)V, (const float*)w, P, p->partials, p->kblocks,
                                    p->sc, (float2*)p->spec, p->N, p->M, p->tb32, p->stream));
   } else {
-    // the multi-dot closes the step (norm by Pythagoras, Givens); the update only forms
-    // v_(j+1) and is skipped when the cycle ends
+    // the update finishes the multi-dot's sums, its block 0 closes the step (norm by Pythagoras,
+    // Givens) and the others form v_(j+1); a plan set's large classes (btc): the multi-dot's last
+    // block closes the step, and the update is skipped when the cycle ends
     LAUNCH(p, OT_PROF_GMRES_UPDATE, j, 1,
            launch_gmres_update<T>(V, w, P, p->partials, p->sc, p->kblocks, p->stream, 3,
                                   btc(p)));
@@ -2997,7 +3002,7 @@ static int set_build(ot_plan_set* s) {
     const int B = (int)c.idx.size();
     RET(ot_plan_create(&c.p, c.N, c.M, s->tau, s->tol));
     RET(ot_plan_set_option(c.p, OT_OPT_PRECISION, 1));
-    c.p->autotune = 0;  // the batched passes are the generic kernels
+    c.p->autotune = 0;  // the batched passes are fixed: pairs where the size allows, else generic
     for (auto& kv : s->opts)
       if (kv.first != OT_OPT_TAU && kv.first != OT_OPT_TOL)
         RET(ot_plan_set_option(c.p, kv.first, kv.second));

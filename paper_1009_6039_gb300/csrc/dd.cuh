@@ -27,9 +27,11 @@ __device__ __forceinline__ dd dd_make(float hi, float lo) { return dd(hi, lo); }
 // warp instruction per 16 clocks and SM on GB300), four of them per split and three per sum, which
 // had become a third to a half of the time of the passes that read or write FP64 planes.
 //
-// The split with cvt instructions (hi rounds ties to even), also for a kernel that has no registers
-// left for the integer form: the residual kernel would spill 108 bytes at its 80 registers and take
-// 79 instead of 75 us at 1024x1024.
+// The split with cvt instructions (hi rounds ties to even): values outside the integer form's range,
+// and the mixed residuals' reading of u, chosen when a form of theirs would have spilled with the
+// integer split.  It no longer does, and the integer split is the faster one there too (us, cvt /
+// integer: cubic 10.7 / 10.2 at 128^2, 24.4 / 23.3 at 512^2, 66.2 / 63.4 at 1024^2, 255.6 / 252.4 at
+// 2048^2; bilinear 57.3 / 55.0, nearest node 51.9 / 49.5 at 1024^2).
 __device__ __forceinline__ dd dd_from_double_cvt(double a) {
   const float h = __double2float_rn(a);
   return dd{h, __double2float_rn(a - (double)h)};

@@ -349,14 +349,7 @@ cudaError_t launch_translate_inputs(const double* f, const double* g, double* ft
   return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------------------------------
-// Residual + coefficients (K1).  A block covers a 32 x 32 tile (each thread 4 points, one
-// column); u is staged in shared memory with a periodic halo of 2 for the 4th-order
-// centred stencils.  GB300's FP64 rate is low, so the kernel avoids FP64 divisions (all
-// reciprocal factors come in as arguments), integer divisions in the inner code, and in the
-// mixed mode evaluates the gradient of the interpolant (which enters only the Jacobian, not
-// the residual) in FP32.
-// ---------------------------------------------------------------------------------------
+// indices modulo L
 __device__ __forceinline__ int wrapi(int a, int L) {
   int r = a % L;
   return r < 0 ? r + L : r;
@@ -367,8 +360,9 @@ __device__ __forceinline__ int wrap_near(int a, int L) {  // a in [-L, 2L)
 }
 
 // ---------------------------------------------------------------------------------------
-// Mixed-mode residual: the same evaluation with every FP64-accuracy quantity (the stencils
-// of u, the displaced point, the B-spline value gather, det, f_n and F) in double-float
+// Mixed-mode residual + coefficients (FP64: residual_f64.cu).  u is staged in shared memory with a
+// periodic halo of 2 for the 4th-order centred stencils; every FP64-accuracy quantity (the stencils
+// of u, the displaced point, the B-spline value gather, det, f_n and F) is in double-float
 // arithmetic on the FP32 pipes (dd.cuh, unit round-off 2^-48), the Jacobian coefficients,
 // the interpolant's gradient and the Simpson sums in FP32.  Inputs: u (FP64), f and c
 // pre-split into (hi, lo) float pairs; output F_raw in FP64.
@@ -379,7 +373,8 @@ struct ResidConstsDD {
   float M, N;
   float w3M, w3N;            // 1/(3M), 1/(3N)
   int nob;                   // 1: the simplified operator (b = 0)
-  int interp;                // as ResidConsts::interp (then cdd = g as (hi, lo) pairs)
+  // interpolation of g: 0 cubic B-spline; 1 bilinear, 2 nearest node (then cdd = g as (hi, lo) pairs)
+  int interp;
   const float* gx;           // grid gradient of g (FP32: the Jacobian only)
   const float* gy;
 };
@@ -1011,7 +1006,9 @@ cudaError_t launch_residual_dd(const float2* fdd, const float2* cdd, const doubl
   const long tiles = (long)mx * ((N + 31) / 32) * (bat.on ? bat.n : 1);
   if (ip.mode) {
     // 32-row tiles (four points per thread), 8-row tiles on the smallest grids, where a thread's
-    // four points in a row are the time
+    // four points in a row are the time.  8 / 32 rows, us, one GB300, bilinear: 10.4 / 16.3 at 128^2,
+    // 13.2 / 16.6 at 256^2, 15.9 / 17.4 at 384 x 256 (96 tiles), 19.2 / 17.8 at 384^2 (144), 94 / 57 at
+    // 1024^2; nearest node 15.3 / 16.3 and 18.4 / 16.6 at 96 and 144 tiles
     if (tiles > 96)
       k_residual_dd<4><<<bgrid(dim3(mx, (N + 31) / 32), bat), 8 * RTX, 0, st>>>(
           fdd, cdd, ua, ub, sel, N, M, K, Fraw, coef, partials, sc, bat);
@@ -1072,9 +1069,11 @@ cudaError_t launch_subtract_mean(double* u, int N, int M, double* partials, DevS
 
 // ---------------------------------------------------------------------------------------
 // GMRES(m) (Sec. 4.2).  The basis V_i is stored unnormalised with v_i = scale[i] V_i so
-// that no kernel pass is spent on normalisation.  Arnoldi uses classical Gram-Schmidt:
-// one fused multi-dot pass and one fused update pass (which also forms ||w||^2).  The
-// Givens rotations and the small triangular solve run in the last block on the device.
+// that no kernel pass is spent on normalisation.  Arnoldi uses classical Gram-Schmidt: a
+// multi-dot pass (V_i.w and w.w) and an update pass, whose first block also closes the step: the
+// norm of the new vector by Pythagoras, the Givens rotation.  A plan set's large classes close it in
+// the multi-dot's last block, and with reorthogonalisation (two such rounds) the second
+// update's last block does, from the new vector's own norm.
 // Every kernel returns at once when the current cycle is finished (cycle_done), so a fixed
 // sequence of launches can be queued without host round trips.
 // ---------------------------------------------------------------------------------------
@@ -1393,7 +1392,7 @@ __device__ __forceinline__ void update_j(T* __restrict__ V, const T* __restrict_
     acc += x * x;
   }
   // mode 1: first of two passes, the norm follows the second; mode 3: the step was closed
-  // by block 0 above (single problems) or by the multi-dot (a plan set's classes)
+  // by block 0 above or by the multi-dot (a plan set's large classes)
   if (mode == 1 || mode == 3) {
     if (mode == 3 && split && !closer && blockIdx.x == 0 && threadIdx.x == 0) {
 #pragma unroll

@@ -49,7 +49,7 @@ struct DevScalars {
   // lie 24 bytes past a 32-byte sector's start: 16 bytes past it plan sets take 1 % longer)
   double pw_norm;
   int j, jend, m, cycle_done, converged, iters, cycles;
-  int jd;  // FP32 single-reduction step: the step index of the last multi-dot (for the update)
+  int jd;  // split Arnoldi step: the step index of the last multi-dot (for the update)
   double eta, tau;
   double tau_switch;  // tau schedule: tau becomes 1 once res_inf < tau_switch (0: off)
   // Newton control, resident on the device for the graph-launched solve
@@ -241,7 +241,8 @@ cudaError_t launch_col_pair(const float2* spec, float2* o0, float2* o1, float2* 
 
 bool fft_length_supported(int L);
 
-// (bat: a batched launch, the generic kernels only; msc: the pair scalars its mask reads)
+// (bat: a batched launch, FP32 only: the pair passes where the size allows and the pairs' scalars,
+// which its mask reads, are given as msc or sc; else the generic kernels)
 template <typename T>
 cudaError_t launch_row_r2c(const T* x, size_t x_stride, const int* jptr, const double* scale,
                            C2<T>* spec, int N, int M, const SpecTables& tb, const int* skip,
@@ -446,8 +447,8 @@ size_t ws_train_scratch_floats();  // per block
 size_t ws_train_part_floats();     // per block
 cudaError_t launch_ws_source(const double* f, const double* g, double* src, long P,
                              cudaStream_t st);
-// transport outputs: *dist (device) = mean |grad u|^2 f, div (optional) = u_xx + u_yy;
-// partials: one (hi, lo) pair per 32 x 32 tile
+// transport outputs: *dist (device or pinned host memory) = mean |grad u|^2 f, div (optional) = u_xx +
+// u_yy; partials: one (hi, lo) pair per tile of 32 columns and 8 or 32 rows
 cudaError_t launch_transport(const double* f, const double* u, int N, int M, double* div,
                              double* partials, unsigned int* ticket, double* dist,
                              cudaStream_t st);

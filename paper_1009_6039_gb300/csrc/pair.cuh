@@ -3,7 +3,9 @@
 // complex numbers in one register pair, the imaginary parts in another), their butterflies
 // and Stockham stages, and the 16-byte-element shared-memory swizzle
 // i ^ ((i >> 2) & 7), under which every stage's reads and writes of a quarter warp fall in
-// distinct bank groups (checked for the radix-4 / radix-2 stages of lengths 256 .. 2048).
+// distinct bank groups for the powers of two (computed for 64 .. 2048, one and two pairs per block).
+// With a factor 3 (96 .. 1536) the reads do too, and the writes from the fourth stage on; those of
+// the first two stages meet threefold, those of the third twofold (one pair) or not (two).
 //
 // Lengths: powers of two by L / 4 threads (4 elements each), and 3 * 2^a by L / 3: the first
 // stage has radix 3, a butterfly per thread; in the others the first L / 4 threads work, as for

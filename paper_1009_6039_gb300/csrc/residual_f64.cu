@@ -2,9 +2,9 @@
 // that shifts the residual by the mass translation and sums its squares.
 //
 // What bounds the residual: FP64 instructions (two per clock and SM on GB300, see
-// spectral_f64.cu).  A point takes about 118: stencils 22, displaced position 8, spline weights
+// spectral_f64.cu).  A point takes about 121: stencils 22, displaced position 8, spline weights
 // 26, 16-tap gather of the value and the gradient 44, determinant, f_n, F and coefficients 12,
-// sums 6, so 197 us at 1024^2 with every SM busy.  What keeps the count down:
+// sums 6, and the tile's halo, so 202 us at 1024^2 with every SM busy.  What keeps the count down:
 //   - 1 + u_xx and 1 + u_yy in one FMA each, M u_x and N u_y straight from the differences (u_x
 //     itself is not needed), the floor by adding 1.5 x 2^52;
 //   - the weights as 6 w and 2 w' (13 instructions per axis), their factors in G's and in the
@@ -15,7 +15,8 @@
 // A block covers 32 columns x TH rows: 32 where that gives four blocks per SM, else 8 or 4, so
 // that small grids reach every SM.  Measured (us per launch under ncu, one
 // GB300; before: 160 instructions per point, 32-row tiles): 1024^2 349 -> 256 (FP64 pipe 85 % busy),
-// 250 x 333 65 -> 35.
+// 250 x 333 65 -> 35.  The test for far displacements (two per point) takes 1 to 2 % of that:
+// graph-replayed 252.0 -> 257.0 at 1024^2, 27.3 -> 27.5 at 256^2.
 #include <math.h>
 
 #include "otgb_internal.cuh"
