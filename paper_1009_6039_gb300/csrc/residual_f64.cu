@@ -2,21 +2,21 @@
 // that shifts the residual by the mass translation and sums its squares.
 //
 // What bounds the residual: FP64 instructions (two per clock and SM on GB300, see
-// spectral_f64.cu).  A point takes about 121: stencils 22, displaced position 8, spline weights
+// spectral_f64.cu).  A point takes about 119: stencils 22, displaced position 6, spline weights
 // 26, 16-tap gather of the value and the gradient 44, determinant, f_n, F and coefficients 12,
-// sums 6, and the tile's halo, so 202 us at 1024^2 with every SM busy.  What keeps the count down:
+// sums 6, and the tile's halo, so 198 us at 1024^2 with every SM busy.  What keeps the count down:
 //   - 1 + u_xx and 1 + u_yy in one FMA each, M u_x and N u_y straight from the differences (u_x
-//     itself is not needed), the floor by adding 1.5 x 2^52;
+//     itself is not needed), the floor and the fraction by FMAs with a constant (cell);
 //   - the weights as 6 w and 2 w' (13 instructions per axis), their factors in G's and in the
 //     determinant's scale;
 //   - maxima, minima and finiteness on the integer pipe (doubles as ordered integers), the
 //     Simpson weight of a thread's points (all of one parity) taken once at the end;
 //   - block sums of six values folded over a warp (9 additions instead of 30).
 // A block covers 32 columns x TH rows: 32 where that gives four blocks per SM, else 8 or 4, so
-// that small grids reach every SM.  Measured (us per launch under ncu, one
-// GB300; before: 160 instructions per point, 32-row tiles): 1024^2 349 -> 256 (FP64 pipe 85 % busy),
-// 250 x 333 65 -> 35.  The test for far displacements (two per point) takes 1 to 2 % of that:
-// graph-replayed 252.0 -> 257.0 at 1024^2, 27.3 -> 27.5 at 256^2.
+// that small grids reach every SM.  Measured (us per launch under ncu, one GB300; before: 160
+// instructions per point, 32-row tiles): 1024^2 349 -> 256 (FP64 pipe 85 % busy), 250 x 333 65 -> 35.
+// Graph-replayed, with the floor from the nearest integer -> rounded down, with the test for far
+// displacements: 1024^2 251.7 -> 248.9, 256^2 27.2 -> 26.9.
 #include <math.h>
 
 #include "otgb_internal.cuh"
@@ -45,35 +45,35 @@ __device__ __forceinline__ int wrap_any(int a, int L) {
   return r < 0 ? r + L : r;
 }
 
-// floor of x and the fraction t = x - floor(x) in [0, 1], |x| < 2^30
-__device__ __forceinline__ int floor_frac(double x, double* t) {
-  const double m = x + 6755399441055744.0;  // 1.5 x 2^52: the nearest integer in the low bits
-  int k = __double2loint(m);
-  double r = x - (m - 6755399441055744.0);
-  if (__double2hiint(r) < 0) {
-    r += 1.0;
-    k -= 1;
-  }
-  *t = r;
-  return k;
-}
-// displaced by 2^30 cells or more, or not finite
+// 1.5 x 2^52 + 2^31: a sum with it, rounded down, holds the floor k as k + 2^31 in its low word, and its
+// high word is kNear for -2^31 <= k < 2^31 alone
+constexpr double kMagic = 6755399441055744.0 + 2147483648.0;
+constexpr int kNear = 0x43380000;
+// 2^30 or more in size, or not finite
 __device__ __forceinline__ bool far(double x) {
   return (__double2hiint(x) & 0x7fffffff) >= 0x41d00000;
 }
-// cell of the position n + x, in [0, L), and the fraction, for any x (Ld = L, iL = 1 / L).  A far
-// position (a diverging iterate's) is reduced first: each x - floor(x / L) L is exact, two leave less
-// than 2^30 of any |x| < 2^100, and beyond, where neighbouring doubles are 2^47 cells apart, node 0
-// is taken.
-__device__ __forceinline__ int cell(int n, double x, int L, double Ld, double iL, double* t) {
-  if (far(x)) {
-    x = __dadd_rn((double)n, x);
+// Cell of the position n + d s, in [0, L), and the fraction t in [0, 1], for any displacement d s (0 <=
+// n < L, iL = 1 / L).  The product enters the floor and the fraction unrounded: two FMAs, and one
+// test of the high word for displacements beyond an int (a diverging iterate's).  Those positions are
+// reduced first: each x - floor(x / L) L is exact, two leave less than 2^30 of any |x| < 2^100, and
+// beyond, where neighbouring doubles are 2^47 cells apart, node 0 is taken.
+__device__ __forceinline__ int cell(int n, double d, double s, int L, double Ld, double iL,
+                                    double* t) {
+  double m = __fma_rd(d, s, kMagic);
+  if (__double2hiint(m) == kNear) {
+    *t = fma(d, s, -(m - kMagic));
+  } else {
+    double x = __dadd_rn((double)n, __dmul_rn(d, s));
     n = 0;
 #pragma unroll 1
     for (int k = 0; k < 2; ++k) x = fma(-floor(x * iL), Ld, x);
     if (far(x)) x *= 0.0;  // (NaN stays NaN, infinity becomes NaN)
+    m = __dadd_rd(x, kMagic);
+    *t = x - (m - kMagic);
   }
-  return wrap_any(n + floor_frac(x, t), L);
+  const int j = wrap_any((int)((unsigned)__double2loint(m) ^ 0x80000000u), L) + n;
+  return j >= L ? j - L : j;
 }
 
 // the result of an operation is NaN (a quiet one: its high word tells)
@@ -196,9 +196,8 @@ __global__ void __launch_bounds__(TWX * (TH < 8 ? TH : 8), TH == 32 ? 3 : 4)
     const int r = ty + 2, q = tx + 2;
     const double u0 = tile[r][q], xm2 = tile[r][q - 2], xm1 = tile[r][q - 1],
                  xp1 = tile[r][q + 1], xp2 = tile[r][q + 2];
-    // M u_x, N u_y (grid cells); 1 + u_xx, 1 + u_yy; u_xy
-    const double dx = (fma(-8.0, xm1, fma(8.0, xp1, -xp2)) + xm2) * K.MM;
-    const double dy = dyt[ty][q] * K.NN;
+    // M u_x, N u_y (grid cells) over MM, NN; 1 + u_xx, 1 + u_yy; u_xy
+    const double dx = fma(-8.0, xm1, fma(8.0, xp1, -xp2)) + xm2, dy = dyt[ty][q];
     const double axx = fma(fma(16.0, xm1, fma(-30.0, u0, fma(16.0, xp1, -xp2))) - xm2, K.MM, 1.0);
     const double ayy = fma(fma(16.0, tile[r - 1][q],
                                fma(-30.0, u0, fma(16.0, tile[r + 1][q], -tile[r + 2][q]))) -
@@ -208,7 +207,7 @@ __global__ void __launch_bounds__(TWX * (TH < 8 ? TH : 8), TH == 32 ? 3 : 4)
     const double det = fma(axx, ayy, -(uxy * uxy));
     // g at the displaced point x + grad u, in grid units, periodic cubic B-spline
     double t, s;
-    const int j0 = cell(j, dx, M, K.Md, K.iM, &t), i0 = cell(i, dy, N, K.Nd, K.iN, &s);
+    const int j0 = cell(j, dx, K.MM, M, K.Md, K.iM, &t), i0 = cell(i, dy, K.NN, N, K.Nd, K.iN, &s);
     int jj[4], ii[4];
     jj[0] = j0 == 0 ? M - 1 : j0 - 1;
     jj[1] = j0;
