@@ -441,6 +441,29 @@ static void transform_roots(int L, std::vector<double>& out) {
   for (int E : {4, 8, 12}) stage_roots(L, E, out);
 }
 
+// The FP64 passes' butterfly table (spectral_f64.cu) of length L, in the place of the stage table for E
+// = 4 behind the base table at tw: the stages of E = 4 or, with a factor 3, of E = 12, a twiddle c + i q
+// (r = 1 and, of radix 4, r = 2) as the larger of its parts and the ratio of the two: (c, q / c), or turned
+// (q, -c / q) for angles between an eighth and three eighths of a circle.
+static void fill_butterflies(int L, double* tw) {
+  const double* src = tw + 2 * (size_t)(L % 3 == 0 ? 3 : 1) * L;
+  double* t = tw + 2 * (size_t)L;
+  int Ns = L % 3 == 0 ? 3 : 1;
+  for (int rem = L / Ns; rem > 1;) {
+    const int R = rem % 4 == 0 ? 4 : 2;
+    for (int r = 1; r <= R / 2; ++r)
+      for (int k = 0; k < Ns; ++k) {
+        const size_t i = (size_t)(Ns - 1) + (size_t)(r - 1) * Ns + k;
+        const double c = src[2 * i], q = src[2 * i + 1];
+        const bool turned = 8 * k * r > R * Ns && 8 * k * r < 3 * R * Ns;
+        t[2 * i] = turned ? q : c;
+        t[2 * i + 1] = turned ? -c / q : q / c;
+      }
+    Ns *= R;
+    rem /= R;
+  }
+}
+
 // (s1, s2) of frequency index k of length L (k <= L/2 for the half axis): spectral
 // 2 pi k (0 at Nyquist) and -(2 pi k)^2 (Sec. 4.2, reading R4), or the Fourier symbols of the
 // 4th-order stencils (8 sin t - sin 2t) L / 6 and (-2 cos 2t + 32 cos t - 30) L^2 / 12,
@@ -531,8 +554,11 @@ static int alloc_tables(ot_plan* p) {
   roots(p->M, (int)L, tw);
   transform_roots(p->N, tw);
   const size_t ntw = tw.size() / 2;
+  std::vector<double> tw64(tw);
+  fill_butterflies((int)L, tw64.data());
+  fill_butterflies(p->N, tw64.data() + 2 * 5 * L);
   CK(cudaMalloc(&p->tw64, ntw * 16));
-  CK(cudaMemcpy(p->tw64, tw.data(), ntw * 16, cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(p->tw64, tw64.data(), ntw * 16, cudaMemcpyHostToDevice));
   std::vector<float> twf(tw.begin(), tw.end());
   CK(cudaMalloc(&p->tw32, ntw * 8));
   CK(cudaMemcpy(p->tw32, twf.data(), ntw * 8, cudaMemcpyHostToDevice));

@@ -5,10 +5,12 @@
 // takes 16 clocks; an FMA, an addition and a product cost the same), 32 times fewer than FP32,
 // while everything else (addresses, shared memory, L2) has 64 issue slots per FP64 warp
 // instruction.  So a pass costs its FP64 instruction count over the SMs that take part, and
-//   - every butterfly is in FMA form: a + w b in four FMAs and a - w b = 2 a - (a + w b) in
-//     two, 6 instructions with the twiddle included (a product, a sum and a difference take
-//     8), 3 per point and level whatever the radix, and the real split and its inverse take 5
-//     per frequency (8 and 6); radix 4, whose 56 to 80 registers leave room for many warps;
+//   - every butterfly is in FMA form: with the twiddle as w = g (1 + i r) or i g (1 + i r), |r| <= 1,
+//     u = b + i r b takes two FMAs and a +- g u four, 6 instructions with the twiddle included (a
+//     product, a sum and a difference take 8), 3 per point and level whatever the radix, and the real
+//     split and its inverse take 5 per frequency (8 and 6); radix 4, whose 56 to 80 registers leave
+//     room for many warps; the exchange of parts and signs that i g asks for is on the integer pipe (as
+//     negations in FP64 it cost 13 %);
 //   - a block holds one row or column (more rows only where the blocks would be tiny), so that
 //     all SMs get work and the last wave is a single row's;
 //   - the independent transforms of a row (five) or column (three) run side by side in thread
@@ -16,19 +18,20 @@
 // Measured on one GB300 (us per launch, graph-replayed; before: radix 8, one thread group per
 // row or column with its terms in sequence, product-and-sum butterflies) ->
 //             64^2           384 x 768        1024^2          2048^2
-//   row r2c   11.1 ->  6.0   23.5 -> 13.8     46.9 ->  36.7   188 -> 149
-//   column    62.0 -> 12.5    102 -> 50        202 -> 166     801 -> 715
-//   combine   48.4 ->  9.2    114 -> 67        230 -> 192     987 -> 793
-//   theta col 49.6 -> 16.5   64.3 -> 33        118 ->  93     442 -> 379
+//   row r2c   11.1 ->  5.8   23.5 -> 13.1     46.9 ->  35.0   188 -> 142
+//   column    62.0 -> 12.0    102 -> 49        202 -> 160     801 -> 674
+//   combine   48.4 ->  9.1    114 -> 65        230 -> 189     987 -> 771
+//   theta col 49.6 -> 15.9   64.3 -> 32        118 ->  91     442 -> 369
 // The FP64 pipe is 82 to 89 % busy in the 2048^2 passes (issue-bound), 10 to 20 % at 64^2
 // (latency: one row or column per SM).
 //
-// Rounding: 2 a - (a + w b) takes the sum's rounding into the difference, and radix 4 has more
-// twiddles than radix 8 had.  Relative rms error of a transform against long double, the product-and-sum
-// radix-8 form -> this one: on image-like densities 2.3e-16 -> 2.9e-16 forward and 2.2e-16 -> 3.2e-16
-// inverse at 512^2, 1.8e-16 -> 2.2e-16 at 64^2; on white noise 3.9e-16 -> 4.2e-16 at 512^2.  Product-and-sum
-// butterflies of radix 4 stay at 2.4e-16 / 2.4e-16 and 4.3e-16, and take 683 instead of 584 us for the two
-// 2048^2 transforms, 177 instead of 158 for the 384 x 768 operator.
+// Rounding: a + w b and a - w b are each rounded once at their own size.  (As s = a + w b in four FMAs and
+// 2 a - s in two, the sum's rounding enters the difference: an image-like density's low frequencies
+// leave theirs in the high ones.)  Relative rms error of a transform against long double, in 1e-16,
+// radix 8 with separate products and sums / 2 a - s / this form: forward 2.32 / 2.86 / 2.33 and inverse 2.24 /
+// 3.16 / 2.30 on smoothed noise and blobs at 512^2, 1.79 / 2.23 / 1.88 and 1.85 / 2.37 / 1.90 at 64^2, 3.87 /
+// 4.15 / 4.03 on white noise at 512^2.  Radix 4 with separate products and sums is no closer and takes 683 us for
+// the two 2048^2 transforms, 2 a - s 585, this form 562 (and 0.2 us a column pass more at 64^2, latency).
 #include "spectral.cuh"
 
 namespace otgb {
@@ -36,22 +39,38 @@ namespace {
 
 constexpr int kMaxThreads = 768;  // launch bound: 80 registers, for two to ten blocks per SM
 
-// the stage table of length L behind its base table
+// the butterflies' table of length L behind its base table (fill_butterflies of api.cu)
 __device__ __forceinline__ const double2* stage_table(const double2* tw, int L) {
-  return tw + (size_t)(L % 3 == 0 ? stage_table_slot<12>() : stage_table_slot<4>()) * L;
+  return tw + (size_t)stage_table_slot<4>() * L;
 }
 
 // ---------------------------------------------------------------------------------------
 // Butterflies.  SIGN -1 forward, +1 inverse (the twiddles are conjugated).
 // ---------------------------------------------------------------------------------------
-// (a, b) <- (a + w b, a - w b)
-template <int SIGN>
-__device__ __forceinline__ void bf(double2& a, double2& b, double2 w) {
-  const double wy = SIGN < 0 ? w.y : -w.y;
-  const double sx = fma(w.x, b.x, fma(-wy, b.y, a.x));
-  const double sy = fma(w.x, b.y, fma(wy, b.x, a.y));
-  b = make_double2(fma(2.0, a.x, -sx), fma(2.0, a.y, -sy));
-  a = make_double2(sx, sy);
+// A twiddle w = exp(-i t) as its larger part and the ratio of the two, so that a +- w b take three
+// FMAs a part and each is rounded once at its own size: not turned (|cos t| >= |sin t|), w = g (1 +
+// i r) with g = cos t; turned, w = i g (1 + i r) with g = -sin t; |r| <= 1.
+struct Tw {
+  double2 gr;
+  bool turned;
+};
+// (a, b) <- (a + w b, a - w b); QUARTER: with -i w for w (conjugated for the inverse)
+template <int SIGN, bool QUARTER = false>
+__device__ __forceinline__ void bf(double2& a, double2& b, const Tw& w) {
+  const double g = w.gr.x, r = SIGN < 0 ? w.gr.y : -w.gr.y;
+  // i b (forward) or -i b, and back by a quarter: on the integer pipe (a negation can become an
+  // FP64 addition)
+  const bool take = w.turned != QUARTER;
+  const unsigned flip = take ? 0x80000000u : 0u;
+  constexpr bool up = (SIGN < 0) != QUARTER;  // (-b.y, b.x), else (b.y, -b.x)
+  const double2 c = make_double2(
+      __hiloint2double((take ? __double2hiint(b.y) : __double2hiint(b.x)) ^ (up ? flip : 0u),
+                       take ? __double2loint(b.y) : __double2loint(b.x)),
+      __hiloint2double((take ? __double2hiint(b.x) : __double2hiint(b.y)) ^ (up ? 0u : flip),
+                       take ? __double2loint(b.x) : __double2loint(b.y)));
+  const double2 u = make_double2(fma(-r, c.y, c.x), fma(r, c.x, c.y));
+  b = make_double2(fma(-g, u.x, a.x), fma(-g, u.y, a.y));
+  a = make_double2(fma(g, u.x, a.x), fma(g, u.y, a.y));
 }
 // (a, b) <- (a + b, a - b)
 __device__ __forceinline__ void bf1(double2& a, double2& b) {
@@ -66,25 +85,23 @@ __device__ __forceinline__ void bfi(double2& a, double2& b) {
   b = make_double2(a.x - t.x, a.y - t.y);
   a = make_double2(a.x + t.x, a.y + t.y);
 }
-// -i w: the twiddle a quarter turn on (bf conjugates it for the inverse)
-__device__ __forceinline__ double2 quarter(double2 w) { return make_double2(w.y, -w.x); }
 
 // DFT of size R of v[r] w^r, w = w1 the stage twiddle (TW 0: w = 1) and w2 = w^2, by decimation
 // in the bits of r, most significant first; results in natural order.
 template <int R, int SIGN, bool TW> struct Dft;
 template <int SIGN, bool TW> struct Dft<2, SIGN, TW> {
-  __device__ __forceinline__ static void run(double2* v, double2 w1, double2) {
+  __device__ __forceinline__ static void run(double2* v, const Tw& w1, const Tw&) {
     if (TW) bf<SIGN>(v[0], v[1], w1);
     else bf1(v[0], v[1]);
   }
 };
 template <int SIGN, bool TW> struct Dft<4, SIGN, TW> {
-  __device__ __forceinline__ static void run(double2* v, double2 w1, double2 w2) {
+  __device__ __forceinline__ static void run(double2* v, const Tw& w1, const Tw& w2) {
     if (TW) {
       bf<SIGN>(v[0], v[2], w2);
       bf<SIGN>(v[1], v[3], w2);
       bf<SIGN>(v[0], v[1], w1);
-      bf<SIGN>(v[2], v[3], quarter(w1));
+      bf<SIGN, true>(v[2], v[3], w1);
     } else {
       bf1(v[0], v[2]);
       bf1(v[1], v[3]);
@@ -136,11 +153,14 @@ __device__ __forceinline__ void stage(double2* buf, int L, int Ns, int t, bool a
     if constexpr (R == 3) {
       dft3<SIGN>(x);
     } else if (Ns == 1) {
-      const double2 one = make_double2(1.0, 0.0);
+      const Tw one{make_double2(1.0, 0.0), false};
       Dft<R, SIGN, false>::run(x, one, one);
     } else {
+      // w's angle is 2 pi k / (R Ns): turned between an eighth and three eighths of a circle
       const double2* s = st + (Ns - 1) + k;
-      Dft<R, SIGN, true>::run(x, s[0], R > 2 ? s[Ns] : s[0]);
+      const bool mid = 4 * k > Ns && 4 * k < 3 * Ns;
+      const Tw w1{s[0], R == 2 ? mid : 2 * k > Ns}, w2{R == 2 ? s[0] : s[Ns], mid};
+      Dft<R, SIGN, true>::run(x, w1, w2);
     }
     const int d = qd * Ns * R + k;
 #pragma unroll
@@ -149,9 +169,8 @@ __device__ __forceinline__ void stage(double2* buf, int L, int Ns, int t, bool a
   __syncthreads();
 }
 
-// Full unnormalised transform in place (plain layout in and out) by L / 4 threads; the radix
-// sequence is that of the stage tables of 12 and 4 elements: [3,] then 4 while it divides,
-// then 2.
+// Full unnormalised transform in place (plain layout in and out) by L / 4 threads; the radices
+// are [3,] then 4 while it divides, then 2.
 template <int SIGN>
 __device__ __forceinline__ void fft64(double2* buf, int L, int t, bool active,
                                       const double2* __restrict__ tw) {
@@ -219,10 +238,10 @@ __global__ void __launch_bounds__(kMaxThreads)
       const double2 zk = buf[k], zm = buf[L - k], w = twM[k];
       const double2 ev = make_double2(zk.x + zm.x, zk.y - zm.y),
                     ov = make_double2(zk.y + zm.y, zm.x - zk.x);
-      const double2 s = make_double2(fma(w.x, ov.x, fma(-w.y, ov.y, ev.x)),
-                                     fma(w.x, ov.y, fma(w.y, ov.x, ev.y)));
-      out[k] = s;
-      if (2 * k != L) out[L - k] = make_double2(fma(2.0, ev.x, -s.x), -fma(2.0, ev.y, -s.y));
+      const double2 s = make_double2(fma(-w.x, ov.x, fma(w.y, ov.y, ev.x)),
+                                     fma(w.x, ov.y, fma(w.y, ov.x, -ev.y)));
+      out[k] = make_double2(fma(2.0, ev.x, -s.x), fma(2.0, ev.y, s.y));
+      if (2 * k != L) out[L - k] = s;
     }
   }
 }
