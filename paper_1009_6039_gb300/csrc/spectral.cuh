@@ -163,7 +163,8 @@ __device__ __forceinline__ int spad(int i, bool on) { return on ? i + (i >> 4) :
 // the length allows is filled): the stage with span Ns and radix R holds exp(-2 pi i k r /
 // (Ns R)) for r = 1..R-1, k = 0..Ns-1 at (Ns - 1) + (r - 1) Ns + k (the stages before it hold
 // sum Ns'(R' - 1) = Ns - 1 entries).  The threads of a warp take consecutive k, so a stage's
-// twiddle loads are contiguous instead of the strided k r L / (Ns R) of the base table.
+// twiddle loads are contiguous instead of the strided k r L / (Ns R) of the base table.  (FP64: the place of
+// E = 4 holds the butterfly table of spectral_f64.cu.)
 template <int E> __host__ __device__ constexpr int stage_table_slot() {
   return E == 4 ? 1 : (E == 8 ? 2 : 3);
 }

@@ -47,7 +47,8 @@ __device__ __forceinline__ const double2* stage_table(const double2* tw, int L) 
 // ---------------------------------------------------------------------------------------
 // Butterflies.  SIGN -1 forward, +1 inverse (the twiddles are conjugated).
 // ---------------------------------------------------------------------------------------
-// A twiddle w = exp(-i t) as its larger part and the ratio of the two, so that a +- w b take three
+// A twiddle w = exp(-i t) as its larger part and the ratio of the two (the scaled butterflies of Linzer and
+// Feig's FMA transforms), so that a +- w b take three
 // FMAs a part and each is rounded once at its own size: not turned (|cos t| >= |sin t|), w = g (1 +
 // i r) with g = cos t; turned, w = i g (1 + i r) with g = -sin t; |r| <= 1.
 struct Tw {
